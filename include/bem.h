@@ -71,9 +71,8 @@ typedef struct {
                           context times every variant on its own far-field block and the
                           context keeps the fastest; k = 1..BEM_FAR_TILE_VARIANTS: variant k,
                           rows x columns per CTA 32x256, 16x256, 64x256, 8x128, 16x128, 32x128,
-                          and (DF64: point loops rolled, at least m CTAs per SM) 8x128 m8,
-                          16x128 m8, 32x128 m8, 8x128 m9, 8x64 m16, 8x64 m18, and with the
-                          point loops unrolled 8x128 m6, 32x128 m6 */
+                          and (DF64: registers capped for at least m CTAs per SM) 8x128 m5,
+                          16x128 m5, 32x128 m5, 4x128 m5, 8x64 m10, 4x64 m10, 2x64 m10, 1x64 m10 */
 } bem_assembly_opts;
 #define BEM_FAR_TILE_VARIANTS 14
 

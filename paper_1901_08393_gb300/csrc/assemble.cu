@@ -3,24 +3,23 @@
 //
 //  * Far field (no common vertex): 7 x 7 product of Radon's degree-5 rule,
 //      V_ij = |Ti||Tj|/(4pi) sum_a w_a sum_b w_b / |x_a - y_b|.
-//    One thread per column j holds its 7 points (FP64, FP32: in registers; DF64: on
-//    the current pair's grid in shared memory); the CTA stages R row triangles in
+//    One thread per column j holds its 7 points (FP64, FP32: in registers; DF64: its
+//    triangle's table in shared memory); the CTA stages R row triangles in
 //    shared memory and walks them (broadcast reads; R x C tile variants, chosen per
 //    size class by timing them).  Only
 //    entries with i <= j are computed; the strict lower triangle is mirrored, so
 //    V is exactly symmetric and an incremental re-assembly reproduces the full
 //    one bit for bit.  Three arithmetic variants:
-//      DF64 -- FP64-accurate double-float on the FP32 pipe: x_a - y_b is formed as
-//              (c_i - c_j) + (o_a - o_b) with the centroid difference taken exactly
-//              from three-float centroids and the offsets o from the centroid as
-//              hi/lo pairs.  Pairs whose centroids are at least 1.12 (R_i + R_j)
-//              apart (R: the largest distance of a triangle's points from its
-//              centroid; almost all far pairs) split every term on one power-of-two
-//              grid chosen for the pair, so that the hi part of x_a - y_b is a single
-//              exact subtraction; closer pairs take it by two-sums.  |r|^2 by
-//              two-product/two-sum; 1/|r| by the MUFU reciprocal square root and one
-//              Newton step in double-float (error ~1.5 e^2 ~ 1e-14); sums by
-//              two-sum.  Entries within ~1e-12 of FP64.  V stored as hi/lo pairs.
+//      DF64 -- FP64-accurate double-float on the FP32 pipe.  The centroid difference
+//              d = c_i - c_j is taken exactly from three-float centroids.  Pairs at
+//              least 1.5 (R_i + R_j) apart (R: the largest distance of a triangle's
+//              points from its centroid; almost all far pairs) expand |x_a - y_b|^2
+//              into dot products of d and the points' offsets, split on one
+//              power-of-two grid chosen for the pair so that hi parts add exactly;
+//              closer pairs form x_a - y_b by two-sums, gathered so that whole warps
+//              take them.  1/|r| by the MUFU reciprocal square root and one step in
+//              double-float.  Entries within 3e-13 of FP64 (r.m.s. 3e-14).  V stored
+//              as hi/lo pairs.
 //      F64  -- native FP64 (GB300 issues FP64 at 1/64 of the FP32 rate).
 //      F32  -- centroid difference from hi + lo float centroids, offsets in FP32, MUFU rsqrt;
 //              no FP64 operation per pair (GB300 issues FP64 at 1/64 of the FP32 rate).
@@ -138,12 +137,11 @@ template <> struct Elem<float2> {
 // more, smaller CTAs) and on the arithmetic, and is chosen by timing (autotune).
 struct FarTileS {
     int rows, cols;
-    int min_ctas;  // DF64: > 0 -- point loops rolled, this many CTAs per SM requested
-                   // (the other arithmetics use their unrolled register form)
+    int min_ctas;  // DF64: > 0 -- registers capped so that this many CTAs fit an SM
 };
 constexpr FarTileS kFarTiles[kFarTileVariants] = {
-    {32, 256, 0}, {16, 256, 0}, {64, 256, 0}, {8, 128, 0}, {16, 128, 0}, {32, 128, 0}, {8, 128, 8},
-    {16, 128, 8}, {32, 128, 8}, {8, 128, 9},  {8, 64, 16},  {8, 64, 18},  {8, 128, 6}, {32, 128, 6}};
+    {32, 256, 0}, {16, 256, 0}, {64, 256, 0}, {8, 128, 0}, {16, 128, 0}, {32, 128, 0}, {8, 128, 5},
+    {16, 128, 5}, {32, 128, 5}, {4, 128, 5},  {8, 64, 10}, {4, 64, 10},  {2, 64, 10}, {1, 64, 10}};
 
 // The far-field bodies take the tile origin (first row i0, first column cbase) as
 // arguments: the per-operator kernels derive it from the block index, the batched
@@ -281,6 +279,12 @@ __global__ void __launch_bounds__(C) k_far_f32(const float *__restrict__ q32,
 // of big is exact (Sterbenz).
 __device__ __forceinline__ float grid_snap(float v, float big) { return __fsub_rn(__fadd_rn(v, big), big); }
 
+// 1.5 * 2^(k + up) for a normal v in [2^k, 2^(k+1))
+__device__ __forceinline__ float grid_big(float v, unsigned up)
+{
+    return __uint_as_float(((__float_as_uint(v) & 0x7f800000u) + (up << 23)) | 0x400000u);
+}
+
 // s + e = a + b exactly for a, b >= 0 (Dekker's fast two-sum with the larger first).
 __device__ __forceinline__ void pos_two_sum(float a, float b, float &s, float &e)
 {
@@ -288,58 +292,55 @@ __device__ __forceinline__ void pos_two_sum(float a, float b, float &s, float &e
     e = __fsub_rn(fminf(a, b), __fsub_rn(s, fmaxf(a, b)));
 }
 
-// 1/|d| = y + yl for |d|^2 = Sh + Sl: the MUFU estimate y and one Newton step in
-// double-float, yl = y t / 2 with t = 1 - S y^2 and y^2 = y2 + y2e by a two-product.
-// The estimate's relative error is below 2^-22, so 1 - Sh y2 is below 2^-20 in size
-// and its single rounding in the FMA is below 2^-44; the other terms are of order
-// 2^-24 and enter by FMAs.
-template <bool FTZ = false>
-__device__ __forceinline__ void df_rsqrt_newton(float Sh, float Sl, float &y, float &yl)
-{
-    if (FTZ)  // Sh known to be a normal number: the bare MUFU estimate
-        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(Sh));
-    else
-        y = rsqrtf(Sh);
-    float y2, y2e;
-    two_prod(y, y, y2, y2e);
-    float t = __fmaf_rn(-Sh, y2, 1.0f);
-    t = __fmaf_rn(-Sh, y2e, t);
-    t = __fmaf_rn(-Sl, y2, t);
-    yl = __fmul_rn(__fmul_rn(0.5f, y), t);
-}
-
-// sh + sl += w (y + yl) with the two-sum of the running sum (pos: sh and w y are not
-// negative, the larger added first)
-template <bool POS = false>
+// sh + sl += w (y + yl) with the two-sum of the running sum
 __device__ __forceinline__ void df_acc_w(float2 w, float y, float yl, float &sh, float &sl)
 {
     float ph, pe, u, ue;
     two_prod(w.x, y, ph, pe);
     pe = __fmaf_rn(w.x, yl, pe);
     pe = __fmaf_rn(w.y, y, pe);
-    if (POS)
-        pos_two_sum(sh, ph, u, ue);
-    else
-        two_sum(sh, ph, u, ue);
+    two_sum(sh, ph, u, ue);
     sh = u;
     sl = __fadd_rn(sl, __fadd_rn(pe, ue));
 }
 
-// Entry sum sum_a w_a sum_b w_b / |x_a - y_b| of a pair whose bounding balls are close
-// (|c_i - c_j| < 1.12 (R_i + R_j)): x_a - y_b = (D + o_a) - o_b in double-float by
-// two-sums, D = c_i - c_j, o the offsets from the centroids (o_b from the table).
-__device__ __forceinline__ void far_df_exact(const float *qi, const float *Dh, const float *Dl,
-                                             const float2 *__restrict__ oj, float &h_out, float &l_out)
+// Centroid difference c_i - c_j from the three-float centroids, one coordinate.
+__device__ __forceinline__ void centroid_diff(float a0, float a1, float a2, float b0, float b1, float b2, float &dh,
+                                              float &dl)
 {
+    float s1, e1, s2, e2, h, l;
+    two_sum(a0, -b0, s1, e1);
+    two_sum(a1, -b1, s2, e2);
+    two_sum(s1, s2, h, l);
+    l = __fadd_rn(l, __fadd_rn(__fadd_rn(e1, e2), __fsub_rn(a2, b2)));
+    fast_two_sum(h, l, dh, dl);
+}
+
+// Entry (i, j) of a pair whose triangles are close (|c_i - c_j| < 1.5 (R_i + R_j)):
+// sum_a w_a sum_b w_b / |x_a - y_b| with x_a - y_b = (D + o_a) - o_b in double-float by
+// two-sums, D = c_i - c_j, o the offsets from the centroids, and 1/|d| = y + y t / 2 from
+// the MUFU estimate y by one Newton step, t = 1 - S y^2 with y^2 by a two-product (the
+// estimate's relative error is below 2^-22, so 1 - Sh y2 is below 2^-20 in size and its
+// single rounding in the FMA is below 2^-44).  74 FP32 operations per point pair; called
+// for the few close pairs of a tile together (far_df_body), so kept out of line.
+__device__ __noinline__ float2 far_df_close(const float *__restrict__ qi, const float *__restrict__ qj)
+{
+    float Dh[3], Dl[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        centroid_diff(qi[42 + 3 * c], qi[43 + 3 * c], qi[44 + 3 * c], qj[42 + 3 * c], qj[43 + 3 * c], qj[44 + 3 * c],
+                      Dh[c], Dl[c]);
+    const float2 *oi = reinterpret_cast<const float2 *>(qi), *oj = reinterpret_cast<const float2 *>(qj);
     float acc_h = 0.0f, acc_l = 0.0f;
 #pragma unroll 1
     for (int a = 0; a < kQ; ++a) {
         float eh[3], el[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
+            const float2 o = oi[3 * a + c];
             float s, e;
-            two_sum(Dh[c], qi[2 * (3 * a + c)], s, e);
-            e = __fadd_rn(e, __fadd_rn(Dl[c], qi[2 * (3 * a + c) + 1]));
+            two_sum(Dh[c], o.x, s, e);
+            e = __fadd_rn(e, __fadd_rn(Dl[c], o.y));
             fast_two_sum(s, e, eh[c], el[c]);
         }
         float sh = 0.0f, sl = 0.0f;
@@ -366,166 +367,336 @@ __device__ __forceinline__ void far_df_exact(const float *qi, const float *Dh, c
                     Sl = __fadd_rn(Sl, __fadd_rn(pe, te));
                 }
             }
-            float y, yl;
-            df_rsqrt_newton(Sh, Sl, y, yl);
-            df_acc_w(c_w7df[b], y, yl, sh, sl);
+            const float y = rsqrtf(Sh);
+            float y2, y2e;
+            two_prod(y, y, y2, y2e);
+            float t = __fmaf_rn(-Sh, y2, 1.0f);
+            t = __fmaf_rn(-Sh, y2e, t);
+            t = __fmaf_rn(-Sl, y2, t);
+            df_acc_w(c_w7df[b], y, __fmul_rn(__fmul_rn(0.5f, y), t), sh, sl);
         }
         df_acc_w(c_w7df[a], sh, sl, acc_h, acc_l);
     }
-    fast_two_sum(acc_h, acc_l, h_out, l_out);
+    float h, l;
+    fast_two_sum(acc_h, acc_l, h, l);
+    return df_mul(df_mul(make_float2(qi[51], qi[52]), df_mul(make_float2(qj[51], qj[52]), c_inv4pi_df)),
+                  make_float2(h, l));
 }
 
-// The same sum for a pair with |D| >= 1.12 (R_i + R_j) (R: the largest distance of a
-// triangle's points from its centroid): D, o_a and o_b are split on the pair's grid
-// q = 2^(e-23), 2^(e-1) > max(|D|_inf, r_i, r_j) (r: the largest |hi| of the offset
-// coordinates) with e odd -- hi parts multiples of q (exact), lo parts the rest -- so
-// that the hi part h of x_a - y_b is one exact subtraction and its lo part l one
-// rounded one; |d|^2 = h^2 + 2 h l + l^2 with h^2 by a two-product.  Every |x_a - y_b|
-// is at least 0.107 |D| and 2^e <= 8 |D|, so the lo parts' roundings (a few units of
-// 2^-24 q each) stay below 1e-11 of the entry.  sg: o_b on the grid, (hi, 2 lo),
-// stride C.
-template <int C, bool UNROLL>
-__device__ __forceinline__ void far_df_grid(const float *qi, const float *Dh, const float *Dl, float big,
-                                            const float2 *sg, float &h_out, float &l_out)
+// The expanded form, for every other pair.  Radon's points of a triangle are its
+// centroid and two orbits o_1k = t v_k, o_2k = s o_1k (v_k: vertex k from the centroid,
+// t = (1 + sqrt 15) / 7, s = (1 - sqrt 15) / (1 + sqrt 15)), and o_12 = -(o_10 + o_11), so
+//   |x_a - y_b|^2 = |d|^2 + A_a + B_b - C_ab,  d = c_i - c_j,
+//   A_1k = 2 d.o_1k + |o_1k|^2,   A_2k = s 2 d.o_1k + |o_2k|^2   (B alike, with -2 d.o),
+//   C = G, s G or s^2 G with G_kl = 2 o_1k.o_1l:
+// 9 dot products of three terms for all 49 squared distances, instead of three
+// differences and three squares for each.  Every product is split on one power-of-two
+// grid of the pair, q = 2^(e-23) with 2^(e-1) > 1.34 |d|^2: its hi part is the multiple of
+// q next to it (an FMA onto 1.5 * 2^e and a subtraction), its lo part the rest (an FMA),
+// so that hi parts add exactly in plain additions: no term exceeds 4/3 |d|^2 and no sum
+// 3 |d|^2 < 2^24 q while |d| >= 1.5 (R_i + R_j).  The lo parts add up with an error of a
+// few units of 2^-24 q; every |x_a - y_b|^2 is at least |d|^2 / 9.  The MUFU estimate of
+// 1/|x_a - y_b| is itself put on a grid (a multiple of 2^-17 .. 2^-18 of 1/|d|), so that
+// estimates of equal weight add exactly; the step from there, y t (1/2 + 3/8 t) with t =
+// 1 - S y^2 below 2^-16, goes to the lo sum.  Error of an entry (CPU emulation on cubes,
+// graded cubes with needles, Fichera, polycubes): 2.2e-13 at most, 3e-14 r.m.s., no bias.
+//
+// 16 FP32 operations per point pair and about 520 per entry, against 50 and 336 of the
+// form that took each of the 49 differences on a grid (three subtractions and squares
+// each).  Bound by FP32 issue (73% of the 128 lanes per SM and cycle).  Measured on rotated
+// polycubes, best tile of each: N = 604 116 -> 35 us, N = 2,416 418 -> 166 us, N = 9,664
+// 4.60 -> 2.03 ms, N = 21,744 22.3 -> 9.88 ms (10.6 -> 23.9 Gpairs/s).
+constexpr double kSqrt15 = 3.87298334620741688518;
+constexpr double kOrbS = (1.0 - kSqrt15) / (1.0 + kSqrt15);
+constexpr float kOrbSh = (float)kOrbS, kOrbSl = (float)(kOrbS - (double)kOrbSh);
+constexpr float kOrbS2h = (float)(kOrbS * kOrbS), kOrbS2l = (float)(kOrbS * kOrbS - (double)kOrbS2h);
+constexpr double kW0 = 9.0 / 40.0, kW1 = (155.0 - kSqrt15) / 1200.0, kW2 = (155.0 + kSqrt15) / 1200.0;
+constexpr float kFarSpread2 = 2.2505f;  // 1.5^2, rounded up past the FP32 errors of the test
+
+// h + l = (ah + al) (bh + bl), h on the grid
+__device__ __forceinline__ void grid_prod(float ah, float al, float bh, float bl, float big, float &h, float &l)
 {
-    float Dg[3], Dl2[3];
+    h = __fsub_rn(__fmaf_rn(ah, bh, big), big);
+    l = __fmaf_rn(ah, bl, __fmaf_rn(al, bh, __fmaf_rn(ah, bh, -h)));
+}
+
+// h + l = a.b for double-float vectors (h, l) x 3
+__device__ __forceinline__ void grid_dot(const float *ah, const float *al, const float *bh, const float *bl, float big,
+                                         float &h, float &l)
+{
+    float p[3], r[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) grid_prod(ah[c], al[c], bh[c], bl[c], big, p[c], r[c]);
+    h = __fadd_rn(__fadd_rn(p[0], p[1]), p[2]);
+    l = __fadd_rn(__fadd_rn(r[0], r[1]), r[2]);
+}
+
+// The offset terms of one triangle's orbits: h1 + l1 = p + |o_1|^2, h2 + l2 = s p +
+// |o_2|^2 for the projection p of vertex k; n: (|o_1|^2 hi, lo, |o_2|^2 hi, lo).
+__device__ __forceinline__ void orbit_terms(float ph, float pl, float4 n, float big, float &h1, float &l1, float &h2,
+                                            float &l2)
+{
+    const float g1 = grid_snap(n.x, big), g2 = grid_snap(n.z, big);
+    h1 = __fadd_rn(ph, g1);
+    l1 = __fadd_rn(pl, __fadd_rn(__fsub_rn(n.x, g1), n.y));
+    grid_prod(kOrbSh, kOrbSl, ph, pl, big, h2, l2);
+    h2 = __fadd_rn(h2, g2);
+    l2 = __fadd_rn(l2, __fadd_rn(__fsub_rn(n.z, g2), n.w));
+}
+
+// s + l += 1 / sqrt(H + L)
+__device__ __forceinline__ void inv_root_acc(float H, float L, float by, float &s, float &l)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(H));  // H: a normal number
+    y = grid_snap(y, by);
+    float y2, y2e;
+    two_prod(y, y, y2, y2e);
+    float t = __fmaf_rn(-H, y2, 1.0f);
+    t = __fmaf_rn(-H, y2e, t);
+    t = __fmaf_rn(-L, y2, t);
+    s = __fadd_rn(s, y);
+    l = __fmaf_rn(y, __fmul_rn(t, __fmaf_rn(t, 0.375f, 0.5f)), l);
+}
+
+// acc += w (s + l), all positive
+__device__ __forceinline__ void class_acc(double w, float s, float l, float &h, float &lo)
+{
+    const float wh = (float)w, wl = (float)(w - (double)wh);
+    float p, e, u, ue;
+    two_prod(wh, s, p, e);
+    e = __fmaf_rn(wl, s, __fmaf_rn(wh, l, e));
+    pos_two_sum(h, p, u, ue);
+    h = u;
+    lo = __fadd_rn(lo, __fadd_rn(e, ue));
+}
+
+// ri: the row triangle's nine float4 of the table (kQdfExp), cj: the column triangle's,
+// stride C; dh, dl: c_i - c_j.
+template <int C>
+__device__ __forceinline__ void far_df_expanded(const float4 *ri, const float4 *cj, const float *dh, const float *dl,
+                                                float big, float &h_out, float &l_out)
+{
+    float d2h[3], d2l[3];  // 2 d
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        Dg[c] = grid_snap(Dh[c], big);
-        Dl2[c] = __fmul_rn(2.0f, __fadd_rn(__fsub_rn(Dh[c], Dg[c]), Dl[c]));
+        d2h[c] = __fadd_rn(dh[c], dh[c]);
+        d2l[c] = __fadd_rn(dl[c], dl[c]);
     }
-    float acc_h = 0.0f, acc_l = 0.0f;
-#pragma unroll(UNROLL ? kQ : 1)
-    for (int a = 0; a < kQ; ++a) {
-        float eh[3], el2[3];  // x_a - c_j: hi on the grid, twice the lo part
+    float Dh, Dl;
+    {
+        float p[3], r[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const float oh = qi[2 * (3 * a + c)], og = grid_snap(oh, big);
-            eh[c] = __fadd_rn(Dg[c], og);
-            el2[c] = __fmaf_rn(2.0f, __fadd_rn(__fsub_rn(oh, og), qi[2 * (3 * a + c) + 1]), Dl2[c]);
+            p[c] = __fsub_rn(__fmaf_rn(dh[c], dh[c], big), big);
+            r[c] = __fmaf_rn(d2h[c], dl[c], __fmaf_rn(dh[c], dh[c], -p[c]));
         }
-        float sh = 0.0f, sl = 0.0f;
-        auto point_pair = [&](int b) {
-            float p[3], pe[3];
+        Dh = __fadd_rn(__fadd_rn(p[0], p[1]), p[2]);
+        Dl = __fadd_rn(__fadd_rn(r[0], r[1]), r[2]);
+    }
+    float y0;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(Dh));
+    const float by = grid_big(y0, 6);
+    // class sums by weight: w0^2, w0 w1, w0 w2, w1^2, w1 w2, w2^2
+    float s[6], l[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s[k] = l[k] = 0.0f;
+    inv_root_acc(Dh, Dl, by, s[0], l[0]);
+    // column side: B_1l, B_2l, and the orbit offsets of vertices 0 and 1
+    float wh[2][3], wl[2][3], B1h[3], B1l[3], B2h[3], B2l[3];
+    {
+        const float4 a = cj[0], b = cj[C], c = cj[2 * C];
+        wh[0][0] = a.x; wl[0][0] = a.y; wh[0][1] = a.z; wl[0][1] = a.w; wh[0][2] = b.x; wl[0][2] = b.y;
+        wh[1][0] = b.z; wl[1][0] = b.w; wh[1][1] = c.x; wl[1][1] = c.y; wh[1][2] = c.z; wl[1][2] = c.w;
+        float qh[3], ql[3];
+        grid_dot(d2h, d2l, wh[0], wl[0], big, qh[0], ql[0]);
+        grid_dot(d2h, d2l, wh[1], wl[1], big, qh[1], ql[1]);
+        qh[2] = -__fadd_rn(qh[0], qh[1]);
+        ql[2] = -__fadd_rn(ql[0], ql[1]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            orbit_terms(-qh[k], -ql[k], cj[(3 + k) * C], big, B1h[k], B1l[k], B2h[k], B2l[k]);
+            inv_root_acc(__fadd_rn(Dh, B1h[k]), __fadd_rn(Dl, B1l[k]), by, s[1], l[1]);
+            inv_root_acc(__fadd_rn(Dh, B2h[k]), __fadd_rn(Dl, B2l[k]), by, s[2], l[2]);
+        }
+    }
+    float psh = 0.0f, psl = 0.0f, Gsh[3] = {0.0f, 0.0f, 0.0f}, Gsl[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        float ph, pl, Gh[3], Gl[3];
+        if (k < 2) {
+            float vh[3], vl[3];
+            if (k == 0) {
+                const float4 a = ri[0], b = ri[1];
+                vh[0] = a.x; vl[0] = a.y; vh[1] = a.z; vl[1] = a.w; vh[2] = b.x; vl[2] = b.y;
+            } else {
+                const float4 b = ri[1], c = ri[2];
+                vh[0] = b.z; vl[0] = b.w; vh[1] = c.x; vl[1] = c.y; vh[2] = c.z; vl[2] = c.w;
+            }
+            grid_dot(d2h, d2l, vh, vl, big, ph, pl);
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float2 o = sg[(3 * b + c) * C];
-                const float dh = __fsub_rn(eh[c], o.x);  // exact
-                const float dl2 = __fsub_rn(el2[c], o.y);
-                p[c] = __fmul_rn(dh, dh);
-                pe[c] = __fmaf_rn(dh, dh, -p[c]);
-                pe[c] = __fmaf_rn(dl2, __fmaf_rn(0.25f, dl2, dh), pe[c]);  // 2 h l + l^2
+                vh[c] = __fadd_rn(vh[c], vh[c]);
+                vl[c] = __fadd_rn(vl[c], vl[c]);
             }
-            float s1, e1, s2, e2, y, yl;
-            pos_two_sum(p[0], p[1], s1, e1);
-            pos_two_sum(s1, p[2], s2, e2);
-            df_rsqrt_newton<true>(s2, __fadd_rn(__fadd_rn(pe[0], pe[1]), __fadd_rn(pe[2], __fadd_rn(e1, e2))), y,
-                                  yl);
-            df_acc_w<true>(c_w7df[b], y, yl, sh, sl);
-        };
-        if (UNROLL) {
+            grid_dot(vh, vl, wh[0], wl[0], big, Gh[0], Gl[0]);
+            grid_dot(vh, vl, wh[1], wl[1], big, Gh[1], Gl[1]);
+            Gh[2] = -__fadd_rn(Gh[0], Gh[1]);
+            Gl[2] = -__fadd_rn(Gl[0], Gl[1]);
+            psh = __fadd_rn(psh, ph);
+            psl = __fadd_rn(psl, pl);
 #pragma unroll
-            for (int b = 0; b < kQ; ++b) point_pair(b);
-        } else {  // two point pairs per trip: half the loop control
-            point_pair(0);
-#pragma unroll 2
-            for (int b = 1; b < kQ; ++b) point_pair(b);
+            for (int j = 0; j < 3; ++j) {
+                Gsh[j] = __fadd_rn(Gsh[j], Gh[j]);
+                Gsl[j] = __fadd_rn(Gsl[j], Gl[j]);
+            }
+        } else {  // vertex 2's offsets are minus the sum of the others'
+            ph = -psh;
+            pl = -psl;
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                Gh[j] = -Gsh[j];
+                Gl[j] = -Gsl[j];
+            }
         }
-        df_acc_w<true>(c_w7df[a], sh, sl, acc_h, acc_l);
+        float A1h, A1l, A2h, A2l;
+        orbit_terms(ph, pl, ri[3 + k], big, A1h, A1l, A2h, A2l);
+        A1h = __fadd_rn(A1h, Dh);
+        A1l = __fadd_rn(A1l, Dl);
+        A2h = __fadd_rn(A2h, Dh);
+        A2l = __fadd_rn(A2l, Dl);
+        inv_root_acc(A1h, A1l, by, s[1], l[1]);
+        inv_root_acc(A2h, A2l, by, s[2], l[2]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float C1h, C1l, C2h, C2l;  // s G, s^2 G
+            grid_prod(kOrbSh, kOrbSl, Gh[j], Gl[j], big, C1h, C1l);
+            grid_prod(kOrbS2h, kOrbS2l, Gh[j], Gl[j], big, C2h, C2l);
+            inv_root_acc(__fsub_rn(__fadd_rn(A1h, B1h[j]), Gh[j]), __fsub_rn(__fadd_rn(A1l, B1l[j]), Gl[j]), by, s[3],
+                         l[3]);
+            inv_root_acc(__fsub_rn(__fadd_rn(A1h, B2h[j]), C1h), __fsub_rn(__fadd_rn(A1l, B2l[j]), C1l), by, s[4],
+                         l[4]);
+            inv_root_acc(__fsub_rn(__fadd_rn(A2h, B1h[j]), C1h), __fsub_rn(__fadd_rn(A2l, B1l[j]), C1l), by, s[4],
+                         l[4]);
+            inv_root_acc(__fsub_rn(__fadd_rn(A2h, B2h[j]), C2h), __fsub_rn(__fadd_rn(A2l, B2l[j]), C2l), by, s[5],
+                         l[5]);
+        }
     }
+    float acc_h = 0.0f, acc_l = 0.0f;
+    class_acc(kW0 * kW0, s[0], l[0], acc_h, acc_l);
+    class_acc(kW0 * kW1, s[1], l[1], acc_h, acc_l);
+    class_acc(kW0 * kW2, s[2], l[2], acc_h, acc_l);
+    class_acc(kW1 * kW1, s[3], l[3], acc_h, acc_l);
+    class_acc(kW1 * kW2, s[4], l[4], acc_h, acc_l);
+    class_acc(kW2 * kW2, s[5], l[5], acc_h, acc_l);
     fast_two_sum(acc_h, acc_l, h_out, l_out);
 }
 
-// MB > 0: MB CTAs per SM requested (registers capped to fit), the point loops rolled
-// unless UB.  The column triangle's offsets on the current pair's grid are kept in
-// dynamic shared memory (3 kQ x C pairs, thread-major: conflict-free), re-split only
-// when the grid changes from one row to the next.
+// The column triangles' table rows are kept in dynamic shared memory (9 x C float4,
+// one column of the array per thread: conflict-free), the row triangles' beside them
+// (broadcast reads).
 template <int C>
-constexpr size_t far_df_smem() { return sizeof(float2) * 3 * kQ * C; }
+constexpr size_t far_df_smem() { return sizeof(float4) * 9 * C; }
 
-template <int R, int C, int MB, bool UB = false>
+// Close pairs (below 1.5 (R_i + R_j): 0.1-0.7% of the pairs from N = 5,000 on, most of them
+// on meshes of a few hundred triangles) cost three times the others: each warp puts its
+// own aside (row, lane) and computes them 32 at a time, so that a warp with one such pair
+// does not run both forms for a whole row.  The last ones run with the lanes there are.
+template <int R, int C>
 __device__ __forceinline__ void far_df_body(const float *__restrict__ qdf, float2 *__restrict__ V, int64_t ld,
                                             int64_t r1, int64_t c1, int64_t i0, int64_t cbase)
 {
-    constexpr bool UNROLL = MB == 0 || UB;
-    __shared__ float sq[R][55];
-    extern __shared__ float2 far_dsm[];
+    __shared__ float4 sq[R][9];
+    __shared__ unsigned short close_s[C / 32][64];
+    extern __shared__ float4 far_dsm[];
     if (i0 > cbase + C - 1 || i0 >= r1) return;
-    for (int k = threadIdx.x; k < R * 55; k += C) {
-        const int r = k / 55, c = k % 55;
-        const int64_t i = i0 + r;
-        sq[r][c] = (i < r1) ? qdf[i * kQdfStride + c] : 0.0f;
+    const float4 *q4 = reinterpret_cast<const float4 *>(qdf + kQdfExp);
+    constexpr int kS4 = kQdfStride / 4;
+    for (int k = threadIdx.x; k < R * 9; k += C) {
+        const int r = k / 9, c = k % 9;
+        const int64_t i = i0 + r < r1 ? i0 + r : r1 - 1;
+        sq[r][c] = q4[i * kS4 + c];
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t jw = cbase + 32 * warp, j = jw + lane;
+    float4 *cj = far_dsm + threadIdx.x;
+    {
+        const float4 *src = q4 + (j < c1 ? j : c1 - 1) * kS4;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) cj[k * C] = src[k];
     }
     __syncthreads();
-    const int64_t j = cbase + threadIdx.x;
-    if (j >= c1) return;
-    const float *qj = qdf + j * kQdfStride;
-    const float2 *oj = reinterpret_cast<const float2 *>(qj);
-    float2 *sg = far_dsm + threadIdx.x;
-    float cj[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) cj[k] = qj[42 + k];
-    const float rj = qj[53], Rj = qj[54];
-    const float2 Aj = df_mul(make_float2(qj[51], qj[52]), c_inv4pi_df);
-    unsigned eg = 0u;  // exponent field of the grid bound sg holds (0: none)
-    const int rows = (int)((r1 - i0) < R ? (r1 - i0) : R);
+    if (jw >= c1) return;
+    unsigned short *list = close_s[warp];
+    int n_close = 0;
+    auto flush = [&](int n) {  // the first n pairs put aside (n <= 32)
+        __syncwarp();
+        if (lane < n) {
+            const int e = list[lane];
+            const int64_t i = i0 + (e >> 5), jc = jw + (e & 31);
+            V[i * ld + jc] = far_df_close(qdf + i * kQdfStride, qdf + jc * kQdfStride);
+        }
+        __syncwarp();
+    };
+    const float2 Aj = df_mul(make_float2(cj[7 * C].w, cj[8 * C].w), c_inv4pi_df);
+    int rows = (int)((r1 - i0) < R ? (r1 - i0) : R);
+    if (jw + 32 - i0 < rows) rows = (int)(jw + 32 - i0);  // rows past the warp's last column: below the diagonal
     for (int r = 0; r < rows; ++r) {
         const int64_t i = i0 + r;
-        if (i > j) break;
-        const float *qi = sq[r];
-        // centroid difference c_i - c_j from the three-float centroids
-        float Dh[3], Dl[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            float s1, e1, s2, e2, h, l;
-            two_sum(qi[42 + 3 * c], -cj[3 * c], s1, e1);
-            two_sum(qi[43 + 3 * c], -cj[3 * c + 1], s2, e2);
-            const float s3 = __fsub_rn(qi[44 + 3 * c], cj[3 * c + 2]);
-            two_sum(s1, s2, h, l);
-            l = __fadd_rn(l, __fadd_rn(__fadd_rn(e1, e2), s3));
-            fast_two_sum(h, l, Dh[c], Dl[c]);
+        const bool valid = j < c1 && i <= j;
+        float dh[3], dl[3], Rs, Ah, Al;
+        {
+            const float4 *ri = sq[r];
+            const float4 a0 = ri[6], a1 = ri[7], a2 = ri[8], b0 = cj[6 * C], b1 = cj[7 * C], b2 = cj[8 * C];
+            centroid_diff(a0.x, a1.x, a2.x, b0.x, b1.x, b2.x, dh[0], dl[0]);
+            centroid_diff(a0.y, a1.y, a2.y, b0.y, b1.y, b2.y, dh[1], dl[1]);
+            centroid_diff(a0.z, a1.z, a2.z, b0.z, b1.z, b2.z, dh[2], dl[2]);
+            Rs = a0.w + b0.w;
+            Ah = a1.w;
+            Al = a2.w;
         }
-        const float ri = qi[53], Rs = qi[54] + Rj;
-        const float bound = fmaxf(fmaxf(fabsf(Dh[0]), fabsf(Dh[1])), fmaxf(fmaxf(fabsf(Dh[2]), ri), rj));
-        // bound in [2^(eb-127), 2^(eb-126)); odd eb, so that the grid changes less often
-        // from one row to the next
-        const unsigned eb = (__float_as_uint(bound) >> 23) | 1u;
-        const float D2 = Dh[0] * Dh[0] + Dh[1] * Dh[1] + Dh[2] * Dh[2];
-        float h, l;
-        // the grid path where its bounds hold (and no product of it can leave the
-        // normal FP32 range); the two-sum path otherwise
-        if (D2 >= 1.26f * (Rs * Rs) && eb >= 93u && eb <= 185u) {
-            const float big = __uint_as_float(((eb + 2u) << 23) | 0x400000u);  // 1.5 * 2^(eb-125)
-            if (eb != eg) {
-#pragma unroll 1
-                for (int k = 0; k < 3 * kQ; ++k) {
-                    const float2 o = oj[k];
-                    const float g = grid_snap(o.x, big);
-                    sg[k * C] = make_float2(g, __fmul_rn(2.0f, __fadd_rn(__fsub_rn(o.x, g), o.y)));
-                }
-                eg = eb;
+        const float D2 = dh[0] * dh[0] + dh[1] * dh[1] + dh[2] * dh[2];
+        const float m = 1.34f * D2;
+        // the expanded form where its bounds hold (and no product of it can leave the
+        // normal FP32 range); not for NaN
+        const bool wide = D2 >= kFarSpread2 * (Rs * Rs) && m >= 0x1p-68f && m <= 0x1p100f;
+        if (valid && wide) {
+            float h, l;
+            far_df_expanded<C>(sq[r], cj, dh, dl, grid_big(m, 2), h, l);
+            V[i * ld + j] = df_mul(df_mul(make_float2(Ah, Al), Aj), make_float2(h, l));
+        }
+        const bool put = valid && !wide && i != j;  // (i, i) is the near field's
+        const unsigned mask = __ballot_sync(0xffffffffu, put);
+        if (mask) {
+            if (put) list[n_close + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(r * 32 + lane);
+            n_close += __popc(mask);
+            if (n_close >= 32) {
+                flush(32);
+                n_close -= 32;
+                unsigned short rest = 0;
+                if (lane < n_close) rest = list[32 + lane];
+                __syncwarp();
+                if (lane < n_close) list[lane] = rest;
+                __syncwarp();
             }
-            far_df_grid<C, UNROLL>(qi, Dh, Dl, big, sg, h, l);
-        } else {
-            far_df_exact(qi, Dh, Dl, oj, h, l);
         }
-        V[i * ld + j] = df_mul(df_mul(make_float2(qi[51], qi[52]), Aj), make_float2(h, l));
     }
+    if (n_close) flush(n_close);
 }
 
+// MB > 0: MB CTAs per SM requested (registers capped to fit)
 template <int R, int C>
 __global__ void __launch_bounds__(C) k_far_df(const float *__restrict__ qdf, float2 *__restrict__ V, int64_t ld,
                                               int64_t r0, int64_t r1, int64_t c0, int64_t c1)
 {
-    far_df_body<R, C, 0>(qdf, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
+    far_df_body<R, C>(qdf, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
 }
 
-// UB: the inner point loop unrolled (more registers: fewer CTAs per SM requested)
-template <int R, int C, int MB, bool UB = false>
+template <int R, int C, int MB>
 __global__ void __launch_bounds__(C, MB) k_far_df_s(const float *__restrict__ qdf, float2 *__restrict__ V, int64_t ld,
                                                     int64_t r0, int64_t r1, int64_t c0, int64_t c1)
 {
-    far_df_body<R, C, MB, UB>(qdf, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
+    far_df_body<R, C>(qdf, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
 }
 
 // Mirror the strict lower triangle of rows [r0, r1): V[i][j] = V[j][i], j < i,
@@ -809,7 +980,7 @@ __global__ void k_diag(const T *V, int64_t ld, int64_t N, double *d)
 }
 
 // ------------------------------------------------------------------ drivers
-template <typename T, int R, int C, int MB = 0, bool UB = false>
+template <typename T, int R, int C, int MB = 0>
 static void far_kernel(bem_operator *op, dim3 grid, int64_t r0, int64_t r1, int64_t c0, int64_t c1)
 {
     bem_mesh *m = op->mesh;
@@ -819,8 +990,8 @@ static void far_kernel(bem_operator *op, dim3 grid, int64_t r0, int64_t r1, int6
     else if (op->precision == BEM_PREC_DF64)
     {
         if constexpr (MB > 0)
-            k_far_df_s<R, C, MB, UB><<<grid, C, far_df_smem<C>(), s>>>(m->qdf, (float2 *)op->V, op->ld, r0, r1,
-                                                                       c0, c1);
+            k_far_df_s<R, C, MB><<<grid, C, far_df_smem<C>(), s>>>(m->qdf, (float2 *)op->V, op->ld, r0, r1,
+                                                                   c0, c1);
         else
             k_far_df<R, C><<<grid, C, far_df_smem<C>(), s>>>(m->qdf, (float2 *)op->V, op->ld, r0, r1, c0, c1);
     }
@@ -849,11 +1020,10 @@ static bem_status launch_far(bem_operator *op, int v, int64_t r0, int64_t r1, in
         return BEM_OK;
     }
     dim3 grid((unsigned)gx, (unsigned)gy);
-    double units = 0.0;  // entries with i <= j in the block
-    for (int64_t i = r0; i < r1; ++i) {
-        const int64_t lo = i > c0 ? i : c0;
-        if (c1 > lo) units += (double)(c1 - lo);
-    }
+    // entries with i <= j in the block: whole rows above the columns' first, then a triangle
+    const int64_t full = (r1 < c0 ? r1 : c0) - r0, t0 = r0 > c0 ? r0 : c0, t1 = r1 < c1 ? r1 : c1;
+    const double units = (full > 0 ? (double)full * (double)(c1 - c0) : 0.0) +
+                         (t1 > t0 ? 0.5 * (double)(t1 - t0) * (double)((c1 - t0) + (c1 - t1 + 1)) : 0.0);
     const int prof = profile ? prof_start(ctx, BEM_KERNEL_FAR, units) : -1;
     switch (v) {
     case 0: far_kernel<T, 32, 256>(op, grid, r0, r1, c0, c1); break;
@@ -862,14 +1032,14 @@ static bem_status launch_far(bem_operator *op, int v, int64_t r0, int64_t r1, in
     case 3: far_kernel<T, 8, 128>(op, grid, r0, r1, c0, c1); break;
     case 4: far_kernel<T, 16, 128>(op, grid, r0, r1, c0, c1); break;
     case 5: far_kernel<T, 32, 128>(op, grid, r0, r1, c0, c1); break;
-    case 6: far_kernel<T, 8, 128, 8>(op, grid, r0, r1, c0, c1); break;
-    case 7: far_kernel<T, 16, 128, 8>(op, grid, r0, r1, c0, c1); break;
-    case 8: far_kernel<T, 32, 128, 8>(op, grid, r0, r1, c0, c1); break;
-    case 9: far_kernel<T, 8, 128, 9>(op, grid, r0, r1, c0, c1); break;
-    case 10: far_kernel<T, 8, 64, 16>(op, grid, r0, r1, c0, c1); break;
-    case 11: far_kernel<T, 8, 64, 18>(op, grid, r0, r1, c0, c1); break;
-    case 12: far_kernel<T, 8, 128, 6, true>(op, grid, r0, r1, c0, c1); break;
-    default: far_kernel<T, 32, 128, 6, true>(op, grid, r0, r1, c0, c1); break;
+    case 6: far_kernel<T, 8, 128, 5>(op, grid, r0, r1, c0, c1); break;
+    case 7: far_kernel<T, 16, 128, 5>(op, grid, r0, r1, c0, c1); break;
+    case 8: far_kernel<T, 32, 128, 5>(op, grid, r0, r1, c0, c1); break;
+    case 9: far_kernel<T, 4, 128, 5>(op, grid, r0, r1, c0, c1); break;
+    case 10: far_kernel<T, 8, 64, 10>(op, grid, r0, r1, c0, c1); break;
+    case 11: far_kernel<T, 4, 64, 10>(op, grid, r0, r1, c0, c1); break;
+    case 12: far_kernel<T, 2, 64, 10>(op, grid, r0, r1, c0, c1); break;
+    default: far_kernel<T, 1, 64, 10>(op, grid, r0, r1, c0, c1); break;
     }
     BEM_COUNT(ctx);
     if (profile) prof_stop(ctx, prof);
@@ -1050,7 +1220,7 @@ __device__ __forceinline__ int batch_find(const int64_t *__restrict__ prefix, in
     return lo;
 }
 
-template <typename T, int R, int C, int MB, bool UB>
+template <typename T, int R, int C, int MB>
 __global__ void __launch_bounds__(C, (MB > 0 ? MB : 1))
     k_far_batch(const BatchAsmProb *__restrict__ prob, const int4 *__restrict__ items)
 {
@@ -1060,7 +1230,7 @@ __global__ void __launch_bounds__(C, (MB > 0 ? MB : 1))
     if constexpr (std::is_same<T, double>::value)
         far_f64_body<R, C>(pb->q64, (double *)pb->V, ld, N, N, it.y, it.z);
     else if constexpr (std::is_same<T, float2>::value)
-        far_df_body<R, C, MB, UB>(pb->qdf, (float2 *)pb->V, ld, N, N, it.y, it.z);
+        far_df_body<R, C>(pb->qdf, (float2 *)pb->V, ld, N, N, it.y, it.z);
     else
         far_f32_body<R, C>(pb->q32, pb->cent, (float *)pb->V, ld, N, N, it.y, it.z);
 }
@@ -1115,11 +1285,11 @@ void batch_far_items(int v, int p, int64_t N, std::vector<int4> &items)
             if (i0 <= c + C - 1) items.push_back(make_int4(p, (int)i0, (int)c, 0));
 }
 
-template <typename T, int R, int C, int MB = 0, bool UB = false>
+template <typename T, int R, int C, int MB = 0>
 static void far_batch_launch(const BatchAsm &b, cudaStream_t s)
 {
     const size_t smem = std::is_same<T, float2>::value ? far_df_smem<C>() : 0;
-    k_far_batch<T, R, C, MB, UB><<<(unsigned)b.n_far, C, smem, s>>>(b.prob, b.far_items);
+    k_far_batch<T, R, C, MB><<<(unsigned)b.n_far, C, smem, s>>>(b.prob, b.far_items);
 }
 
 // The DF64 tiles of 256 columns whose shared memory (row staging + the column
@@ -1129,9 +1299,9 @@ static bem_status far_df_attributes(bem_ctx *ctx)
     const int dyn = (int)far_df_smem<256>();
     BEM_CK(ctx, cudaFuncSetAttribute(k_far_df<32, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     BEM_CK(ctx, cudaFuncSetAttribute(k_far_df<64, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 32, 256, 0, false>,
+    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 32, 256, 0>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 64, 256, 0, false>,
+    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 64, 256, 0>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     return BEM_OK;
 }
@@ -1162,14 +1332,14 @@ static bem_status batch_assemble_t(bem_ctx *ctx, const BatchAsm &b, cudaEvent_t 
         case 3: far_batch_launch<T, 8, 128>(b, s); break;
         case 4: far_batch_launch<T, 16, 128>(b, s); break;
         case 5: far_batch_launch<T, 32, 128>(b, s); break;
-        case 6: far_batch_launch<T, 8, 128, 8>(b, s); break;
-        case 7: far_batch_launch<T, 16, 128, 8>(b, s); break;
-        case 8: far_batch_launch<T, 32, 128, 8>(b, s); break;
-        case 9: far_batch_launch<T, 8, 128, 9>(b, s); break;
-        case 10: far_batch_launch<T, 8, 64, 16>(b, s); break;
-        case 11: far_batch_launch<T, 8, 64, 18>(b, s); break;
-        case 12: far_batch_launch<T, 8, 128, 6, true>(b, s); break;
-        default: far_batch_launch<T, 32, 128, 6, true>(b, s); break;
+        case 6: far_batch_launch<T, 8, 128, 5>(b, s); break;
+        case 7: far_batch_launch<T, 16, 128, 5>(b, s); break;
+        case 8: far_batch_launch<T, 32, 128, 5>(b, s); break;
+        case 9: far_batch_launch<T, 4, 128, 5>(b, s); break;
+        case 10: far_batch_launch<T, 8, 64, 10>(b, s); break;
+        case 11: far_batch_launch<T, 4, 64, 10>(b, s); break;
+        case 12: far_batch_launch<T, 2, 64, 10>(b, s); break;
+        default: far_batch_launch<T, 1, 64, 10>(b, s); break;
         }
         BEM_COUNT(ctx);
         BEM_CK_LAUNCH(ctx);

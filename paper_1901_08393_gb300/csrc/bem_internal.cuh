@@ -15,11 +15,17 @@ namespace bem {
 constexpr int kQ = 7;              // far-field points per triangle (Radon degree 5)
 constexpr int kQ64Stride = 24;     // doubles per triangle in the FP64 point table
 constexpr int kQ32Stride = 24;     // floats per triangle in the FP32 offset table
-constexpr int kQdfStride = 56;     // floats per triangle in the double-float table:
+constexpr int kQdfStride = 92;     // floats per triangle in the double-float table:
                                    // [0,42) offsets hi/lo, [42,51) centroid as 3 floats
                                    // per coordinate, [51,53) area hi/lo, [53] the
                                    // largest |hi| of the offsets, [54] the largest
-                                   // distance of a point from the centroid
+                                   // distance of a point from the centroid, [56,92)
+                                   // nine float4 of the expanded form (kQdfExp)
+constexpr int kQdfExp = 56;        // offsets of the first orbit's points of vertices 0 and 1
+                                   // (x, y, z as hi/lo: 12 floats), per vertex k |o_1k|^2 and
+                                   // |o_2k|^2 as hi/lo (3 x 4), then the centroid's first,
+                                   // second and third floats with [w] = the largest point
+                                   // distance, the area's hi and lo
 constexpr int kMaxSS = 16;         // largest Sauter-Schwab order accepted
 constexpr int kMaxValence = 96;    // triangles per vertex accepted by the pair builder
 constexpr double kInv4Pi = 0.079577471545947668;  // 1 / (4 pi)

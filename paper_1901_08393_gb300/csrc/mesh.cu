@@ -314,6 +314,29 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
     f[53] = rm;
     f[54] = __double2float_ru(sqrt(rd2) * (1.0 + 1e-12));
     f[55] = 0.0f;
+    // expanded form: orbit offsets o_1k = t (P_k - c), t = 1 - 3 a of the first orbit, and
+    // their squared lengths (o_2k = s o_1k; vertex 2's offset as minus the others' sum)
+    float *g = f + kQdfExp;
+    const double r15 = sqrt(15.0), ot = (1.0 + r15) / 7.0, os = (1.0 - r15) / (1.0 + r15);
+    double o1[3][3];
+    for (int c = 0; c < 3; ++c) {
+        o1[0][c] = ot * R[0][c];
+        o1[1][c] = ot * R[1][c];
+        o1[2][c] = -(o1[0][c] + o1[1][c]);
+        split2(o1[0][c], g + 2 * c);
+        split2(o1[1][c], g + 6 + 2 * c);
+        g[24 + c] = f[42 + 3 * c];
+        g[28 + c] = f[43 + 3 * c];
+        g[32 + c] = f[44 + 3 * c];
+    }
+    for (int k = 0; k < 3; ++k) {
+        const double n2 = (o1[k][0] * o1[k][0] + o1[k][1] * o1[k][1]) + o1[k][2] * o1[k][2];
+        split2(n2, g + 12 + 4 * k);
+        split2(os * os * n2, g + 14 + 4 * k);
+    }
+    g[27] = f[54];
+    g[31] = f[51];
+    g[35] = f[52];
     cent[4 * t + 0] = c3[0];
     cent[4 * t + 1] = c3[1];
     cent[4 * t + 2] = c3[2];
