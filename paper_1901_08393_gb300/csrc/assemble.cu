@@ -31,6 +31,7 @@
 //    rule with >= 2 points gives in those variables -- and the remaining
 //    variables use n Gauss-Legendre points each: identical 6 hexagon sectors x n,
 //    common edge 4 sub-regions x n^2, common vertex 2 regions x n^3.  FP64.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -1090,7 +1091,27 @@ static bem_status far_variant(bem_operator *op, int64_t K, int64_t N, int *v_out
     return BEM_OK;
 }
 
-int far_cached_variant(const bem_ctx *ctx, int precision, int64_t N) { return ctx->far_tile[precision][far_bucket(N)]; }
+// A batch lists its tiles: below kFarBatchArea entries each the list would outgrow what is
+// set aside for it, so only meshes of the smallest class (N < 1,024) take such tiles there.
+constexpr int kFarBatchArea = 512;
+int far_batch_variant(const bem_ctx *ctx, int precision, int64_t N)
+{
+    const int v = std::max<int>(0, ctx->far_tile[precision][far_bucket(N)]);
+    return far_bucket(N) > 0 && kFarTiles[v].rows * kFarTiles[v].cols < kFarBatchArea ? 6 : v;
+}
+
+double far_batch_items_bound(int tile, int64_t N)
+{
+    int R = 8, C = 64;  // the smallest tile of kFarBatchArea entries or more
+    if (tile > 0) {
+        R = kFarTiles[tile - 1].rows;
+        C = kFarTiles[tile - 1].cols;
+    } else if (far_bucket(N) == 0) {
+        R = 1;
+    }
+    const double n = (double)N;
+    return n * n / (2.0 * R * C) + n / R + 2.0;
+}
 
 bem_status far_tune(bem_operator *op)
 {

@@ -239,8 +239,11 @@ bem_status batch_assemble(bem_ctx *ctx, const BatchAsm &b, cudaEvent_t *ev);
 // Record e on the context's stream so that it also fires in replays of a graph being
 // captured from that stream.
 bem_status record_timing_event(bem_ctx *ctx, cudaEvent_t e);
-// The autotuned far-field variant of (precision, N) in ctx, or -1 while not timed.
-int far_cached_variant(const bem_ctx *ctx, int precision, int64_t N);
+// The autotuned far-field variant of (precision, N) in ctx for a batch wave whose largest
+// mesh has N triangles (0 while not timed), and a bound on the tiles listed for a mesh
+// (tile: the requested variant, 0 for the autotuned one).
+int far_batch_variant(const bem_ctx *ctx, int precision, int64_t N);
+double far_batch_items_bound(int tile, int64_t N);
 
 // ----------------------------------------------------------------- solve (solve.cu)
 bem_status matvec_f64(bem_operator *op, const double *x, double *y);

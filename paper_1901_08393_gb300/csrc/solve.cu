@@ -2477,14 +2477,15 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
         size_t fr = 0, tot = 0;
         if (e == cudaSuccess) e = cudaMemGetInfo(&fr, &tot);
         if (e != cudaSuccess) return fail(cuda_error(ctx, e, "batch memory query"));
-        // room for what is allocated after the arena: the far-field work lists (bounded
-        // by the smallest tile, 8 x 64), the cluster orders and the wave tables
+        // room for what is allocated after the arena: the far-field work lists, the
+        // cluster orders and the wave tables
+        const int tile = aopts && aopts->tile >= 0 && aopts->tile <= BEM_FAR_TILE_VARIANTS ? aopts->tile : 0;
         double later = 4.0 * 1048576.0;
         for (int p = 0; p < count; ++p) {
             const double N = (double)meshes[p]->N;
             int64_t n2 = 2;
             while (n2 < meshes[p]->N) n2 <<= 1;
-            later += 16.0 * (N * N / 1024.0 + N / 8.0 + 2.0) + 1024.0 + sizeof(PcgArgs) + 512.0;
+            later += 16.0 * far_batch_items_bound(tile, meshes[p]->N) + 1024.0 + sizeof(PcgArgs) + 512.0;
             if (block) later += 8.0 * (double)n2 + 4.0 * kBJ * std::ceil(N / kBJ) + 6.0 * 8.0 * 80.0 + 1024.0;
         }
         avail = (int64_t)((double)fr * 0.9) - (int64_t)later;
@@ -2740,7 +2741,7 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
         // one far-field tile for the wave: the autotuned one of its largest size class
         // (or the requested one)
         const int tile_req = aopts ? aopts->tile : 0;
-        w.variant = tile_req > 0 ? tile_req - 1 : std::max(0, far_cached_variant(ctx, prec, nmax));
+        w.variant = tile_req > 0 ? tile_req - 1 : far_batch_variant(ctx, prec, nmax);
         items.clear();
         for (int k = 0; k < P; ++k) batch_far_items(w.variant, k, bt->prob[w.first + k].op->N, items);
         int4 *d_items = nullptr;
