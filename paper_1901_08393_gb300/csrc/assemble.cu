@@ -1110,7 +1110,7 @@ double far_batch_items_bound(int tile, int64_t N)
         R = 1;
     }
     const double n = (double)N;
-    return n * n / (2.0 * R * C) + n / R + 2.0;
+    return n * n / (2.0 * R * C) + n / std::min(R, 4) + 2.0;  // 4 x 128 has the fewest rows of that area
 }
 
 bem_status far_tune(bem_operator *op)

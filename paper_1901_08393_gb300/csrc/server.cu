@@ -81,7 +81,7 @@ int64_t estimate_bytes(int64_t N0, int64_t max_N, int32_t levels, int precision,
     const double n = (levels <= 1 ? (double)N0 : reach) + 64.0;
     if (basis == BEM_BASIS_DUAL) return (int64_t)((72.0 * es + 4.0) * n * n + 6.0 * 4096.0 * n) + (64ll << 20);
     const double ops = levels <= 1 ? (precision == BEM_PREC_DF64 ? 1.25 : precision == BEM_PREC_F32 ? 1.5 : 1.0) : 2.0;
-    return (int64_t)(ops * es * n * n + 4096.0 * n) + (64ll << 20);
+    return (int64_t)(ops * es * n * n + 4608.0 * n) + (64ll << 20);
 }
 
 // A request on its slot's context (one per slot, kept across requests: its stream,

@@ -13,6 +13,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_fp16.h>
@@ -263,9 +264,35 @@ __device__ __forceinline__ int symv_grab(unsigned long long *ctr, unsigned long 
     return s_k;
 }
 
-// pack (nullable): also write the FP32 hi parts of each staged tile, row-major
-// 64 x 64 at pack + 4096 k for tile k of the list (the packed upper triangle).
+// pack (nullable): also write the FP32 hi parts of each staged tile, scaled by pack_sc,
+// row-major 64 x 64 at pack + 4096 k for tile k of the list (the packed upper triangle),
+// and its exponents at pack_ex + kTileExp k.
 constexpr int kTileF = kSB * kSB;
+// A packed copy is followed by the scales 2^k of the rows (ld floats) and kTileExp bytes per
+// tile: the biased exponents of the largest scaled entry of rows 4 g .. 4 g + 3 (g < 16),
+// then of columns 4 g .. 4 g + 3.
+constexpr int kTileExp = 2 * kSB / 4;
+__host__ __device__ __forceinline__ size_t packed_bytes(size_t nt, size_t ld)
+{
+    return nt * kTileF * sizeof(float) + ld * sizeof(float) + nt * kTileExp;
+}
+__host__ __device__ __forceinline__ float *packed_scale(float *vp, size_t nt) { return vp + nt * kTileF; }
+__host__ __device__ __forceinline__ unsigned char *packed_exps(float *vp, size_t nt, size_t ld)
+{
+    return reinterpret_cast<unsigned char *>(packed_scale(vp, nt) + ld);
+}
+
+// 2^k with 4^k <= |d| < 4^(k + 1) (1 for zero, infinity and NaN), kept well inside the
+// FP32 range.
+__device__ __forceinline__ float tile_scale(double d)
+{
+    const int e = (int)((__double2hiint(d) >> 20) & 0x7ff);
+    if (e == 0 || e == 0x7ff) return 1.0f;
+    return __int_as_float((127 + min(max((e - 1023) >> 1, -60), 60)) << 23);
+}
+// 1 / s for a power of two s
+__device__ __forceinline__ float recip_pow2(float s) { return __int_as_float((254 << 23) - __float_as_int(s)); }
+
 // BEM_PRODUCTS_FP16: replaced residual after every 10^2-fold drop of ||r|| (r.r by
 // 10^4); fallback to the exact products when a replacement finds r.r above
 // kH16Progress times the previous replacement's (||r|| fallen by less than 10x)
@@ -278,7 +305,8 @@ constexpr int kH16SegMax = 400;
 __device__ void symv_tiles(const float2 *__restrict__ V, int64_t ld, int64_t N, const int2 *__restrict__ tiles,
                            int ntiles, const float2 *__restrict__ xdf, float2 *__restrict__ prow,
                            float2 *__restrict__ pcol, float2 *sm, int cta, int G,
-                           unsigned long long *ctr = nullptr, unsigned long long base = 0, float *pack = nullptr)
+                           unsigned long long *ctr = nullptr, unsigned long long base = 0, float *pack = nullptr,
+                           const float *pack_sc = nullptr, unsigned char *pack_ex = nullptr)
 {
     // [tile buffer 0][tile buffer 1][x segments 0][x segments 1][column partials 4 x 64]
     float2 *const xs0 = sm + 2 * kSB * kSP;
@@ -300,13 +328,40 @@ __device__ void symv_tiles(const float2 *__restrict__ V, int64_t ld, int64_t N, 
         const float2 *xi = xs0 + cur * 2 * kSB, *xj = xi + kSB;
         const int64_t base = (int64_t)k * kSB;
         if (pack) {
+            // scaled (see symv_hi_tiles); 1 / scales of rows and columns in cpart
+            float *rs = reinterpret_cast<float *>(cpart);
+            if (t < 2 * kSB) rs[t] = recip_pow2(__ldcg(pack_sc + (int64_t)(t < kSB ? tj.x : tj.y) * kSB + (t & (kSB - 1))));
+            __syncthreads();
             float4 *dst = reinterpret_cast<float4 *>(pack + (int64_t)k * kTileF);
+            unsigned *ms = reinterpret_cast<unsigned *>(rs) + 2 * kSB;  // [4][8] rows, then [8][16] columns
+            float cm = 0.f;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int f = t + kSymThreads * u;  // float4 f: row f / 16, columns 4 (f % 16) ..
                 const float2 *src = T + (f >> 4) * kSP + 4 * (f & 15);
-                dst[f] = make_float4(src[0].x, src[1].x, src[2].x, src[3].x);
+                const float p = rs[f >> 4];
+                const float4 q = *reinterpret_cast<const float4 *>(rs + kSB + 4 * (f & 15));
+                const float4 v = make_float4(src[0].x * p * q.x, src[1].x * p * q.y, src[2].x * p * q.z,
+                                             src[3].x * p * q.w);
+                dst[f] = v;
+                const float m = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+                cm = fmaxf(cm, m);
+                const unsigned wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));  // rows 16 u + 2 (warp) + {0, 1}
+                if ((t & 31) == 0) ms[8 * u + (t >> 5)] = wm;
             }
+            cm = fmaxf(cm, __shfl_xor_sync(0xffffffffu, cm, 16));
+            if ((t & 31) < 16) ms[32 + 16 * (t >> 5) + (t & 15)] = __float_as_uint(cm);
+            __syncthreads();
+            if (t < kTileExp) {
+                unsigned e = 0;
+                if (t < 16) {  // rows 4 t .. 4 t + 3: two warps of one u
+                    e = max(ms[8 * (t >> 2) + 2 * (t & 3)], ms[8 * (t >> 2) + 2 * (t & 3) + 1]);
+                } else {
+                    for (int w = 0; w < kSymThreads / 32; ++w) e = max(e, ms[32 + 16 * w + (t & 15)]);
+                }
+                pack_ex[(int64_t)k * kTileExp + t] = (unsigned char)(e >> 23);
+            }
+            __syncthreads();
         }
         {  // row pass: row r, columns q, q+4, ..., q+60
             const int r = t >> 2, q = t & 3;
@@ -446,11 +501,25 @@ __device__ __forceinline__ double symv_row4(const float2 *__restrict__ prow, con
 // iteration products of the mixed-precision solver): exact FP32 x FP32 products
 // and double-float sums, as the DF64 product but reading 4 instead of 8 bytes per
 // entry.  Each warp takes whole tiles from the counter (one 16 KB contiguous
-// block per tile); lane l covers columns 4 (l % 16) .. +3 and rows 32 (l / 16) ..
-// +31, eight rows per step.  Row partials (V_IJ x_J) are summed over the 16 lanes
-// of a row half by a halving butterfly, column partials (V_IJ^T x_I, off the
-// diagonal) over the two row halves; both in the DF64 partial layout.
-// xsw: 128 pairs of shared memory per warp.
+// block per tile).
+//
+// The packed entries are scaled by powers of two, v' = v 2^-(k_r + k_c) with 4^k <= |V_ii|
+// < 4^(k + 1) (exact; the vector by 2^k_c when it is staged, the sums by 2^k_r when they
+// are stored), so that the entries of a tile are of similar size however small some of its
+// triangles are.
+//
+// A two-product and a two-sum for each of the entry's two products took 22 FP32
+// operations.  Here each lane's sum starts from big = 1.5 * 2^E, an FMA adds the product
+// (rounded to a multiple of q = 2^(E-23)), the difference of the two sums is exact, and an
+// FMA gives what the rounding left of the product; with the product by the vector's lo
+// part, 5 operations, and 5 instructions for two entries as packed pairs.  2^(E-3) (rows, 8
+// products a lane) or 2^(E-4) (columns, 16) bounds |v' x'|, from the exponents of the
+// largest entry of four rows or columns, kept with the tile, and of the lane's values of
+// the vector: the sum stays between 2^(E-1) and 2.5 * 2^E, above every product.  The lo
+// sum's error is a few units of 2^-24 q, 2^-43 of the largest product.  The lanes' sums are
+// added by two-sums.  Bound by HBM: 163 us at N = 21,744 (946 MB, 5.8 TB/s of 6.76
+// measured) with 16 warps of 128 registers per SM, against 211 us with either kind of sums
+// and 24 warps of 80.
 __device__ __forceinline__ int warp_grab(unsigned long long *ctr, unsigned long long base)
 {
     int k = 0;
@@ -469,81 +538,249 @@ __device__ __forceinline__ void acc_hi(float &sh, float &sl, float v, float xh, 
     sl = __fadd_rn(sl, __fadd_rn(e, t));
 }
 
+// The grid of a sum: 1.5 * 2^E, E = up + the exponents of the entries and of the vector x
+// (both biased), kept where 2^(E-47) is a normal number.
+__device__ __forceinline__ f2 sum_grid(unsigned e, float x, int up)
+{
+    const int E = min(max((int)(e + (__float_as_uint(x) >> 23)) + (up - 127), 50), 250);
+    const float b = __uint_as_float(((unsigned)E << 23) | 0x400000u);
+    return f2_make(b, b);
+}
+
+// Shared memory of one warp: x'_I as (h, h, l, l), x'_J's hi and lo parts, the scales.
+struct HiStage {
+    float4 xi[kSB];
+    float xjh[kSB], xjl[kSB], si[kSB], sj[kSB];
+};
+
 __device__ __forceinline__ float2 shfl_df(float2 v, int o)
 {
     return make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o));
 }
 
+// One product step on a packed pair of sums: (s, l) += v (xh + xl)
+__device__ __forceinline__ void grid_acc(f2 &s, f2 &l, f2 v, f2 xh, f2 xl)
+{
+    const f2 t = f2_fma(v, xh, s);
+    const f2 r = f2_fma(v, xl, f2_fma(v, xh, f2_sub(s, t)));
+    s = t;
+    l = f2_add(l, r);
+}
+
+// The same with a two-product and a two-sum, for any sizes of s and of the product: 11
+// instructions for two products.  The lo sum's error is 2^-24 of itself, 2^-48 of s.
+__device__ __forceinline__ void two_sum_acc(f2 &s, f2 &l, f2 v, f2 xh, f2 xl)
+{
+    const f2 p = f2_fma(v, xh, 0ull), t = f2_add(s, p), b = f2_sub(t, s);
+    const f2 e = f2_add(f2_sub(s, f2_sub(t, b)), f2_sub(p, b));
+    const f2 r = f2_fma(v, xl, f2_fma(v, xh, f2_neg(p)));
+    s = t;
+    l = f2_add(l, f2_add(r, e));
+}
+
+// kGrid: sums on grids (the products of the iteration); else by two-sums (the residuals of
+// FP32 operators, which decide convergence, and the operator preconditioner C, whose sums
+// cancel far more than V's: with the grids the preconditioned solves took 0.6 iterations
+// of 28 more).
+// Lane l covers columns 4 (l % 8) .. +3 and 32 + 4 (l % 8) .. +3 of rows 16 (l / 8) ..
+// +15, four rows per step.  Row partials (V_IJ x_J) are summed over the 8 lanes of a row
+// by a halving butterfly, column partials (V_IJ^T x_I, off the diagonal) over the four
+// row groups; both in the DF64 partial layout.
 // static_k >= 0: at most one tile per warp, this one (no counter: when there are no
 // more tiles than warps, dynamic grabs only add two L2 atomic round trips)
-__device__ void symv_hi_tiles(const float *__restrict__ vp, const int2 *__restrict__ tiles, int ntiles,
+template <bool kGrid>
+__device__ void symv_hi_tiles(const float *__restrict__ vp, const float *__restrict__ sc,
+                              const unsigned char *__restrict__ vex, const int2 *__restrict__ tiles, int ntiles,
                               const float2 *__restrict__ xdf, float2 *__restrict__ prow, float2 *__restrict__ pcol,
-                              float2 *xsw, unsigned long long *ctr, unsigned long long base, int static_k = -1)
+                              HiStage *st, unsigned long long *ctr, unsigned long long base, int static_k = -1)
 {
-    const int lane = threadIdx.x & 31, cg = lane & 15, par = lane >> 4;
-    const bool b1 = lane & 2, b2 = lane & 4, b3 = lane & 8;
+    const int lane = threadIdx.x & 31, cg = lane & 7, rg = lane >> 3;
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, b3 = lane & 8, b4 = lane & 16;
     for (int k = static_k >= 0 ? static_k : warp_grab(ctr, base); k < ntiles;
          k = static_k >= 0 ? ntiles : warp_grab(ctr, base)) {
         const int2 tj = tiles[k];
+        const unsigned char *te = vex + (int64_t)k * kTileExp;
+        const unsigned er = __ldcg(reinterpret_cast<const unsigned *>(te) + rg);  // rows 16 rg .. +15, four a byte
+        const unsigned ec[2] = {__ldcg(te + 16 + cg), __ldcg(te + 24 + cg)};
+        float2 x[4];  // I: lane, 32 + lane, J: the same
+        float s4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = (int64_t)(u < 2 ? tj.x : tj.y) * kSB + 32 * (u & 1) + lane;
+            x[u] = __ldcg(xdf + i);
+            s4[u] = __ldcg(sc + i);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            x[u].x *= s4[u];
+            x[u].y *= s4[u];
+        }
+        // the largest of x'_I on rows 16 rg .. +15
+        float mi[2] = {fabsf(x[0].x), fabsf(x[1].x)};
+#pragma unroll
+        for (int o = 1; o < 16; o <<= 1) {
+            mi[0] = fmaxf(mi[0], __shfl_xor_sync(0xffffffffu, mi[0], o));
+            mi[1] = fmaxf(mi[1], __shfl_xor_sync(0xffffffffu, mi[1], o));
+        }
+        mi[0] = __shfl_sync(0xffffffffu, mi[0], 16 * (rg & 1));
+        mi[1] = __shfl_sync(0xffffffffu, mi[1], 16 * (rg & 1));
+        const float xim = rg & 2 ? mi[1] : mi[0];
+        const f2 cbig[2] = {kGrid ? sum_grid(ec[0], xim, 6) : 0ull, kGrid ? sum_grid(ec[1], xim, 6) : 0ull};
         __syncwarp();
-        // x_I in xsw[0..63] (lanes 0..15), x_J in xsw[64..127] (lanes 16..31)
-        {
-            const float4 *src = reinterpret_cast<const float4 *>(xdf + (int64_t)(par ? tj.y : tj.x) * kSB) + 2 * cg;
-            float4 *dst = reinterpret_cast<float4 *>(xsw) + 2 * lane;
-            dst[0] = __ldcg(src);
-            dst[1] = __ldcg(src + 1);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            st->xi[32 * u + lane] = make_float4(x[u].x, x[u].x, x[u].y, x[u].y);
+            st->xjh[32 * u + lane] = x[2 + u].x;
+            st->xjl[32 * u + lane] = x[2 + u].y;
+            st->si[32 * u + lane] = s4[u];
+            st->sj[32 * u + lane] = s4[2 + u];
         }
         __syncwarp();
-        float2 xc[4];
+        f2 xh[4], xl[4], cs[4], cl[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xc[u] = xsw[kSB + 4 * cg + u];
-        const float4 *T = reinterpret_cast<const float4 *>(vp + (int64_t)k * kTileF);
-        float2 cs[4];
+        for (int u = 0; u < 4; ++u) {  // column pairs: 4 cg + {0, 1}, {2, 3}, then 32 columns on
+            const int c = 32 * (u >> 1) + 4 * cg + 2 * (u & 1);
+            xh[u] = *reinterpret_cast<const f2 *>(st->xjh + c);
+            xl[u] = *reinterpret_cast<const f2 *>(st->xjl + c);
+            cs[u] = cbig[u >> 1];
+            cl[u] = 0ull;
+        }
+        float xjm = 0.0f;  // the largest of the lane's x'_J
 #pragma unroll
-        for (int u = 0; u < 4; ++u) cs[u] = make_float2(0.f, 0.f);
+        for (int u = 0; u < 4; ++u) {
+            const float2 t = f2_get(xh[u]);
+            xjm = fmaxf(xjm, fmaxf(fabsf(t.x), fabsf(t.y)));
+        }
+        const float4 *T = reinterpret_cast<const float4 *>(vp + (int64_t)k * kTileF) + 256 * rg + cg;
 #pragma unroll 1
         for (int ch = 0; ch < 4; ++ch) {
-            const int r0 = 32 * par + 8 * ch;
             float4 v[8];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) v[m] = __ldcs(T + (r0 + m) * 16 + cg);
-            float2 sr[8];
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const float2 xr = xsw[r0 + m];
-                const float e[4] = {v[m].x, v[m].y, v[m].z, v[m].w};
-                // the row sum starts from the first exact product itself (a two-sum
-                // with zero adds nothing)
-                float h, l;
-                two_prod(e[0], xc[0].x, h, l);
-                l = __fmaf_rn(e[0], xc[0].y, l);
-#pragma unroll
-                for (int u = 1; u < 4; ++u) acc_hi(h, l, e[u], xc[u].x, xc[u].y);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) acc_hi(cs[u].x, cs[u].y, e[u], xr.x, xr.y);
-                sr[m] = make_float2(h, l);
+            for (int m = 0; m < 4; ++m) {
+                v[2 * m] = __ldcs(T + (4 * ch + m) * 16);
+                v[2 * m + 1] = __ldcs(T + (4 * ch + m) * 16 + 8);
             }
-            // rows m of this lane: 8 -> 4 (xor 8) -> 2 (xor 4) -> 1 (xor 2), then xor 1
-            // (renormalised there); lane keeps row (l / 2) % 8
-            float2 t4[4], t2[2];
+            const f2 rbig = kGrid ? sum_grid((er >> (8 * ch)) & 0xffu, xjm, 5) : 0ull;
+            float2 h[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) t4[j] = df_add_u(b3 ? sr[j + 4] : sr[j], shfl_df(b3 ? sr[j] : sr[j + 4], 8));
+            for (int m = 0; m < 4; ++m) {
+                const int r = 16 * rg + 4 * ch + m;
+                const float4 x = st->xi[r];
+                const f2 rh = f2_make(x.x, x.y), rl = f2_make(x.z, x.w);
+                const f2 e[4] = {f2_make(v[2 * m].x, v[2 * m].y), f2_make(v[2 * m].z, v[2 * m].w),
+                                 f2_make(v[2 * m + 1].x, v[2 * m + 1].y), f2_make(v[2 * m + 1].z, v[2 * m + 1].w)};
+                f2 s = rbig, sl = 0ull;
 #pragma unroll
-            for (int j = 0; j < 2; ++j) t2[j] = df_add_u(b2 ? t4[j + 2] : t4[j], shfl_df(b2 ? t4[j] : t4[j + 2], 4));
-            float2 w = df_add_u(b1 ? t2[1] : t2[0], shfl_df(b1 ? t2[0] : t2[1], 2));
+                for (int u = 0; u < 4; ++u) {
+                    if (kGrid) {
+                        grid_acc(s, sl, e[u], xh[u], xl[u]);
+                        grid_acc(cs[u], cl[u], e[u], rh, rl);
+                    } else {
+                        two_sum_acc(s, sl, e[u], xh[u], xl[u]);
+                        two_sum_acc(cs[u], cl[u], e[u], rh, rl);
+                    }
+                }
+                const float2 a = f2_get(kGrid ? f2_sub(s, rbig) : s), b = f2_get(sl);
+                if (kGrid)  // multiples of one q
+                    h[m] = make_float2(a.x + a.y, b.x + b.y);
+                else
+                    h[m] = df_add_u(make_float2(a.x, b.x), make_float2(a.y, b.y));
+            }
+            // rows m of this lane's group: 4 -> 2 (xor 4) -> 1 (xor 2), then xor 1
+            float2 g[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) g[j] = df_add_u(b2 ? h[j + 2] : h[j], shfl_df(b2 ? h[j] : h[j + 2], 4));
+            float2 w = df_add_u(b1 ? g[1] : g[0], shfl_df(b1 ? g[0] : g[1], 2));
             const float2 o = shfl_df(w, 1);
-            w = (lane & 1) ? df_add(o, w) : df_add(w, o);
-            if (!(lane & 1)) prow[(int64_t)k * kSB + r0 + ((lane >> 1) & 7)] = w;
+            w = b0 ? df_add(o, w) : df_add(w, o);
+            if (!b0) {
+                const int r = 16 * rg + 4 * ch + (b2 ? 2 : 0) + (b1 ? 1 : 0);
+                const float sr = st->si[r];
+                prow[(int64_t)k * kSB + r] = make_float2(w.x * sr, w.y * sr);
+            }
         }
-        if (tj.x != tj.y) {  // lane keeps columns 4 (l % 16) + 2 (l / 16) + {0, 1}, rows 0..31 first
-            const float2 a0 = shfl_df(par ? cs[0] : cs[2], 16), a1 = shfl_df(par ? cs[1] : cs[3], 16);
-            float4 out;
-            const float2 s0 = par ? df_add(a0, cs[2]) : df_add(cs[0], a0);
-            const float2 s1 = par ? df_add(a1, cs[3]) : df_add(cs[1], a1);
-            out = make_float4(s0.x, s0.y, s1.x, s1.y);
-            reinterpret_cast<float4 *>(pcol + (int64_t)k * kSB)[2 * cg + par] = out;
+        if (tj.x != tj.y) {  // lane keeps columns 32 (b4) + 4 cg + 2 (b3) + {0, 1}
+            float2 a[8];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float2 hh = f2_get(kGrid ? f2_sub(cs[u], cbig[u >> 1]) : cs[u]), ll = f2_get(cl[u]);
+                a[2 * u] = make_float2(hh.x, ll.x);
+                a[2 * u + 1] = make_float2(hh.y, ll.y);
+            }
+            float2 c4[4], c2[2];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c4[j] = df_add_u(b4 ? a[j + 4] : a[j], shfl_df(b4 ? a[j] : a[j + 4], 16));
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float2 keep = b3 ? c4[j + 2] : c4[j], o = shfl_df(b3 ? c4[j] : c4[j + 2], 8);
+                c2[j] = df_add(keep, o);
+            }
+            const int c = (b4 ? 32 : 0) + 4 * cg + (b3 ? 2 : 0);
+            const float2 sj = *reinterpret_cast<const float2 *>(st->sj + c);
+            *reinterpret_cast<float4 *>(pcol + (int64_t)k * kSB + c) =
+                make_float4(c2[0].x * sj.x, c2[0].y * sj.x, c2[1].x * sj.y, c2[1].y * sj.y);
         }
     }
+}
+
+// Tile k of the packed copy from the entries of an FP32 matrix, by one warp in the lane
+// layout of symv_hi_tiles, and its exponents.
+__device__ __forceinline__ void pack_tile_f32(const float *__restrict__ V, int64_t ld, int64_t N, int2 tj, int64_t k,
+                                              float *__restrict__ vp, const float *__restrict__ sc,
+                                              unsigned char *__restrict__ vex)
+{
+    const int lane = threadIdx.x & 31, cg = lane & 7, rg = lane >> 3;
+    float4 *dst = reinterpret_cast<float4 *>(vp + k * kTileF);
+    const float4 *sj = reinterpret_cast<const float4 *>(sc + (int64_t)tj.y * kSB);
+    const float4 c0 = sj[cg], c1 = sj[8 + cg];
+    const float q[8] = {recip_pow2(c0.x), recip_pow2(c0.y), recip_pow2(c0.z), recip_pow2(c0.w),
+                        recip_pow2(c1.x), recip_pow2(c1.y), recip_pow2(c1.z), recip_pow2(c1.w)};
+    unsigned char *ex = vex + k * kTileExp;
+    float ca = 0.0f, cb = 0.0f;  // the lane's columns, over its rows
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+        float rm = 0.0f;
+#pragma unroll
+        for (int m = 4 * g; m < 4 * g + 4; ++m) {
+            const int r = 16 * rg + m;
+            const int64_t row = (int64_t)tj.x * kSB + r;
+            float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+            if (row < N) {
+                const float4 *src = reinterpret_cast<const float4 *>(V + row * ld + (int64_t)tj.y * kSB);
+                a = __ldcs(src + cg);
+                b = __ldcs(src + 8 + cg);
+            }
+            const float p = recip_pow2(sc[row]);
+            a = make_float4(a.x * p * q[0], a.y * p * q[1], a.z * p * q[2], a.w * p * q[3]);
+            b = make_float4(b.x * p * q[4], b.y * p * q[5], b.z * p * q[6], b.w * p * q[7]);
+            dst[r * 16 + cg] = a;
+            dst[r * 16 + 8 + cg] = b;
+            const float ma = fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fmaxf(fabsf(a.z), fabsf(a.w)));
+            const float mb = fmaxf(fmaxf(fabsf(b.x), fabsf(b.y)), fmaxf(fabsf(b.z), fabsf(b.w)));
+            rm = fmaxf(rm, fmaxf(ma, mb));
+            ca = fmaxf(ca, ma);
+            cb = fmaxf(cb, mb);
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) rm = fmaxf(rm, __shfl_xor_sync(0xffffffffu, rm, o));
+        if (cg == 0) ex[4 * rg + g] = (unsigned char)(__float_as_uint(rm) >> 23);
+    }
+#pragma unroll
+    for (int o = 8; o < 32; o <<= 1) {
+        ca = fmaxf(ca, __shfl_xor_sync(0xffffffffu, ca, o));
+        cb = fmaxf(cb, __shfl_xor_sync(0xffffffffu, cb, o));
+    }
+    if (rg == 0) {
+        ex[16 + cg] = (unsigned char)(__float_as_uint(ca) >> 23);
+        ex[24 + cg] = (unsigned char)(__float_as_uint(cb) >> 23);
+    }
+}
+
+// The scales of an FP32 matrix's rows from its diagonal.
+__global__ void k_tile_scale(const float *__restrict__ V, int64_t ld, int64_t N, float *__restrict__ sc)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < ld) sc[i] = i < N ? tile_scale((double)V[i * ld + i]) : 1.0f;
 }
 
 // FP16 working copy of the packed tiles (BEM_PRODUCTS_FP16).  Each 64 x 64 tile is
@@ -581,74 +818,99 @@ __global__ void k_pack_h16(const float *__restrict__ vp, int ntiles, __half *__r
     pack_h16_tiles(vp, ntiles, vh, vsc, w0, ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
 
-// Product with the FP16 working copy: the layout and partials of symv_hi_tiles (lane
-// l: columns 4 (l % 16) .. +3, rows 32 (l / 16) + 8 c .. +7 in step c), 8 bytes per
-// lane and row, FP32 products of the half entries with the hi part of x and FP32
-// sums; the tile's scale multiplies its partials.  The iteration products of
+// Product with the FP16 working copy: FP32 products of the half entries with the hi part
+// of x and FP32 sums, two entries per instruction (packed pairs); the tile's scale
+// multiplies its partials.  Lane l covers columns 8 (l % 8) .. +7 (16 bytes) of rows 16
+// (l / 8) .. +15, eight rows per step: 4 KB in flight per warp, so that two CTAs per SM
+// keep HBM busy.  Partials as symv_hi_tiles.  The iteration products of
 // BEM_PRODUCTS_FP16 only: the residuals that decide convergence use the exact form.
 __device__ void symv_h16_tiles(const __half *__restrict__ vh, const float *__restrict__ vsc,
-                               const int2 *__restrict__ tiles, int ntiles, const float2 *__restrict__ xdf,
-                               float2 *__restrict__ prow, float2 *__restrict__ pcol, float2 *xsw,
-                               unsigned long long *ctr, unsigned long long base, int static_k = -1)
+                               const float *__restrict__ sc, const int2 *__restrict__ tiles, int ntiles,
+                               const float2 *__restrict__ xdf, float2 *__restrict__ prow, float2 *__restrict__ pcol,
+                               HiStage *st, unsigned long long *ctr, unsigned long long base, int static_k = -1)
 {
-    const int lane = threadIdx.x & 31, cg = lane & 15, par = lane >> 4;
-    const bool b1 = lane & 2, b2 = lane & 4, b3 = lane & 8;
+    const int lane = threadIdx.x & 31, cg = lane & 7, rg = lane >> 3;
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, b3 = lane & 8, b4 = lane & 16;
+    float2 *const xd = reinterpret_cast<float2 *>(st->xi);  // x'_I twice
     for (int k = static_k >= 0 ? static_k : warp_grab(ctr, base); k < ntiles;
          k = static_k >= 0 ? ntiles : warp_grab(ctr, base)) {
         const int2 tj = tiles[k];
-        const float sk = vsc[k];
-        __syncwarp();
-        {
-            const float4 *src = reinterpret_cast<const float4 *>(xdf + (int64_t)(par ? tj.y : tj.x) * kSB) + 2 * cg;
-            float4 *dst = reinterpret_cast<float4 *>(xsw) + 2 * lane;
-            dst[0] = __ldcg(src);
-            dst[1] = __ldcg(src + 1);
+        const float sk = __ldcg(vsc + k);
+        float x[4], s4[4];  // I: lane, 32 + lane, J: the same
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int64_t i = (int64_t)(u < 2 ? tj.x : tj.y) * kSB + 32 * (u & 1) + lane;
+            x[u] = __ldcg(&xdf[i].x);
+            s4[u] = __ldcg(sc + i);
         }
         __syncwarp();
-        float xc[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) xc[u] = xsw[kSB + 4 * cg + u].x;
-        const uint2 *T = reinterpret_cast<const uint2 *>(vh + (int64_t)k * kTileF);
-        float cs[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int u = 0; u < 2; ++u) {
+            const float xi = x[u] * s4[u];
+            xd[32 * u + lane] = make_float2(xi, xi);
+            st->xjh[32 * u + lane] = x[2 + u] * s4[2 + u];
+            st->si[32 * u + lane] = s4[u] * sk;
+            st->sj[32 * u + lane] = s4[2 + u] * sk;
+        }
+        __syncwarp();
+        f2 xc[4], cs[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            xc[u] = *reinterpret_cast<const f2 *>(st->xjh + 8 * cg + 2 * u);
+            cs[u] = 0ull;
+        }
+        const uint4 *T = reinterpret_cast<const uint4 *>(vh + (int64_t)k * kTileF) + 128 * rg + cg;
 #pragma unroll 1
-        for (int ch = 0; ch < 4; ++ch) {
-            const int r0 = 32 * par + 8 * ch;
-            uint2 raw[8];
+        for (int ch = 0; ch < 2; ++ch) {
+            uint4 raw[8];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) raw[m] = __ldcs(T + (r0 + m) * 16 + cg);
+            for (int m = 0; m < 8; ++m) raw[m] = __ldcs(T + (8 * ch + m) * 8);
             float sr[8];
 #pragma unroll
             for (int m = 0; m < 8; ++m) {
-                const float xr = xsw[r0 + m].x;
-                __half2 h01, h23;
-                memcpy(&h01, &raw[m].x, 4);
-                memcpy(&h23, &raw[m].y, 4);
-                const float2 a01 = __half22float2(h01), a23 = __half22float2(h23);
-                const float e[4] = {a01.x, a01.y, a23.x, a23.y};
-                float h = e[0] * xc[0];
+                const f2 xr = *reinterpret_cast<const f2 *>(xd + 16 * rg + 8 * ch + m);
+                const unsigned w[4] = {raw[m].x, raw[m].y, raw[m].z, raw[m].w};
+                f2 s = 0ull;
 #pragma unroll
-                for (int u = 1; u < 4; ++u) h = __fmaf_rn(e[u], xc[u], h);
-                sr[m] = h;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) cs[u] = __fmaf_rn(e[u], xr, cs[u]);
+                for (int u = 0; u < 4; ++u) {
+                    __half2 hh;
+                    memcpy(&hh, &w[u], 4);
+                    const float2 a = __half22float2(hh);
+                    const f2 e = f2_make(a.x, a.y);
+                    s = f2_fma(e, xc[u], s);
+                    cs[u] = f2_fma(e, xr, cs[u]);
+                }
+                const float2 t = f2_get(s);
+                sr[m] = t.x + t.y;
             }
-            // rows m: 8 -> 4 (xor 8) -> 2 (xor 4) -> 1 (xor 2), then xor 1
+            // rows m of this lane's group: 8 -> 4 (xor 4) -> 2 (xor 2) -> 1 (xor 1)
             float t4[4], t2[2];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                t4[j] = (b3 ? sr[j + 4] : sr[j]) + __shfl_xor_sync(0xffffffffu, b3 ? sr[j] : sr[j + 4], 8);
+                t4[j] = (b2 ? sr[j + 4] : sr[j]) + __shfl_xor_sync(0xffffffffu, b2 ? sr[j] : sr[j + 4], 4);
 #pragma unroll
             for (int j = 0; j < 2; ++j)
-                t2[j] = (b2 ? t4[j + 2] : t4[j]) + __shfl_xor_sync(0xffffffffu, b2 ? t4[j] : t4[j + 2], 4);
-            float w = (b1 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? t2[0] : t2[1], 2);
-            w += __shfl_xor_sync(0xffffffffu, w, 1);
-            if (!(lane & 1)) prow[(int64_t)k * kSB + r0 + ((lane >> 1) & 7)] = make_float2(w * sk, 0.f);
+                t2[j] = (b1 ? t4[j + 2] : t4[j]) + __shfl_xor_sync(0xffffffffu, b1 ? t4[j] : t4[j + 2], 2);
+            const float w = (b0 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, b0 ? t2[0] : t2[1], 1);
+            const int r = 16 * rg + 8 * ch + (b2 ? 4 : 0) + (b1 ? 2 : 0) + (b0 ? 1 : 0);
+            prow[(int64_t)k * kSB + r] = make_float2(w * st->si[r], 0.f);
         }
-        if (tj.x != tj.y) {  // lane keeps columns 4 (l % 16) + 2 (l / 16) + {0, 1}
-            const float a0 = __shfl_xor_sync(0xffffffffu, par ? cs[0] : cs[2], 16);
-            const float a1 = __shfl_xor_sync(0xffffffffu, par ? cs[1] : cs[3], 16);
-            const float s0 = (par ? cs[2] : cs[0]) + a0, s1 = (par ? cs[3] : cs[1]) + a1;
-            reinterpret_cast<float4 *>(pcol + (int64_t)k * kSB)[2 * cg + par] = make_float4(s0 * sk, 0.f, s1 * sk, 0.f);
+        if (tj.x != tj.y) {  // lane keeps columns 8 cg + 4 (b4) + 2 (b3) + {0, 1}
+            float2 c[4], d[2];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) c[u] = f2_get(cs[u]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const float2 keep = b4 ? c[j + 2] : c[j], give = b4 ? c[j] : c[j + 2];
+                d[j].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
+                d[j].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
+            }
+            const float2 keep = b3 ? d[1] : d[0], give = b3 ? d[0] : d[1];
+            const float s0 = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8);
+            const float s1 = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8);
+            const int q = 8 * cg + (b4 ? 4 : 0) + (b3 ? 2 : 0);
+            const float2 sj = *reinterpret_cast<const float2 *>(st->sj + q);
+            *reinterpret_cast<float4 *>(pcol + (int64_t)k * kSB + q) = make_float4(s0 * sj.x, 0.f, s1 * sj.y, 0.f);
         }
     }
 }
@@ -1000,7 +1262,7 @@ __global__ void __launch_bounds__(256) k_block_inverse(const T *__restrict__ V, 
 __device__ __forceinline__ void block_apply(const int32_t *__restrict__ perm, const double *__restrict__ binv, int blk,
                                             double *x, double *r, double *z, double *p, const double *q,
                                             float2 *pdf, double alpha, bool update, bool init, double *rs,
-                                            double &rz_l, double &rr_l)
+                                            double (&sums)[2])
 {
     const int t = threadIdx.x;
     const int32_t *pk = perm + (int64_t)blk * kBJ;
@@ -1043,8 +1305,8 @@ __device__ __forceinline__ void block_apply(const int32_t *__restrict__ perm, co
                 p[g] = sacc;
                 pdf[g] = df_from_double(sacc);
             }
-            rz_l += rv * sacc;
-            rr_l += rv * rv;
+            sums[0] += rv * sacc;
+            sums[1] += rv * rv;
         }
     }
     __syncthreads();  // rs is refilled for the next cluster
@@ -1052,19 +1314,15 @@ __device__ __forceinline__ void block_apply(const int32_t *__restrict__ perm, co
 
 // Packed upper triangle of an FP32 operator: tile k of the list, row-major 64 x 64 at
 // vp + 4096 k (rows past N zero; columns past N are the operator's zero padding).
-__global__ void k_pack_f32(const float *__restrict__ V, int64_t ld, int64_t N, const int2 *__restrict__ tiles,
-                           int64_t ntiles, float *__restrict__ vp)
+__global__ void __launch_bounds__(256) k_pack_f32(const float *__restrict__ V, int64_t ld, int64_t N,
+                                                  const int2 *__restrict__ tiles, int64_t ntiles,
+                                                  float *__restrict__ vp)
 {
-    const int64_t n4 = ntiles * (kTileF / 4);
-    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < n4; f += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = f / (kTileF / 4);
-        const int e = (int)(f % (kTileF / 4)), r = e >> 4, c4 = e & 15;
-        const int2 tj = tiles[k];
-        const int64_t row = (int64_t)tj.x * kSB + r;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row < N) v = __ldcs(reinterpret_cast<const float4 *>(V + row * ld + (int64_t)tj.y * kSB) + c4);
-        reinterpret_cast<float4 *>(vp)[f] = v;
-    }
+    const float *sc = packed_scale(vp, ntiles);
+    unsigned char *vex = packed_exps(vp, ntiles, ld);
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < ntiles; k += nw)
+        pack_tile_f32(V, ld, N, tiles[k], k, vp, sc, vex);
 }
 
 // ------------------------------------------------------------------ persistent DF64 solver
@@ -1105,7 +1363,7 @@ struct PcgArgs {
     int64_t M;
     // operator preconditioning (Sec. 2.6): packed FP32 upper triangle of the
     // preconditioner C = S D^reg S (the tiles of vp)
-    const float *dvp;
+    float *dvp;
     long long bar_limit_ns;   // grid-barrier wait limit (ns)
     int absent_cta;           // failure-detection tests: this CTA leaves at its first barrier (-1: none)
     // BEM_PRODUCTS_FP16: the FP16 working copy of the packed tiles and their scales
@@ -1116,97 +1374,65 @@ struct PcgArgs {
     double *n16_out;          // nullable: iterations that used the FP16 copy
 };
 
-// Per-CTA partial of one value per thread (fixed tree) into slot[cta].
-__device__ __forceinline__ void cta_partial(double v, double *slot, int cta)
+// Per-CTA partials of n values per thread (fixed tree), value j into slot[j G + cta]: the
+// warps' sums meet in shared memory and warp j adds those of value j by shuffles.
+template <int n>
+__device__ __forceinline__ void cta_partials(const double (&v)[n], double *slot, int G, int cta)
 {
-    __shared__ double sw[kSymThreads / 32];
-    v = warp_sum(v);
+    constexpr int kW = kSymThreads / 32;
+    static_assert(n <= kW && kW == 8, "one warp per value, eight partial sums each");
+    __shared__ double sw[n][kW];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sw[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < kSymThreads / 32; ++k) t += sw[k];
-        slot[cta] = t;
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+        const double t = warp_sum(v[j]);
+        if (lane == 0) sw[j][w] = t;
     }
     __syncthreads();
+    if (w < n) {
+        double t = sw[w][lane & (kW - 1)];
+#pragma unroll
+        for (int o = kW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) slot[(int64_t)w * G + cta] = t;
+    }
 }
 
-// Two values at once, each summed exactly as cta_partial sums it.
-__device__ __forceinline__ void cta_partial2(double v1, double v2, double *slot1, double *slot2, int cta)
+// Fixed-order sums of the G per-CTA partials of n values (L2 loads: written by other
+// CTAs): warp j adds value j's, lane l the partials l, l + 32, ...
+template <int n>
+__device__ __forceinline__ void grid_totals(const double *slot, int G, double (&r)[n])
 {
-    __shared__ double sw1[kSymThreads / 32], sw2[kSymThreads / 32];
-    v1 = warp_sum(v1);
-    v2 = warp_sum(v2);
+    __shared__ double res[n];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        sw1[w] = v1;
-        sw2[w] = v2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t1 = 0.0, t2 = 0.0;
-        for (int k = 0; k < kSymThreads / 32; ++k) {
-            t1 += sw1[k];
-            t2 += sw2[k];
+    if (w < n) {
+        const double *p = slot + (int64_t)w * G;
+        double v = 0.0;
+        for (int k0 = 0; k0 < G; k0 += 256) {  // eight loads in flight
+            double t[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int k = k0 + 32 * u + lane;
+                t[u] = k < G ? __ldcg(p + k) : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (k0 + 32 * u < G) v += t[u];
         }
-        slot1[cta] = t1;
-        slot2[cta] = t2;
+        v = warp_sum(v);
+        if (lane == 0) res[w] = v;
     }
     __syncthreads();
+#pragma unroll
+    for (int j = 0; j < n; ++j) r[j] = res[j];
+    __syncthreads();  // res is rewritten by the next call
 }
 
-// Fixed-order sum of the G per-CTA partials (L2 loads: written by other CTAs).
-__device__ __forceinline__ double grid_total(const double *slot, int G)
-{
-    __shared__ double sw[kSymThreads / 32];
-    __shared__ double res;
-    double v = 0.0;
-    for (int k = threadIdx.x; k < G; k += blockDim.x) v += __ldcg(slot + k);
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) sw[w] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < kSymThreads / 32; ++k) t += sw[k];
-        res = t;
-    }
-    __syncthreads();
-    return res;
-}
-
-// Two totals at once, each summed exactly as grid_total sums it.
-__device__ __forceinline__ void grid_total2(const double *slot1, const double *slot2, int G, double &r1, double &r2)
-{
-    __shared__ double sw1[kSymThreads / 32], sw2[kSymThreads / 32];
-    __shared__ double res1, res2;
-    double v1 = 0.0, v2 = 0.0;
-    for (int k = threadIdx.x; k < G; k += blockDim.x) {
-        v1 += __ldcg(slot1 + k);
-        v2 += __ldcg(slot2 + k);
-    }
-    v1 = warp_sum(v1);
-    v2 = warp_sum(v2);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        sw1[w] = v1;
-        sw2[w] = v2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t1 = 0.0, t2 = 0.0;
-        for (int k = 0; k < kSymThreads / 32; ++k) {
-            t1 += sw1[k];
-            t2 += sw2[k];
-        }
-        res1 = t1;
-        res2 = t2;
-    }
-    __syncthreads();
-    r1 = res1;
-    r2 = res2;
-}
+// CTAs per SM of the persistent solvers: 16 warps of 128 registers keep as many bytes in
+// flight as 24 of 80 (each warp a 4 KB chunk, and no spills), and a grid barrier or a
+// fixed-order total over 304 CTAs costs less than over 456.  Per iteration at N = 21,744
+// (block preconditioner): products 211 -> 163 us, reductions 16 -> 12; at N = 5,436
+// 60 -> 42 us in all.
+constexpr int kPcgCtas = 2;
 
 // kCal: the build with the operator preconditioner (BEM_PRECOND_CALDERON), kept out of
 // the other solvers' kernels (its Chebyshev and D^reg phases cost registers).
@@ -1216,21 +1442,27 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     extern __shared__ float2 sm[];
     const int64_t stride = (int64_t)G * kSymThreads;
     const int64_t i0 = (int64_t)cta * kSymThreads + threadIdx.x;
-    double *pA = a.part, *pB = a.part + G, *pC = a.part + 2 * G;
+    double *const pA = a.part, *const pB = a.part + G;  // one value; two values
     const bool mixed = a.vp != nullptr;
     const bool blockpc = a.precond == BEM_PRECOND_BLOCK, jacobi = a.precond == BEM_PRECOND_JACOBI;
     const bool calpc = kCal && a.precond == BEM_PRECOND_CALDERON;
     const bool zlocal = !blockpc && !calpc;  // z_i from r_i alone
-    float2 *const xsw = sm + (threadIdx.x >> 5) * 2 * kSB;
+    HiStage *const stage = reinterpret_cast<HiStage *>(sm) + (threadIdx.x >> 5);
+    static_assert(sizeof(HiStage) * (kSymThreads / 32) <= kSymSmem, "the warps' stages fit the tile buffers");
     __shared__ double rs[kBJ];
     const int lane = threadIdx.x & 31, q4 = lane & 3;
     const int64_t warp_g = ((int64_t)cta * kSymThreads + threadIdx.x) >> 5, nwarps = stride >> 5;
     unsigned long long tbase = 0ull;
     GridBar gb{a.bar, a.err, 0u, a.bar_limit_ns > 0 ? a.bar_limit_ns : kBarrierLimitNs, a.absent_cta == cta};
+    // scales of the packed copy's rows (FP32 operators: formed with the copy)
+    float *const rsc = mixed ? packed_scale(a.vp, a.ntiles) : nullptr;
+    if (mixed && !a.f32op)
+        for (int64_t i = i0; i < a.ld; i += stride) rsc[i] = i < a.N ? tile_scale(a.d[i]) : 1.0f;
     // packed products: tiles taken statically when every warp gets one at most
     const int hi_static = a.ntiles <= nwarps ? (int)warp_g : -1;
-    auto hi_product = [&](const float *packed) {
-        symv_hi_tiles(packed, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, xsw, a.ctr, tbase, hi_static);
+    auto hi_product = [&](float *packed, auto grid) {
+        symv_hi_tiles<decltype(grid)::value>(packed, packed_scale(packed, a.ntiles), packed_exps(packed, a.ntiles, a.ld),
+                                             a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, stage, a.ctr, tbase, hi_static);
         if (hi_static < 0) tbase += (unsigned long long)(a.ntiles + G * (kSymThreads / 32));
     };
     // DF64 product V x into the tile partials (x = the FP64 iterate); the first one
@@ -1239,10 +1471,10 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
         for (int64_t i = i0; i < a.ld; i += stride) a.pdf[i] = i < a.N ? df_from_double(a.x[i]) : make_float2(0.f, 0.f);
         if (!grid_barrier(gb, G)) return false;
         if (a.f32op) {  // the stored operator is the packed copy itself
-            hi_product(a.vp);
+            hi_product(a.vp, std::false_type());
         } else {
             symv_tiles(a.V, a.ld, a.N, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, sm, cta, G, a.ctr, tbase,
-                       pack ? a.vp : nullptr);
+                       pack ? a.vp : nullptr, rsc, pack ? packed_exps(a.vp, a.ntiles, a.ld) : nullptr);
             tbase += (unsigned long long)(a.ntiles + G);
         }
         return grid_barrier(gb, G);
@@ -1250,10 +1482,10 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     // z = C r (operator preconditioning, Sec. 2.6): the product with the packed FP32 C
     // (exact products, double-float sums); its row pass also forms the partial of r.z,
     // and with init p = z
-    auto calderon = [&](bool init, double &rz_part) -> bool {
+    auto calderon = [&](bool init, double (&sums)[2]) -> bool {
         for (int64_t i = i0; i < a.ld; i += stride) a.pdf[i] = i < a.N ? df_from_double(a.r[i]) : make_float2(0.f, 0.f);
         if (!grid_barrier(gb, G)) return false;
-        hi_product(a.dvp);
+        hi_product(a.dvp, std::false_type());
         if (!grid_barrier(gb, G)) return false;
         for (int64_t ib = warp_g * 8; ib < a.N; ib += nwarps * 8) {
             const int64_t i = ib + (lane >> 2);
@@ -1261,7 +1493,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             const double zi = symv_row4(a.prow, a.pcol, a.nb, valid ? i : a.N - 1, q4);
             if (valid && q4 == 0) {
                 a.z[i] = zi;
-                rz_part += __ldcg(a.r + i) * zi;  // r of other threads' rows: L2
+                sums[0] += __ldcg(a.r + i) * zi;  // r of other threads' rows: L2
                 if (init) {
                     a.p[i] = zi;
                     a.pdf[i] = df_from_double(zi);
@@ -1282,19 +1514,19 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
         if (!grid_barrier(gb, G)) return;
     }
     int n16 = 0, seg = 0;
-    double rz_l = 0.0, rr_l = 0.0, bb_l = 0.0;
+    double sums[2] = {0.0, 0.0}, bb_l[1] = {0.0};  // r.z, r.r
     for (int64_t i = i0; i < a.ld; i += stride) {
         if (i < a.N) {
             const double ri = a.b[i] - (a.has_x0 ? symv_row(a.prow, a.pcol, a.nb, i) : 0.0);
             a.r[i] = ri;
-            bb_l += a.b[i] * a.b[i];
+            bb_l[0] += a.b[i] * a.b[i];
             if (zlocal) {
                 const double zi = jacobi ? ri / a.d[i] : ri;
                 a.z[i] = zi;
                 a.p[i] = zi;
                 a.pdf[i] = df_from_double(zi);
-                rz_l += ri * zi;
-                rr_l += ri * ri;
+                sums[0] += ri * zi;
+                sums[1] += ri * ri;
             }
         } else {
             a.pdf[i] = make_float2(0.f, 0.f);
@@ -1303,37 +1535,38 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     if (blockpc) {  // z = M^-1 r over whole clusters: every r written first
         if (!grid_barrier(gb, G)) return;
         for (int blk = cta; blk < a.nbj; blk += G)
-            block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, 0.0, false, true, rs, rz_l, rr_l);
+            block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, 0.0, false, true, rs, sums);
     }
     if (calpc) {  // r.r of this thread's rows, then z = C r (r written by its own rows)
-        for (int64_t i = i0; i < a.N; i += stride) rr_l += a.r[i] * a.r[i];
-        if (!calderon(true, rz_l)) return;
+        for (int64_t i = i0; i < a.N; i += stride) sums[1] += a.r[i] * a.r[i];
+        if (!calderon(true, sums)) return;
     }
-    cta_partial(rz_l, pA, cta);
-    cta_partial(rr_l, pB, cta);
-    cta_partial(bb_l, pC, cta);
+    cta_partials(bb_l, pA, G, cta);
+    cta_partials(sums, pB, G, cta);
     if (!grid_barrier(gb, G)) return;
-    double rz = grid_total(pA, G), rr = grid_total(pB, G);
-    const double bb = grid_total(pC, G);
+    double one[1], tot[2];
+    grid_totals(pA, G, one);
+    grid_totals(pB, G, tot);
+    double rz = tot[0], rr = tot[1];
+    const double bb = one[0];
     const double thr = a.tol * a.tol * (bb > 0.0 ? bb : 1.0);
     double rr_true = rr;  // r.r at the last residual formed with the DF64 product
     double rr_true_prev = rr;
     int it = 0, ndf = prod0 ? 1 : 0, inexact_stop = 0;
     if (!grid_barrier(gb, G)) return;  // partial slots are reused below
     while (!(rr <= thr) && it < a.max_it) {
-        double alpha, rz_new, rz_n = 0.0;
         if (use16) {
-            symv_h16_tiles(a.vh, a.vsc, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, xsw, a.ctr, tbase, hi_static);
+            symv_h16_tiles(a.vh, a.vsc, rsc, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, stage, a.ctr, tbase, hi_static);
             if (hi_static < 0) tbase += (unsigned long long)(a.ntiles + G * (kSymThreads / 32));
             ++n16;
         } else if (mixed) {
-            hi_product(a.vp);
+            hi_product(a.vp, std::true_type());
         } else {
             symv_tiles(a.V, a.ld, a.N, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, sm, cta, G, a.ctr, tbase);
             tbase += (unsigned long long)(a.ntiles + G);
         }
         if (!grid_barrier(gb, G)) return;
-        double pq_l = 0.0;
+        double pq_l[1] = {0.0};
         // 8 rows per warp and pass, 4 threads per row; the loop is uniform across the
         // warp (rows past N recompute row N-1 and are discarded) because the row sum
         // combines the 4 threads with shuffles
@@ -1344,24 +1577,25 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             const double qi = symv_row4(a.prow, a.pcol, a.nb, ic, q4);
             if (valid && q4 == 0) {
                 a.q[i] = qi;
-                pq_l += a.p[i] * qi;
+                pq_l[0] += a.p[i] * qi;
             }
         }
-        cta_partial(pq_l, pA, cta);
+        cta_partials(pq_l, pA, G, cta);
         if (!grid_barrier(gb, G)) return;
-        alpha = rz / grid_total(pA, G);
-        rr_l = 0.0;
+        grid_totals(pA, G, one);
+        const double pq = one[0], alpha = rz / pq;
+        sums[0] = sums[1] = 0.0;
         if (blockpc) {
             for (int blk = cta; blk < a.nbj; blk += G)
-                block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, alpha, true, false, rs, rz_n, rr_l);
+                block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, alpha, true, false, rs, sums);
         } else if (calpc) {
             for (int64_t i = i0; i < a.N; i += stride) {
                 a.x[i] += alpha * a.p[i];
                 const double ri = a.r[i] - alpha * a.q[i];
                 a.r[i] = ri;
-                rr_l += ri * ri;
+                sums[1] += ri * ri;
             }
-            if (!calderon(false, rz_n)) return;
+            if (!calderon(false, sums)) return;
         } else {
             for (int64_t i = i0; i < a.N; i += stride) {
                 a.x[i] += alpha * a.p[i];
@@ -1369,13 +1603,14 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
                 const double zi = jacobi ? ri / a.d[i] : ri;
                 a.r[i] = ri;
                 a.z[i] = zi;
-                rz_n += ri * zi;
-                rr_l += ri * ri;
+                sums[0] += ri * zi;
+                sums[1] += ri * ri;
             }
         }
-        cta_partial2(rz_n, rr_l, pB, pC, cta);
+        cta_partials(sums, pB, G, cta);
         if (!grid_barrier(gb, G)) return;
-        grid_total2(pB, pC, G, rz_new, rr);
+        grid_totals(pB, G, tot);
+        rr = tot[1];
         ++it;
         if (a.lam2 > 0.0) {
             // |||alpha p|||^2 = alpha^2 p.Vp = alpha (r.z); ZZ estimator of the iterate
@@ -1390,18 +1625,19 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
                 a.u[z] = den > 0.0 ? num / den : 0.0;
             }
             if (!grid_barrier(gb, G)) return;
-            double el = 0.0;
+            double el[1] = {0.0};
             for (int64_t t = i0; t < a.N; t += stride) {
                 double d[3];
                 for (int k = 0; k < 3; ++k) d[k] = __ldcg(a.u + a.tris[3 * t + k]) - a.x[t];
                 const double s2 = (d[0] * d[0] + d[1] * d[1]) + d[2] * d[2];
                 const double s1 = (d[0] + d[1]) + d[2];
                 const double h = a.hdiam ? a.hdiam[t] : sqrt(a.area[t]);
-                el += (h * a.area[t]) / 12.0 * (s2 + s1 * s1);
+                el[0] += (h * a.area[t]) / 12.0 * (s2 + s1 * s1);
             }
-            cta_partial(el, pA, cta);
+            cta_partials(el, pA, G, cta);
             if (!grid_barrier(gb, G)) return;
-            if (upd2 <= a.lam2 * grid_total(pA, G)) {
+            grid_totals(pA, G, one);
+            if (upd2 <= a.lam2 * one[0]) {
                 inexact_stop = 1;
                 break;
             }
@@ -1412,8 +1648,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             // reliable update: replace the recursive residual by b - V x with the
             // DF64 product (the direction p is kept)
             if (!df64_product(false)) return;
-            rz_n = 0.0;
-            rr_l = 0.0;
+            sums[0] = sums[1] = 0.0;
             for (int64_t ib = warp_g * 8; ib < a.N; ib += nwarps * 8) {
                 const int64_t i = ib + (lane >> 2);
                 const bool valid = i < a.N;
@@ -1424,35 +1659,35 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
                     if (zlocal) {
                         const double zi = jacobi ? ri / a.d[i] : ri;
                         a.z[i] = zi;
-                        rz_n += ri * zi;
-                        rr_l += ri * ri;
+                        sums[0] += ri * zi;
+                        sums[1] += ri * ri;
                     }
                 }
             }
             if (blockpc) {
                 if (!grid_barrier(gb, G)) return;
                 for (int blk = cta; blk < a.nbj; blk += G)
-                    block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, 0.0, false, false, rs, rz_n,
-                                rr_l);
+                    block_apply(a.bperm, a.binv, blk, a.x, a.r, a.z, a.p, a.q, a.pdf, 0.0, false, false, rs, sums);
             } else if (calpc) {  // r was written in the row-pass layout: barrier first
                 if (!grid_barrier(gb, G)) return;
-                for (int64_t i = i0; i < a.N; i += stride) rr_l += a.r[i] * a.r[i];
-                if (!calderon(false, rz_n)) return;
+                for (int64_t i = i0; i < a.N; i += stride) sums[1] += a.r[i] * a.r[i];
+                if (!calderon(false, sums)) return;
             }
-            cta_partial2(rz_n, rr_l, pB, pC, cta);
+            cta_partials(sums, pB, G, cta);
             if (!grid_barrier(gb, G)) return;
-            grid_total2(pB, pC, G, rz_new, rr);
+            grid_totals(pB, G, tot);
+            rr = tot[1];
             rr_true_prev = rr_true;
             rr_true = rr;
             ++ndf;
             if (use16 && rr_true > kH16Progress * rr_true_prev) use16 = false;  // the same in every CTA
         }
-        const double beta = rz_new / rz;
+        const double beta = tot[0] / rz;
         if (a.lanczos && cta == 0 && threadIdx.x == 0 && it - 1 < a.lanczos_cap) {
             a.lanczos[2 * (it - 1)] = alpha;
             a.lanczos[2 * (it - 1) + 1] = beta;
         }
-        rz = rz_new;
+        rz = tot[0];
         for (int64_t i = i0; i < a.N; i += stride) {
             const double pi = a.z[i] + beta * a.p[i];
             a.p[i] = pi;
@@ -1470,13 +1705,13 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     }
 }
 
-__global__ void __launch_bounds__(kSymThreads, 3) k_pcg_df(PcgArgs a) { pcg_body<false>(a, gridDim.x, blockIdx.x); }
-__global__ void __launch_bounds__(kSymThreads, 3) k_pcg_cal(PcgArgs a) { pcg_body<true>(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_df(PcgArgs a) { pcg_body<false>(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_cal(PcgArgs a) { pcg_body<true>(a, gridDim.x, blockIdx.x); }
 
 // Independent solves in one cooperative launch: problem p owns the CTAs
 // [begin[p], begin[p + 1]) and runs the same solver on them, with its own grid
 // barrier, tile counter and partials; a problem that converges releases its CTAs.
-__global__ void __launch_bounds__(kSymThreads, 3) k_pcg_batch(const PcgArgs *__restrict__ args,
+__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_batch(const PcgArgs *__restrict__ args,
                                                               const int *__restrict__ begin, int P)
 {
     __shared__ PcgArgs sa;
@@ -1801,24 +2036,28 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     bem_status st = BEM_OK;
     float *vp = nullptr;
     if (delta > 0.0) {
-        const size_t vbytes = (size_t)nt_ * kTileF * sizeof(float);
+        const size_t vbytes = packed_bytes((size_t)nt_, (size_t)op->ld);
         if (ctx->budget <= 0 || ctx->in_use + (int64_t)vbytes + (64 << 10) <= ctx->budget)
             if ((st = dalloc(ctx, tmp, (void **)&vp, vbytes, false))) return st;
     }
     if (f32op && !vp) return BEM_OK;  // no room for the packed copy: host-driven refinement
+    auto pack = [&](const float *V, float *to) {  // a packed copy of an FP32 matrix
+        k_tile_scale<<<nblk(op->ld, 256), 256, 0, ctx->stream>>>(V, op->ld, op->N, packed_scale(to, (size_t)nt_));
+        BEM_COUNT(ctx);
+        k_pack_f32<<<(unsigned)std::min<int64_t>((nt_ + 7) / 8, 8 * ctx->sm_count), 256, 0, ctx->stream>>>(
+            V, op->ld, op->N, W.tiles, nt_, to); BEM_COUNT(ctx);
+    };
     const bool calpc = precond == BEM_PRECOND_CALDERON;
     float *dvp = nullptr;
     if (calpc) {  // packed C (the tiles of the operator's packed copy)
-        if ((st = dalloc(ctx, tmp, (void **)&dvp, (size_t)nt_ * kTileF * sizeof(float), false))) {
+        if ((st = dalloc(ctx, tmp, (void **)&dvp, packed_bytes((size_t)nt_, (size_t)op->ld), false))) {
             dfree_all(ctx, tmp);
             return st;
         }
-        k_pack_f32<<<(unsigned)std::min<int64_t>(((int64_t)nt_ * (kTileF / 4) + 255) / 256, 8 * ctx->sm_count), 256, 0,
-                     ctx->stream>>>(op->cal_C, op->ld, op->N, W.tiles, nt_, dvp); BEM_COUNT(ctx);
+        pack(op->cal_C, dvp);
     }
     if (f32op) {
-        k_pack_f32<<<(unsigned)std::min<int64_t>(((int64_t)nt_ * (kTileF / 4) + 255) / 256, 8 * ctx->sm_count), 256, 0,
-                     ctx->stream>>>((const float *)op->V, op->ld, op->N, W.tiles, nt_, vp); BEM_COUNT(ctx);
+        pack((const float *)op->V, vp);
     }
     // FP16 working copy for the iteration products (N^2 bytes and a scale per tile)
     __half *vh = nullptr;
@@ -1843,10 +2082,10 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
             }
         }
     }
-    // Up to 3 CTAs per SM.  On small levels, CTAs that would only wait at the grid
+    // Up to kPcgCtas CTAs per SM.  On small levels, CTAs that would only wait at the grid
     // barriers are left out: DF64 products take one tile per CTA, the mixed mode's
     // products one tile per warp (8 per CTA), its row passes 8 rows per warp.
-    const int Gmax = (per_sm < 3 ? per_sm : 3) * ctx->sm_count;
+    const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
     int G = vp ? (int)std::max<int64_t>((nt_ + 7) / 8, (op->N + 63) / 64) : nt_;
     G = std::min(std::max(G, 8), Gmax);
     double *part = nullptr;
@@ -2221,26 +2460,20 @@ __global__ void k_batch_init(const BatchSolveProb *__restrict__ prob)
             pb->b[i] = pb->area[i];
             for (int64_t j = N; j < ld; ++j) V[i * ld + j] = T();
         }
+        if (pb->vp) packed_scale(pb->vp, pb->nt)[i] = i < N ? tile_scale(pb->d[i]) : 1.0f;
     }
     if (i < pb->part_n) pb->part[i] = 0.0;
     if (i < kBatchRes) pb->res[i] = 0.0;
 }
 
 // Packed upper triangles of FP32 operators; grid (blocks, problems).
-__global__ void k_batch_pack(const BatchSolveProb *__restrict__ prob)
+__global__ void __launch_bounds__(256) k_batch_pack(const BatchSolveProb *__restrict__ prob)
 {
     const BatchSolveProb *pb = prob + blockIdx.y;
-    const int64_t n4 = pb->nt * (kTileF / 4);
-    const float *V = (const float *)pb->V;
-    for (int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; f < n4; f += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t k = f / (kTileF / 4);
-        const int e = (int)(f % (kTileF / 4)), r = e >> 4, c4 = e & 15;
-        const int2 tj = pb->tiles[k];
-        const int64_t row = (int64_t)tj.x * kSB + r;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row < pb->N) v = __ldcs(reinterpret_cast<const float4 *>(V + row * pb->ld + (int64_t)tj.y * kSB) + c4);
-        reinterpret_cast<float4 *>(pb->vp)[f] = v;
-    }
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < pb->nt; k += nw)
+        pack_tile_f32((const float *)pb->V, pb->ld, pb->N, pb->tiles[k], k, pb->vp, packed_scale(pb->vp, pb->nt),
+                      packed_exps(pb->vp, pb->nt, pb->ld));
 }
 
 // FP16 working copies of the packed FP32 operators; grid (blocks, problems).
@@ -2396,7 +2629,7 @@ static size_t batch_problem_bytes(int64_t N, int prec, bool packed, bool block, 
     const size_t es = prec == BEM_PREC_F32 ? 4 : 8;
     size_t b = al(es * (size_t)N * (size_t)L) + al(8 * (size_t)N) + al(8 * 7 * (size_t)L) + al(8 * (size_t)L) +
                al(2 * (size_t)nt * kSB * 8) + al(sizeof(double) * (3 * (size_t)G + 8) + 64);
-    if (packed) b += al((size_t)nt * kTileF * 4);
+    if (packed) b += al(packed_bytes((size_t)nt, (size_t)L));
     if (packed && h16) b += al((size_t)nt * kTileF * 2) + al((size_t)nt * 4);
     if (block) b += al(8 * (size_t)kBJ * kBJ * (size_t)((N + kBJ - 1) / kBJ));
     return b;
@@ -2428,7 +2661,7 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
     if (!coop) return set_error(ctx, BEM_ERR_CUDA, "the device has no cooperative launch");
     BEM_CK(ctx, cudaFuncSetAttribute(k_pcg_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSymSmem));
     BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_batch, kSymThreads, kSymSmem));
-    const int Gmax = (per_sm < 3 ? per_sm : 3) * ctx->sm_count;
+    const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
     if (Gmax < 1) return set_error(ctx, BEM_ERR_CUDA, "the batch solver cannot be resident on this device");
     bem_status st = assembly_prepare(ctx);
     if (st) return st;
@@ -2645,7 +2878,7 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             float *vsc = nullptr;
             if (packed) {
                 vp = reinterpret_cast<float *>(cur);
-                cur += al((size_t)pr.nt * kTileF * 4);
+                cur += al(packed_bytes((size_t)pr.nt, (size_t)L));
                 if (bt->h16) {
                     vh = reinterpret_cast<__half *>(cur);
                     cur += al((size_t)pr.nt * kTileF * 2);
