@@ -201,25 +201,25 @@ __device__ __forceinline__ void far_f32_body(const float *__restrict__ q32, cons
     // FP32 only in the pair loop: centroids as hi + lo floats, so that the centroid
     // difference (hi_i - hi_j) + (lo_i - lo_j) keeps FP32 relative accuracy for
     // distant pairs; weights and areas rounded to FP32 once
-    __shared__ float so[R][3 * kQ];
-    __shared__ float sc[R][7];  // centroid hi (3), lo (3), area
+    __shared__ float4 so[R][kQ32Stride / 4];  // offsets (21 of 24 floats)
+    __shared__ float4 sc[R][2];               // centroid hi (3) and area, lo (3)
+    static_assert(kQ32Stride % 4 == 0 && kQ32Stride >= 3 * kQ, "rows of whole float4");
     if (i0 > cbase + C - 1 || i0 >= r1) return;
-    for (int k = threadIdx.x; k < R * 3 * kQ; k += C) {
-        const int r = k / (3 * kQ), c = k % (3 * kQ);
-        const int64_t i = i0 + r;
-        so[r][c] = (i < r1) ? q32[i * kQ32Stride + c] : 0.0f;
+    for (int k = threadIdx.x; k < R * (kQ32Stride / 4); k += C) {
+        const int r = k / (kQ32Stride / 4), c = k % (kQ32Stride / 4);
+        const int64_t i = i0 + r < r1 ? i0 + r : r1 - 1;
+        so[r][c] = reinterpret_cast<const float4 *>(q32 + i * kQ32Stride)[c];
     }
-    for (int k = threadIdx.x; k < R * 4; k += C) {
-        const int r = k / 4, c = k % 4;
-        const int64_t i = i0 + r;
-        const double v = (i < r1) ? cent[i * 4 + c] : 0.0;
-        const float h = (float)v;
-        if (c < 3) {
-            sc[r][c] = h;
-            sc[r][3 + c] = (float)(v - (double)h);
-        } else {
-            sc[r][6] = h;
+    for (int r = threadIdx.x; r < R; r += C) {
+        const int64_t i = i0 + r < r1 ? i0 + r : r1 - 1;
+        float h[4], l[3];
+        for (int c = 0; c < 4; ++c) {
+            const double v = cent[i * 4 + c];
+            h[c] = (float)v;
+            if (c < 3) l[c] = (float)(v - (double)h[c]);
         }
+        sc[r][0] = make_float4(h[0], h[1], h[2], h[3]);
+        sc[r][1] = make_float4(l[0], l[1], l[2], 0.0f);
     }
     __syncthreads();
     const int64_t j = cbase + threadIdx.x;
@@ -245,22 +245,49 @@ __device__ __forceinline__ void far_f32_body(const float *__restrict__ q32, cons
     for (int r = 0; r < rows; ++r) {
         const int64_t i = i0 + r;
         if (i > j) break;
-        const float Dx = (sc[r][0] - ch[0]) + (sc[r][3] - cl[0]);
-        const float Dy = (sc[r][1] - ch[1]) + (sc[r][4] - cl[1]);
-        const float Dz = (sc[r][2] - ch[2]) + (sc[r][5] - cl[2]);
-        float acc = 0.0f;
+        const float4 h4 = sc[r][0], l4 = sc[r][1];
+        const float Dx = (h4.x - ch[0]) + (l4.x - cl[0]);
+        const float Dy = (h4.y - ch[1]) + (l4.y - cl[1]);
+        const float Dz = (h4.z - ch[2]) + (l4.z - cl[2]);
+        float o[kQ32Stride];
 #pragma unroll
-        for (int a = 0; a < kQ; ++a) {
-            const float xa = Dx + so[r][3 * a], ya = Dy + so[r][3 * a + 1], za = Dz + so[r][3 * a + 2];
-            float s = 0.0f;
-#pragma unroll
-            for (int b = 0; b < kQ; ++b) {
-                const float dx = xa - y[3 * b], dy = ya - y[3 * b + 1], dz = za - y[3 * b + 2];
-                s += wf[b] * rsqrtf(dx * dx + dy * dy + dz * dz);
-            }
-            acc += wf[a] * s;
+        for (int k = 0; k < kQ32Stride / 4; ++k) {
+            const float4 v = so[r][k];
+            o[4 * k] = v.x;
+            o[4 * k + 1] = v.y;
+            o[4 * k + 2] = v.z;
+            o[4 * k + 3] = v.w;
         }
-        V[i * ld + j] = sc[r][6] * Aj * acc;
+        // The bare MUFU estimate gives rsqrtf's bits for normal arguments without the
+        // scaling of subnormal ones (about 4 of 11 instructions per point pair); a
+        // subnormal |d|^2 is infinity there, and the sum is then taken again with rsqrtf.
+        // Bound by issue, then by MUFU (49 per entry, 16 lanes per SM and cycle: 103
+        // Gpairs/s): N = 2,416 69.9 -> 55.2 us, N = 21,744 4.08 -> 3.31 ms (58.0 -> 71.4
+        // Gpairs/s), the same bits.
+        auto sum = [&](auto bare) {
+            float acc = 0.0f;
+#pragma unroll
+            for (int a = 0; a < kQ; ++a) {
+                const float xa = Dx + o[3 * a], ya = Dy + o[3 * a + 1], za = Dz + o[3 * a + 2];
+                float s = 0.0f;
+#pragma unroll
+                for (int b = 0; b < kQ; ++b) {
+                    const float dx = xa - y[3 * b], dy = ya - y[3 * b + 1], dz = za - y[3 * b + 2];
+                    const float d2 = dx * dx + dy * dy + dz * dz;
+                    float q;
+                    if (decltype(bare)::value)
+                        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(d2));
+                    else
+                        q = rsqrtf(d2);
+                    s += wf[b] * q;
+                }
+                acc += wf[a] * s;
+            }
+            return acc;
+        };
+        float acc = sum(std::true_type());
+        if (!(acc < INFINITY) && i != j) acc = sum(std::false_type());  // (i, i) is the near field's
+        V[i * ld + j] = h4.w * Aj * acc;
     }
 }
 
