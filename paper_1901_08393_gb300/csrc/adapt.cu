@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "bem_internal.cuh"
+#include "dfloat.cuh"
 
 namespace bem {
 
@@ -1031,10 +1032,267 @@ static bem_status cheb_cols(bem_ctx *ctx, bem_mesh *pm, const float *dinv, int64
     return BEM_OK;
 }
 
+// ---- V^dual and D^reg in four passes
+// Gathering the 144 children pairs of every pair of vertices and the 36 of every pair of
+// triangles straight from V^bary took two scattered passes over it (2.6 ms each at N =
+// 3,674, 8x the time of its bytes) and a third of FP64 work repeated per vertex pair.  Now
+// one streaming pass over the upper half of V^bary contracts it per pair of triangles,
+//   U[(T, k)][(T', l)] = sum over the two children of T at its vertex k and of T' at l
+//   V^T[T][T'] = sum_kl U,
+// both with their mirror images; then rows are summed over the star of each vertex
+// (coalesced), and the rows' entries over the stars of the others:
+//   Z[z] = sum_{T at z} U[(T, k(z))],   V^dual[z][w] = sum_{T' at w} Z[z][(T', l(w))]
+//   R[i][T'] = sum_{T at i} curl phi_i|T V^T[T][T'],  D[i][j] = sum_{T' at j} curl phi_j|T' . R[i][T'].
+// Scratch: 92 N^2 bytes (V^bary has 288 N^2).  DF64 sums in double-float (2^-47; FP64 sums
+// ran at 1/64 of that rate).
+
+// Sums of contracted elements: double (F64) or hi/lo pairs.
+__device__ __forceinline__ double u_add(double a, double b) { return a + b; }
+__device__ __forceinline__ float2 u_add(float2 a, float2 b) { return df_add(a, b); }
+__device__ __forceinline__ double u_double(double a) { return a; }
+__device__ __forceinline__ double u_double(float2 a) { return df_to_double(a); }
+template <typename T> struct ContractElem { using type = float2; };
+template <> struct ContractElem<double> { using type = double; };
+
+__device__ __forceinline__ void vb_row6(const float2 *p, float2 (&v)[6])
+{
+    const float4 *q = reinterpret_cast<const float4 *>(p);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const float4 f = __ldg(q + u);
+        v[2 * u] = make_float2(f.x, f.y);
+        v[2 * u + 1] = make_float2(f.z, f.w);
+    }
+}
+__device__ __forceinline__ void vb_row6(const double *p, double (&v)[6])
+{
+    const double2 *q = reinterpret_cast<const double2 *>(p);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const double2 f = __ldg(q + u);
+        v[2 * u] = f.x;
+        v[2 * u + 1] = f.y;
+    }
+}
+__device__ __forceinline__ void vb_row6(const float *p, float2 (&v)[6])
+{
+    const float2 *q = reinterpret_cast<const float2 *>(p);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const float2 f = __ldg(q + u);
+        v[2 * u] = make_float2(f.x, 0.0f);
+        v[2 * u + 1] = make_float2(f.y, 0.0f);
+    }
+}
+__device__ __forceinline__ float2 vb_one(const float2 *p) { return *p; }
+__device__ __forceinline__ double vb_one(const double *p) { return *p; }
+__device__ __forceinline__ float2 vb_one(const float *p) { return make_float2(*p, 0.0f); }
+
+// Tile of 8 triangles T (one per warp) x 32 triangles T' (one per lane), pairs T <= T' only:
+// 18 loads of 16 bytes per thread; the results go through shared memory so that rows and
+// mirrored rows are written in whole segments.  Children 0, 5 belong to vertex 0, 1, 2 to
+// vertex 1, 3, 4 to vertex 2.
+template <typename T, typename E>
+__global__ void __launch_bounds__(256) k_contract(const T *__restrict__ Vb, int64_t ldb, int64_t N, E *__restrict__ U,
+                                                  double *__restrict__ VT)
+{
+    const int64_t t0 = 8 * (int64_t)blockIdx.y, s0 = 32 * (int64_t)blockIdx.x;
+    if (s0 + 31 < t0) return;
+    __shared__ E us[24][97];
+    __shared__ double vs[8][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t t = t0 + w, t2 = s0 + lane;
+    if (t < N && t2 < N && t <= t2) {
+        E c[6][3];  // the row's children by columns
+        if (t < t2) {
+#pragma unroll
+            for (int a = 0; a < 6; ++a) {
+                E v[6];
+                vb_row6(Vb + (6 * t + a) * ldb + 6 * t2, v);
+                c[a][0] = u_add(v[0], v[5]);
+                c[a][1] = u_add(v[1], v[2]);
+                c[a][2] = u_add(v[3], v[4]);
+            }
+        } else {  // entries below the diagonal from above it
+#pragma unroll
+            for (int a = 0; a < 6; ++a) {
+                E v[6];
+#pragma unroll
+                for (int b = 0; b < 6; ++b) {
+                    const int lo = a < b ? a : b, hi = a < b ? b : a;
+                    v[b] = vb_one(Vb + (6 * t + lo) * ldb + 6 * t + hi);
+                }
+                c[a][0] = u_add(v[0], v[5]);
+                c[a][1] = u_add(v[1], v[2]);
+                c[a][2] = u_add(v[3], v[4]);
+            }
+        }
+        E tot;
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+            const E u0 = u_add(c[0][l], c[5][l]), u1 = u_add(c[1][l], c[2][l]), u2 = u_add(c[3][l], c[4][l]);
+            us[3 * w][3 * lane + l] = u0;
+            us[3 * w + 1][3 * lane + l] = u1;
+            us[3 * w + 2][3 * lane + l] = u2;
+            const E r = u_add(u_add(u0, u1), u2);
+            tot = l ? u_add(tot, r) : r;
+        }
+        vs[w][lane] = u_double(tot);
+    }
+    __syncthreads();
+    const int64_t L = 3 * N;
+    for (int e = threadIdx.x; e < 24 * 96; e += 256) {  // rows (T, k)
+        const int r = e / 96, q = e % 96;
+        const int64_t a = t0 + r / 3, b = s0 + q / 3;
+        if (a < N && b < N && a <= b) U[(3 * t0 + r) * L + 3 * s0 + q] = us[r][q];
+    }
+    for (int e = threadIdx.x; e < 24 * 96; e += 256) {  // rows (T', l)
+        const int q = e / 24, r = e % 24;
+        const int64_t a = t0 + r / 3, b = s0 + q / 3;
+        if (a < N && b < N && a < b) U[(3 * s0 + q) * L + 3 * t0 + r] = us[r][q];
+    }
+    if (t < N && t2 < N && t <= t2) VT[t * N + t2] = vs[w][lane];
+    {
+        const int64_t a = t0 + (threadIdx.x & 7), b = s0 + (threadIdx.x >> 3);
+        if (a < N && b < N && a < b) VT[b * N + a] = vs[threadIdx.x & 7][threadIdx.x >> 3];
+    }
+}
+
+// Per incidence p (triangle v2t[p] at vertex z): its row 3 T + k of U and the surface curl
+// of the hat of z on it.
+__global__ void k_star_table(const double *V, const int32_t *tris, const double *area, const int32_t *v2t_off,
+                             const int32_t *v2t, int64_t M, int32_t *row, double *curl, int *bad)
+{
+    const int64_t z = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (z >= M) return;
+    const int32_t b = v2t_off[z], e = v2t_off[z + 1];
+    if (e - b > kMaxStar) atomicExch(bad, 1);
+    for (int32_t p = b; p < e; ++p) {
+        const int32_t t = v2t[p];
+        const int k = tris[3 * (int64_t)t] == z ? 0 : (tris[3 * (int64_t)t + 1] == z ? 1 : 2);
+        row[p] = 3 * t + k;
+        double g[3];
+        hat_curl(V, tris, area, t, z, g);
+        for (int c = 0; c < 3; ++c) curl[3 * (int64_t)p + c] = g[c];
+    }
+}
+
+// Z[z] = sum of the star's rows of U; grid (columns, vertices).
+template <typename E>
+__global__ void __launch_bounds__(256) k_star_rows(const E *__restrict__ U, const int32_t *__restrict__ row,
+                                                   const int32_t *__restrict__ v2t_off, int64_t L, E *__restrict__ Z)
+{
+    const int64_t z = blockIdx.y, c = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (c >= L) return;
+    const int32_t b = v2t_off[z], e = v2t_off[z + 1];
+    E s = E();
+    for (int32_t p = b; p < e; p += 4) {  // four loads in flight
+        E v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (p + u < e) v[u] = U[(int64_t)row[p + u] * L + c];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (p + u < e) s = u_add(s, v[u]);
+    }
+    Z[z * L + c] = s;
+}
+
+// V^dual[z][w], w >= z, mirrored.
+template <typename E, typename O>
+__global__ void __launch_bounds__(128) k_dual_gather(const E *__restrict__ Z, const int32_t *__restrict__ row,
+                                                     const int32_t *__restrict__ v2t_off, int64_t L, int64_t M, O *Vd,
+                                                     int64_t ldd)
+{
+    const int64_t z = blockIdx.y, w = z + (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (w >= M) return;
+    E s = E();
+    for (int32_t q = v2t_off[w]; q < v2t_off[w + 1]; ++q) s = u_add(s, Z[z * L + row[q]]);
+    Vd[z * ldd + w] = s;
+    Vd[w * ldd + z] = s;
+}
+
+// R[i][T'] (three components); grid (columns, vertices).
+__global__ void __launch_bounds__(128) k_star_field(const double *__restrict__ VT, const double *__restrict__ curl,
+                                                    const int32_t *__restrict__ v2t_off,
+                                                    const int32_t *__restrict__ v2t, int64_t N, double *__restrict__ R)
+{
+    const int64_t i = blockIdx.y, t = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (t >= N) return;
+    double a[3] = {0.0, 0.0, 0.0};
+    for (int32_t p = v2t_off[i]; p < v2t_off[i + 1]; ++p) {
+        const double v = __ldg(VT + (int64_t)v2t[p] * N + t);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[c] = fma(__ldg(curl + 3 * (int64_t)p + c), v, a[c]);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) R[(i * N + t) * 3 + c] = a[c];
+}
+
+// D^reg[i][j], j >= i, mirrored, stored FP32.
+__global__ void __launch_bounds__(128) k_hyper_gather(const double *__restrict__ R, const double *__restrict__ curl,
+                                                      const int32_t *__restrict__ v2t_off,
+                                                      const int32_t *__restrict__ v2t, int64_t N, const double *a_int,
+                                                      int64_t M, float *Dm, int64_t ldd)
+{
+    const int64_t i = blockIdx.y, j = i + (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (j >= M) return;
+    double acc = 0.0;
+    for (int32_t q = v2t_off[j]; q < v2t_off[j + 1]; ++q) {
+        const double *r = R + (i * N + v2t[q]) * 3;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) acc = fma(__ldg(curl + 3 * (int64_t)q + c), __ldg(r + c), acc);
+    }
+    const float v = __double2float_rn(acc + a_int[i] * a_int[j]);
+    Dm[i * ldd + j] = v;
+    Dm[j * ldd + i] = v;
+}
+
+// V^dual into op->V and D^reg into op->cal_D from the operator of the barycentric
+// refinement (its upper triangle).  *done false: no room for the scratch.
+template <typename T>
+static bem_status dual_contract(const bem_operator *ob, bem_mesh *pm, bem_operator *op, int *bad, bool *done)
+{
+    using E = typename ContractElem<T>::type;
+    bem_ctx *ctx = pm->ctx;
+    cudaStream_t s = ctx->stream;
+    const int64_t N = pm->N, M = pm->M, L = 3 * N;
+    *done = false;
+    const size_t ub = sizeof(E) * (size_t)L * (size_t)L, zb = sizeof(E) * (size_t)L * (size_t)M,
+                 vb = sizeof(double) * (size_t)N * (size_t)N, rb = 3 * sizeof(double) * (size_t)N * (size_t)M,
+                 tb = (size_t)L * (3 * sizeof(double) + sizeof(int32_t));
+    Allocs tu, tr;
+    E *U = nullptr, *Z = nullptr;
+    double *VT = nullptr, *R = nullptr, *curl = nullptr;
+    if (ctx->budget > 0 && ctx->in_use + (int64_t)(ub + zb + vb + rb + tb) + (1 << 20) > ctx->budget) return BEM_OK;
+    if (dalloc(ctx, tu, (void **)&U, ub, false) || dalloc(ctx, tu, (void **)&Z, zb, false) ||
+        dalloc(ctx, tr, (void **)&VT, vb, false) || dalloc(ctx, tr, (void **)&R, rb, false) ||
+        dalloc(ctx, tr, (void **)&curl, tb, false)) {
+        dfree_all(ctx, tu);
+        dfree_all(ctx, tr);
+        ctx->err[0] = 0;
+        return BEM_OK;
+    }
+    int32_t *row = reinterpret_cast<int32_t *>(curl + 3 * L);
+    *done = true;
+    k_star_table<<<nblk(M, 128), 128, 0, s>>>(pm->verts, pm->tris, pm->area, pm->v2t_off, pm->v2t, M, row, curl, bad); BEM_COUNT(ctx);
+    k_contract<T, E><<<dim3(nblk(N, 32), nblk(N, 8)), 256, 0, s>>>((const T *)ob->V, ob->ld, N, U, VT); BEM_COUNT(ctx);
+    k_star_rows<E><<<dim3(nblk(L, 256), (unsigned)M), 256, 0, s>>>(U, row, pm->v2t_off, L, Z); BEM_COUNT(ctx);
+    k_dual_gather<E, E><<<dim3(nblk(M, 128), (unsigned)M), 128, 0, s>>>(Z, row, pm->v2t_off, L, M, (E *)op->V, op->ld); BEM_COUNT(ctx);
+    dfree_all(ctx, tu);  // stream-ordered
+    k_star_field<<<dim3(nblk(N, 128), (unsigned)M), 128, 0, s>>>(VT, curl, pm->v2t_off, pm->v2t, N, R); BEM_COUNT(ctx);
+    k_hyper_gather<<<dim3(nblk(M, 128), (unsigned)M), 128, 0, s>>>(R, curl, pm->v2t_off, pm->v2t, N, op->mesh->area, M,
+                                                                  op->cal_D, op->ld); BEM_COUNT(ctx);
+    const cudaError_t e = cudaGetLastError();
+    dfree_all(ctx, tr);
+    return e == cudaSuccess ? BEM_OK : cuda_error(ctx, e, "dual contraction");
+}
+
 // The operator preconditioner of Sec. 2.6 for CG on V^dual: D^reg (FP32, from V^bary),
 // then C = S D^reg S with S the Chebyshev approximation of M^-1 (W = S D^reg by
 // columns, C = S W^T, which equals S D^reg S since it is symmetric), stored FP32.
-static bem_status calderon_setup(bem_operator *ob, bem_mesh *pm, bem_operator *op, int *bad)
+// with_D: also D^reg, by the gathers (no room for the scratch of dual_contract).
+static bem_status calderon_setup(bem_operator *ob, bem_mesh *pm, bem_operator *op, int *bad, bool with_D)
 {
     bem_ctx *ctx = pm->ctx;
     cudaStream_t s = ctx->stream;
@@ -1042,24 +1300,22 @@ static bem_status calderon_setup(bem_operator *ob, bem_mesh *pm, bem_operator *o
     Allocs tmp;
     double *VT = nullptr;
     float *W = nullptr, *work = nullptr, *dinv = nullptr;
-    bem_status st = dalloc(ctx, op->allocs, (void **)&op->cal_D, sizeof(float) * (size_t)M * (size_t)ld, true);
-    if (!st) st = dalloc(ctx, op->allocs, (void **)&op->cal_C, sizeof(float) * (size_t)M * (size_t)ld, true);
-    if (!st) st = dalloc(ctx, tmp, (void **)&VT, sizeof(double) * (size_t)N * (size_t)N, false);
-    if (st) {
-        dfree_all(ctx, tmp);
-        return st;
+    bem_status st = BEM_OK;
+    if (with_D) {
+        st = dalloc(ctx, tmp, (void **)&VT, sizeof(double) * (size_t)N * (size_t)N, false);
+        if (st) return st;
+        const dim3 gc((unsigned)nblk(N, 128), (unsigned)std::min<int64_t>(N, 65535));
+        if (ob->precision == BEM_PREC_F64)
+            { k_contract_children<double><<<gc, 128, 0, s>>>((const double *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
+        else if (ob->precision == BEM_PREC_DF64)
+            { k_contract_children<float2><<<gc, 128, 0, s>>>((const float2 *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
+        else
+            { k_contract_children<float><<<gc, 128, 0, s>>>((const float *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
+        const dim3 gh((unsigned)nblk(M, 128), (unsigned)std::min<int64_t>(M, 65535));
+        k_hypersingular<<<gh, 128, 0, s>>>(pm->verts, pm->tris, pm->v2t_off, pm->v2t, pm->area, VT, N,
+                                           op->mesh->area, M, op->cal_D, ld, bad); BEM_COUNT(ctx);
+        dfree_all(ctx, tmp);  // stream-ordered: V^T is freed after the kernel that reads it
     }
-    const dim3 gc((unsigned)nblk(N, 128), (unsigned)std::min<int64_t>(N, 65535));
-    if (ob->precision == BEM_PREC_F64)
-        { k_contract_children<double><<<gc, 128, 0, s>>>((const double *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
-    else if (ob->precision == BEM_PREC_DF64)
-        { k_contract_children<float2><<<gc, 128, 0, s>>>((const float2 *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
-    else
-        { k_contract_children<float><<<gc, 128, 0, s>>>((const float *)ob->V, ob->ld, N, VT); BEM_COUNT(ctx); }
-    const dim3 gh((unsigned)nblk(M, 128), (unsigned)std::min<int64_t>(M, 65535));
-    k_hypersingular<<<gh, 128, 0, s>>>(pm->verts, pm->tris, pm->v2t_off, pm->v2t, pm->area, VT, N,
-                                       op->mesh->area, M, op->cal_D, ld, bad); BEM_COUNT(ctx);
-    dfree_all(ctx, tmp);  // stream-ordered: V^T is freed after the kernel that reads it
     // C = S D^reg S: W = S D^reg, then S W^T (all buffers zeroed: padding columns stay 0)
     st = dalloc(ctx, tmp, (void **)&W, sizeof(float) * ((size_t)M * (size_t)ld * 5 + (size_t)M), true);
     if (st) return st;
@@ -1115,9 +1371,19 @@ bem_status dual_operator(bem_operator *ob, bem_mesh *pm, bem_operator **out)
     if (!st) st = dalloc(ctx, tmp, (void **)&bad, sizeof(int), true);
     if (!st) {
         k_dual_cells<<<nblk(M, 256), 256, 0, s>>>(pm->verts, pm->v2t_off, pm->v2t, pm->area, M, cm->area, cm->cent); BEM_COUNT(ctx);
-        const dim3 grid((unsigned)nblk(M, 128), (unsigned)M);
         if (M > 65535) st = set_error(ctx, BEM_ERR_INVALID, "dual operator: more than 65535 vertices");
-        else if (ob->precision == BEM_PREC_F64)
+    }
+    if (!st) st = dalloc(ctx, op->allocs, (void **)&op->cal_D, sizeof(float) * (size_t)M * (size_t)op->ld, true);
+    if (!st) st = dalloc(ctx, op->allocs, (void **)&op->cal_C, sizeof(float) * (size_t)M * (size_t)op->ld, true);
+    bool contracted = false;
+    if (!st)
+        st = ob->precision == BEM_PREC_F64    ? dual_contract<double>(ob, pm, op, bad, &contracted)
+             : ob->precision == BEM_PREC_DF64 ? dual_contract<float2>(ob, pm, op, bad, &contracted)
+                                              : dual_contract<float>(ob, pm, op, bad, &contracted);
+    if (!st && !contracted) st = ensure_full(ob);
+    if (!st && !contracted) {
+        const dim3 grid((unsigned)nblk(M, 128), (unsigned)M);
+        if (ob->precision == BEM_PREC_F64)
             { k_dual_operator<double, double><<<grid, 128, 0, s>>>((const double *)ob->V, ob->ld, pm->tris, pm->v2t_off, pm->v2t, M, (double *)op->V, op->ld, bad); BEM_COUNT(ctx); }
         else if (ob->precision == BEM_PREC_DF64)
             { k_dual_operator<float2, float2><<<grid, 128, 0, s>>>((const float2 *)ob->V, ob->ld, pm->tris, pm->v2t_off, pm->v2t, M, (float2 *)op->V, op->ld, bad); BEM_COUNT(ctx); }
@@ -1125,7 +1391,7 @@ bem_status dual_operator(bem_operator *ob, bem_mesh *pm, bem_operator **out)
             { k_dual_operator<float, float2><<<grid, 128, 0, s>>>((const float *)ob->V, ob->ld, pm->tris, pm->v2t_off, pm->v2t, M, (float2 *)op->V, op->ld, bad); BEM_COUNT(ctx); }
     }
     if (!st) st = operator_diag(op);
-    if (!st) st = calderon_setup(ob, pm, op, bad);
+    if (!st) st = calderon_setup(ob, pm, op, bad, !contracted);
     if (!st) {
         cudaError_t e = cudaMemcpyAsync(ctx->h_pinned, bad, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -916,10 +916,11 @@ struct BaryLevel {
 };
 
 // Operator of one level of the dual-basis loop: barycentric refinement, its operator,
-// V^dual.  With incremental, the children of the kept primal triangles (the first 6K
-// barycentric triangles, geometry and adjacency unchanged under conforming NVB) take
-// their entries from the previous level's barycentric operator (bem_assemble_V_update);
-// the refinement and its operator are then kept for the next level.
+// V^dual.  The barycentric operator keeps its upper triangle only.  With incremental, the
+// children of the kept primal triangles (the first 6K barycentric triangles, geometry and
+// adjacency unchanged under conforming NVB) take their entries from the previous level's
+// barycentric operator (bem_assemble_V_update); the refinement and its operator are then
+// kept for the next level.
 static bem_status dual_level_operator(bem_mesh *cur, const bem_assembly_opts *aopts, bool incremental,
                                       BaryLevel &prev, bem_operator **out)
 {
@@ -935,10 +936,10 @@ static bem_status dual_level_operator(bem_mesh *cur, const bem_assembly_opts *ao
             BEM_COUNT(ctx);
             b->n_kept = 6 * cur->n_kept;
             b->src_N = prev.op->N;
-            st = bem_assemble_V_update(b, prev.op, aopts, &ob);
+            st = assemble_impl(b, aopts, prev.op, false, &ob, true);
         }
     } else if (!st) {
-        st = bem_assemble_V(b, aopts, &ob);
+        st = assemble_impl(b, aopts, nullptr, false, &ob, true);
     }
     prev.release();
     if (!st) st = dual_operator(ob, cur, out);
