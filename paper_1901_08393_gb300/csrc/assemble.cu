@@ -20,7 +20,9 @@
 //              take them.  1/|r| by the MUFU reciprocal square root and one step in
 //              double-float.  Entries within 3e-13 of FP64 (r.m.s. 3e-14).  V stored
 //              as hi/lo pairs.
-//      F64  -- native FP64 (GB300 issues FP64 at 1/64 of the FP32 rate).
+//      F64  -- native FP64 (GB300 issues FP64 at 1/64 of the FP32 rate): 7 FP64
+//              operations per point pair, the reciprocal root's estimate and its
+//              quadratic correction on the FP32 pipe.
 //      F32  -- centroid difference from hi + lo float centroids, offsets in FP32, MUFU rsqrt;
 //              no FP64 operation per pair (GB300 issues FP64 at 1/64 of the FP32 rate).
 //  * Near field (common vertex, common edge, identical): Sauter-Schwab
@@ -147,50 +149,188 @@ constexpr FarTileS kFarTiles[kFarTileVariants] = {
 // The far-field bodies take the tile origin (first row i0, first column cbase) as
 // arguments: the per-operator kernels derive it from the block index, the batched
 // kernel (several operators in one launch) from its work list.
-template <int R, int C>
-__device__ __forceinline__ void far_f64_body(const double *__restrict__ q64, double *__restrict__ V, int64_t ld,
-                                             int64_t r1, int64_t c1, int64_t i0, int64_t cbase)
+// v rounded to the nearest multiple of q = 2^(e-23), for |v| < 2^(e-1) and big =
+// 1.5 * 2^e: v + big lies in [2^e, 2^(e+1)], whose spacing is q, and the subtraction
+// of big is exact (Sterbenz).
+__device__ __forceinline__ float grid_snap(float v, float big) { return __fsub_rn(__fadd_rn(v, big), big); }
+
+// 1.5 * 2^(k + up) for a normal v in [2^k, 2^(k+1))
+__device__ __forceinline__ float grid_big(float v, unsigned up)
 {
-    __shared__ double sx[R][22];
+    return __uint_as_float(((__float_as_uint(v) & 0x7f800000u) + (up << 23)) | 0x400000u);
+}
+
+constexpr double kSqrt15 = 3.87298334620741688518;
+constexpr double kW0 = 9.0 / 40.0, kW1 = (155.0 - kSqrt15) / 1200.0, kW2 = (155.0 + kSqrt15) / 1200.0;
+constexpr float kFarSpread2 = 2.2505f;  // 1.5^2, rounded up past the FP32 errors of the test
+
+// FP64 <-> FP32 by integer operations, for magnitudes in the normal FP32 range (a
+// conversion costs as much as an FP64 operation): a positive v truncated.
+__device__ __forceinline__ float f64_to_f32_trunc(double v)
+{
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), (unsigned)__double2hiint(v) - (896u << 20), 3));
+}
+// |v| truncated, at least 2^-127
+__device__ __forceinline__ float f64_to_f32_abs(double v)
+{
+    const unsigned h = max((unsigned)__double2hiint(v) & 0x7fffffffu, 896u << 20) - (896u << 20);
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), h, 3));
+}
+// -2 v for a normal v (a zero becomes -+2^-1022)
+__device__ __forceinline__ double f64_m2(double v)
+{
+    return __hiloint2double((int)(((unsigned)__double2hiint(v) ^ 0x80000000u) + (1u << 20)), __double2loint(v));
+}
+// a positive v exactly (zero: 2^-127)
+__device__ __forceinline__ double f32_to_f64_pos(float v)
+{
+    const unsigned b = __float_as_uint(v);
+    return __hiloint2double((int)((b >> 3) + (896u << 20)), (int)(b << 29));
+}
+
+// Entry (i, j) of a close pair (see far_f64_body): every difference in FP64.
+__device__ __noinline__ double far_f64_close(const double *__restrict__ qi, const double *__restrict__ qj)
+{
+    double acc = 0.0;
+#pragma unroll 1
+    for (int a = 0; a < kQ; ++a) {
+        const double xa = qi[3 * a], ya = qi[3 * a + 1], za = qi[3 * a + 2];
+        double s = 0.0;
+#pragma unroll 1
+        for (int b = 0; b < kQ; ++b) {
+            const double dx = xa - qj[3 * b], dy = ya - qj[3 * b + 1], dz = za - qj[3 * b + 2];
+            s += c_w7[b] * rsqrt(dx * dx + dy * dy + dz * dz);
+        }
+        acc += c_w7[a] * s;
+    }
+    return qi[21] * (qj[21] * kInv4Pi) * acc;
+}
+
+// Pairs at least 1.5 (R_i + R_j) apart (R: the largest distance of a triangle's points from
+// its centroid) take |x_a - y_b|^2 = E_a + n_b - 2 e_a.o_b, e_a = x_a - c_j, o_b = y_b -
+// c_j, n_b = |o_b|^2: 4 FP64 operations per point pair instead of 6.  The reciprocal root is
+// the FP32 MUFU estimate on a grid (estimates of equal weight add exactly in FP32) and the
+// correction y t / 2 + 3/8 y t^2, t = 1 - S y^2: 3 FP64 operations (y^2, t, the sum of y t)
+// and the t^2 term, below 2^-34, in FP32, where rsqrt took about 8.  Conversions are integer
+// operations.  7 FP64 operations per point pair instead of 15; bound by the FP64 pipe (2
+// lanes per SM and cycle: 84% of it, 402 operations per entry).  Rotated polycubes, best tile:
+// N = 604 434 -> 238 us, N = 2,416 3.40 -> 2.43 ms, N = 9,664 51.2 -> 34.7 ms.  Error of an entry (CPU emulation against 80 bits): r.m.s. 0.9 -
+// 1.3e-16, 1.0 - 1.4e-16 before.  Close pairs are put aside per warp as in far_df_body.
+template <int R, int C>
+__device__ __forceinline__ void far_f64_body(const double *__restrict__ q64, const double *__restrict__ cent,
+                                             double *__restrict__ V, int64_t ld, int64_t r1, int64_t c1, int64_t i0,
+                                             int64_t cbase)
+{
+    __shared__ double sx[R][kQ64Stride];
+    __shared__ double sc[R][3];
+    __shared__ unsigned short close_s[C / 32][64];
     if (i0 > cbase + C - 1 || i0 >= r1) return;  // tile strictly below the diagonal
-    for (int k = threadIdx.x; k < R * 22; k += C) {
-        const int r = k / 22, c = k % 22;
-        const int64_t i = i0 + r;
-        sx[r][c] = (i < r1) ? q64[i * kQ64Stride + c] : 0.0;
+    for (int k = threadIdx.x; k < R * kQ64Stride; k += C) {
+        const int r = k / kQ64Stride, c = k % kQ64Stride;
+        const int64_t i = i0 + r < r1 ? i0 + r : r1 - 1;
+        sx[r][c] = q64[i * kQ64Stride + c];
+        if (c < 3) sc[r][c] = cent[4 * i + c];
     }
     __syncthreads();
-    const int64_t j = cbase + threadIdx.x;
-    if (j >= c1) return;
-    double y[3 * kQ];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t jw = cbase + 32 * warp, j = jw + lane, jc = j < c1 ? j : c1 - 1;
+    if (jw >= c1) return;
+    const double cj[3] = {cent[4 * jc], cent[4 * jc + 1], cent[4 * jc + 2]};
+    double o[3 * kQ], n[kQ];
 #pragma unroll
-    for (int c = 0; c < 3 * kQ; ++c) y[c] = q64[j * kQ64Stride + c];
-    const double Aj = q64[j * kQ64Stride + 21] * kInv4Pi;
-    const int rows = (int)((r1 - i0) < R ? (r1 - i0) : R);
+    for (int b = 0; b < kQ; ++b) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) o[3 * b + c] = q64[jc * kQ64Stride + 3 * b + c] - cj[c];
+        n[b] = fma(o[3 * b + 2], o[3 * b + 2], fma(o[3 * b + 1], o[3 * b + 1], o[3 * b] * o[3 * b]));
+    }
+    const double Aj = q64[jc * kQ64Stride + 21] * kInv4Pi;
+    const float Rj = (float)q64[jc * kQ64Stride + 23];
+    unsigned short *list = close_s[warp];
+    int n_close = 0;
+    auto flush = [&](int m) {  // the first m pairs put aside (m <= 32)
+        __syncwarp();
+        if (lane < m) {
+            const int e = list[lane];
+            const int64_t i = i0 + (e >> 5), jj = jw + (e & 31);
+            V[i * ld + jj] = far_f64_close(q64 + i * kQ64Stride, q64 + jj * kQ64Stride);
+        }
+        __syncwarp();
+    };
+    int rows = (int)((r1 - i0) < R ? (r1 - i0) : R);
+    if (jw + 32 - i0 < rows) rows = (int)(jw + 32 - i0);  // rows past the warp's last column: below the diagonal
     for (int r = 0; r < rows; ++r) {
         const int64_t i = i0 + r;
-        if (i > j) break;
-        double acc = 0.0;
+        const bool valid = j < c1 && i <= j;
+        const float fx = f64_to_f32_abs(sc[r][0] - cj[0]), fy = f64_to_f32_abs(sc[r][1] - cj[1]),
+                    fz = f64_to_f32_abs(sc[r][2] - cj[2]);
+        const float D2 = fx * fx + fy * fy + fz * fz, Rs = f64_to_f32_abs(sx[r][23]) + Rj;
+        // where the bounds hold and |x - y|^2 is a normal FP32 number; not for NaN
+        const bool wide = D2 >= kFarSpread2 * (Rs * Rs) && D2 >= 0x1p-68f && D2 <= 0x1p100f;
+        if (valid && wide) {
+            float y0;
+            asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"(D2));
+            const float by = grid_big(y0, 6);
+            // class sums by weight: w0^2, w0 w1, w0 w2, w1^2, w1 w2, w2^2
+            float s[6], q[6];
+            double l[6];
 #pragma unroll
-        for (int a = 0; a < kQ; ++a) {
-            const double xa = sx[r][3 * a], ya = sx[r][3 * a + 1], za = sx[r][3 * a + 2];
-            double s = 0.0;
-#pragma unroll
-            for (int b = 0; b < kQ; ++b) {
-                const double dx = xa - y[3 * b], dy = ya - y[3 * b + 1], dz = za - y[3 * b + 2];
-                s += c_w7[b] * rsqrt(dx * dx + dy * dy + dz * dz);
+            for (int k = 0; k < 6; ++k) {
+                s[k] = q[k] = 0.0f;
+                l[k] = 0.0;
             }
-            acc += c_w7[a] * s;
+#pragma unroll
+            for (int a = 0; a < kQ; ++a) {
+                const double ex = sx[r][3 * a] - cj[0], ey = sx[r][3 * a + 1] - cj[1], ez = sx[r][3 * a + 2] - cj[2];
+                const double E = fma(ez, ez, fma(ey, ey, ex * ex));
+                const double mx = f64_m2(ex), my = f64_m2(ey), mz = f64_m2(ez);
+#pragma unroll
+                for (int b = 0; b < kQ; ++b) {
+                    constexpr int kClass[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+                    const int k = kClass[(a + 2) / 3][(b + 2) / 3];
+                    const double S = fma(mz, o[3 * b + 2], fma(my, o[3 * b + 1], fma(mx, o[3 * b], E + n[b])));
+                    float y;
+                    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(f64_to_f32_trunc(S)));
+                    y = grid_snap(y, by);
+                    const double yd = f32_to_f64_pos(y);
+                    const double t = fma(-S, yd * yd, 1.0);
+                    const float tf = f64_to_f32_abs(t);
+                    s[k] = __fadd_rn(s[k], y);
+                    l[k] = fma(yd, t, l[k]);
+                    q[k] = __fmaf_rn(y * tf, tf, q[k]);
+                }
+            }
+            constexpr double w[6] = {kW0 * kW0, kW0 * kW1, kW0 * kW2, kW1 * kW1, kW1 * kW2, kW2 * kW2};
+            double acc = 0.0;
+#pragma unroll
+            for (int k = 0; k < 6; ++k)
+                acc = fma(w[k], fma(0.5, l[k], f32_to_f64_pos(s[k])) + f32_to_f64_pos(0.375f * q[k]), acc);
+            V[i * ld + j] = sx[r][21] * Aj * acc;
         }
-        V[i * ld + j] = sx[r][21] * Aj * acc;
+        const bool put = valid && !wide && i != j;  // (i, i) is the near field's
+        const unsigned mask = __ballot_sync(0xffffffffu, put);
+        if (mask) {
+            if (put) list[n_close + __popc(mask & ((1u << lane) - 1u))] = (unsigned short)(r * 32 + lane);
+            n_close += __popc(mask);
+            if (n_close >= 32) {
+                flush(32);
+                n_close -= 32;
+                unsigned short rest = 0;
+                if (lane < n_close) rest = list[32 + lane];
+                __syncwarp();
+                if (lane < n_close) list[lane] = rest;
+                __syncwarp();
+            }
+        }
     }
+    if (n_close) flush(n_close);
 }
 
 template <int R, int C>
-__global__ void __launch_bounds__(C) k_far_f64(const double *__restrict__ q64, double *__restrict__ V,
-                                                      int64_t ld, int64_t r0, int64_t r1, int64_t c0,
-                                                      int64_t c1)
+__global__ void __launch_bounds__(C) k_far_f64(const double *__restrict__ q64, const double *__restrict__ cent,
+                                               double *__restrict__ V, int64_t ld, int64_t r0, int64_t r1, int64_t c0,
+                                               int64_t c1)
 {
-    far_f64_body<R, C>(q64, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
+    far_f64_body<R, C>(q64, cent, V, ld, r1, c1, r0 + (int64_t)blockIdx.y * R, c0 + (int64_t)blockIdx.x * C);
 }
 
 template <int R, int C>
@@ -302,17 +442,6 @@ __global__ void __launch_bounds__(C) k_far_f32(const float *__restrict__ q32,
 
 // Double-float far field: see the file comment.
 //
-// v rounded to the nearest multiple of q = 2^(e-23), for |v| < 2^(e-1) and big =
-// 1.5 * 2^e: v + big lies in [2^e, 2^(e+1)], whose spacing is q, and the subtraction
-// of big is exact (Sterbenz).
-__device__ __forceinline__ float grid_snap(float v, float big) { return __fsub_rn(__fadd_rn(v, big), big); }
-
-// 1.5 * 2^(k + up) for a normal v in [2^k, 2^(k+1))
-__device__ __forceinline__ float grid_big(float v, unsigned up)
-{
-    return __uint_as_float(((__float_as_uint(v) & 0x7f800000u) + (up << 23)) | 0x400000u);
-}
-
 // s + e = a + b exactly for a, b >= 0 (Dekker's fast two-sum with the larger first).
 __device__ __forceinline__ void pos_two_sum(float a, float b, float &s, float &e)
 {
@@ -434,12 +563,9 @@ __device__ __noinline__ float2 far_df_close(const float *__restrict__ qi, const 
 // each).  Bound by FP32 issue (73% of the 128 lanes per SM and cycle).  Measured on rotated
 // polycubes, best tile of each: N = 604 116 -> 35 us, N = 2,416 418 -> 166 us, N = 9,664
 // 4.60 -> 2.03 ms, N = 21,744 22.3 -> 9.88 ms (10.6 -> 23.9 Gpairs/s).
-constexpr double kSqrt15 = 3.87298334620741688518;
 constexpr double kOrbS = (1.0 - kSqrt15) / (1.0 + kSqrt15);
 constexpr float kOrbSh = (float)kOrbS, kOrbSl = (float)(kOrbS - (double)kOrbSh);
 constexpr float kOrbS2h = (float)(kOrbS * kOrbS), kOrbS2l = (float)(kOrbS * kOrbS - (double)kOrbS2h);
-constexpr double kW0 = 9.0 / 40.0, kW1 = (155.0 - kSqrt15) / 1200.0, kW2 = (155.0 + kSqrt15) / 1200.0;
-constexpr float kFarSpread2 = 2.2505f;  // 1.5^2, rounded up past the FP32 errors of the test
 
 // h + l = (ah + al) (bh + bl), h on the grid
 __device__ __forceinline__ void grid_prod(float ah, float al, float bh, float bl, float big, float &h, float &l)
@@ -1014,7 +1140,7 @@ static void far_kernel(bem_operator *op, dim3 grid, int64_t r0, int64_t r1, int6
     bem_mesh *m = op->mesh;
     cudaStream_t s = m->ctx->stream;
     if (op->precision == BEM_PREC_F64)
-        k_far_f64<R, C><<<grid, C, 0, s>>>(m->q64, (double *)op->V, op->ld, r0, r1, c0, c1);
+        k_far_f64<R, C><<<grid, C, 0, s>>>(m->q64, m->cent, (double *)op->V, op->ld, r0, r1, c0, c1);
     else if (op->precision == BEM_PREC_DF64)
     {
         if constexpr (MB > 0)
@@ -1276,7 +1402,7 @@ __global__ void __launch_bounds__(C, (MB > 0 ? MB : 1))
     const BatchAsmProb *pb = prob + it.x;
     const int64_t N = pb->N, ld = pb->ld;
     if constexpr (std::is_same<T, double>::value)
-        far_f64_body<R, C>(pb->q64, (double *)pb->V, ld, N, N, it.y, it.z);
+        far_f64_body<R, C>(pb->q64, pb->cent, (double *)pb->V, ld, N, N, it.y, it.z);
     else if constexpr (std::is_same<T, float2>::value)
         far_df_body<R, C>(pb->qdf, (float2 *)pb->V, ld, N, N, it.y, it.z);
     else

@@ -96,7 +96,8 @@ struct bem_mesh {
     int32_t *tris = nullptr;    // N x 3, reference edge first
     double *area = nullptr;     // N
     double *diam = nullptr;     // N
-    double *q64 = nullptr;      // N x 24: 7 points (x,y,z), [21] = area
+    double *q64 = nullptr;      // N x 24: 7 points (x,y,z), [21] = area, [22] = diam, [23] = the
+                                // largest distance of a point from the centroid
     float *q32 = nullptr;       // N x 24: 7 offsets from the centroid (x,y,z)
     double *cent = nullptr;     // N x 4: centroid (x,y,z), area
     float *qdf = nullptr;       // N x 56: double-float table (see kQdfStride)

@@ -281,7 +281,6 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
         }
     q[21] = A;
     q[22] = d;
-    q[23] = 0.0;
     o[21] = o[22] = o[23] = 0.0f;
     // double-float table: offsets lambda . (P - c) from the centroid, the centroid
     // itself as an exact sum of three floats, and the area
@@ -313,6 +312,7 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
     }
     f[53] = rm;
     f[54] = __double2float_ru(sqrt(rd2) * (1.0 + 1e-12));
+    q[23] = (double)f[54];
     f[55] = 0.0f;
     // expanded form: orbit offsets o_1k = t (P_k - c), t = 1 - 3 a of the first orbit, and
     // their squared lengths (o_2k = s o_1k; vertex 2's offset as minus the others' sum)
