@@ -10,6 +10,8 @@
 #include <new>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "bem_internal.cuh"
 #include "dfloat.cuh"
 
@@ -70,17 +72,28 @@ __global__ void k_zz_eta(const int32_t *tris, const double *area, const double *
     }
 }
 
-__global__ void k_sum2(const double *a, const double *b, int n, double *out)
+// Two left-to-right sums, each by one thread from shared memory: the loads of a chunk are
+// issued together (one thread reading global memory took 20 us for 151 terms,
+// now 8).
+__global__ void __launch_bounds__(256) k_sum2(const double *a, const double *b, int n, double *out)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0, t = 0.0;
-        for (int k = 0; k < n; ++k) {
-            s += a[k];
-            t += b[k];
+    __shared__ double sa[512], sb[512];
+    double s = 0.0;
+    for (int k0 = 0; k0 < n; k0 += 512) {
+        const int m = n - k0 < 512 ? n - k0 : 512;
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += blockDim.x) {
+            sa[k] = a[k0 + k];
+            sb[k] = b[k0 + k];
         }
-        out[0] = s;
-        out[1] = t;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int k = 0; k < m; ++k) s += sa[k];
+        if (threadIdx.x == 32)
+            for (int k = 0; k < m; ++k) s += sb[k];
     }
+    if (threadIdx.x == 0) out[0] = s;
+    if (threadIdx.x == 32) out[1] = s;
 }
 
 bem_status zz_estimate(bem_mesh *m, const double *d_phi, int h_mode, double *d_eta2, double *h_totals,
@@ -96,7 +109,7 @@ bem_status zz_estimate(bem_mesh *m, const double *d_phi, int h_mode, double *d_e
     double *pe = u + m->M, *ps = pe + nb, *tot = d_totals ? d_totals : ps + nb;
     k_zz_nodal<<<nblk(m->M, 128), 128, 0, s>>>(m->v2t_off, m->v2t, m->area, d_phi, u, m->M); BEM_COUNT(ctx);
     k_zz_eta<<<nb, 256, 0, s>>>(m->tris, m->area, m->diam, d_phi, u, m->N, h_mode, d_eta2, pe, ps); BEM_COUNT(ctx);
-    k_sum2<<<1, 32, 0, s>>>(pe, ps, nb, tot); BEM_COUNT(ctx);
+    k_sum2<<<1, 256, 0, s>>>(pe, ps, nb, tot); BEM_COUNT(ctx);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) st = cuda_error(ctx, e, "zz kernels");
     if (!st && h_totals) {
@@ -168,16 +181,14 @@ __global__ void k_bitonic_shared(unsigned long long *keys, int64_t n2, int64_t k
     for (int q = threadIdx.x; q < chunk; q += blockDim.x) keys[base + q] = sk[q];
 }
 
-// The whole bitonic network of n2 <= kSortBlockMax keys in one CTA's shared memory
-// (one launch instead of one per stage for the arrays of the first adaptive levels);
-// the keys are unique, so the result is the array the per-stage kernels produce.
-constexpr int64_t kSortBlockMax = 16384;  // 128 KB of shared memory
+// The whole bitonic network of each chunk of n2 keys in one CTA's shared memory.
 constexpr int kSortBlockThreads = 1024;
 
 __global__ void __launch_bounds__(kSortBlockThreads) k_bitonic_block(unsigned long long *keys, int64_t n2)
 {
     extern __shared__ unsigned long long sk[];
     const int n = (int)n2, half = n / 2;
+    keys += (int64_t)blockIdx.x * n2;
     for (int q = threadIdx.x; q < n; q += blockDim.x) sk[q] = keys[q];
     __syncthreads();
     for (int k = 2; k <= n; k <<= 1)
@@ -196,6 +207,39 @@ __global__ void __launch_bounds__(kSortBlockThreads) k_bitonic_block(unsigned lo
     for (int q = threadIdx.x; q < n; q += blockDim.x) keys[q] = sk[q];
 }
 
+// Each key of nc sorted chunks (chunk a power of two) to its place in the whole: its rank is
+// its place in its own chunk plus, for every other chunk, the number of smaller keys there, by
+// a binary search; four searches in flight.  The padding (all ones, never a key) stays where
+// it is.
+__global__ void __launch_bounds__(256) k_sort_merge(const unsigned long long *__restrict__ keys, int nc, int chunk,
+                                                    unsigned long long *__restrict__ out)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)nc * chunk) return;
+    const unsigned long long key = keys[i];
+    if (key == ~0ull) return;
+    const int own = (int)(i / chunk);
+    int64_t rank = i % chunk;
+    for (int c0 = 0; c0 < nc; c0 += 4) {
+        int lo[4] = {0, 0, 0, 0};
+        for (int step = chunk >> 1; step; step >>= 1)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int c = c0 + u < nc ? c0 + u : own;
+                const unsigned long long v = __ldg(keys + (int64_t)c * chunk + lo[u] + step - 1);
+                if (v < key) lo[u] += step;
+            }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int c = c0 + u;
+            if (c >= nc || c == own) continue;
+            const unsigned long long v = __ldg(keys + (int64_t)c * chunk + lo[u]);
+            rank += lo[u] + (v < key ? 1 : 0);
+        }
+    }
+    out[rank] = key;
+}
+
 // Running FP64 sums of eta2 in key order, in a fixed two-level order: the sorted
 // sequence is cut into blocks of kDorflerBlock; l = the running sum inside a block
 // (from 0, left to right), o_b = the offset of block b (o_0 = 0, o_(b+1) = o_b +
@@ -205,81 +249,100 @@ __global__ void __launch_bounds__(kSortBlockThreads) k_bitonic_block(unsigned lo
 // instead of N.
 constexpr int kDorflerBlock = 128;
 
-// One thread per block: the running sums inside the block and the block's sum.
-__global__ void k_dorfler_blocks(const unsigned long long *__restrict__ keys, const double *__restrict__ eta2,
-                                 int64_t N, double *__restrict__ prefix, double *__restrict__ bsum)
+// One warp per block: the indicators gathered by all lanes, the running sums by the first
+// from shared memory (one thread gathering its own took 24 us at N = 38,656, now 10).
+__global__ void __launch_bounds__(128) k_dorfler_blocks(const unsigned long long *__restrict__ keys,
+                                                        const double *__restrict__ eta2, int64_t N,
+                                                        double *__restrict__ prefix, double *__restrict__ bsum)
 {
-    const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t b0 = b * kDorflerBlock;
+    __shared__ double sv[4][kDorflerBlock];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t b = (int64_t)blockIdx.x * 4 + w, b0 = b * kDorflerBlock;
     if (b0 >= N) return;
     const int n = (int)((N - b0) < kDorflerBlock ? (N - b0) : kDorflerBlock);
-    double l = 0.0;
-    int q = 0;
-    for (; q + 16 <= n; q += 16) {  // loads of a group issued before its additions
-        double r[16];
+    double *v = sv[w];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) r[u] = eta2[keys[b0 + q + u] & 0xFFFFFFFFull];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            l = l + r[u];
-            prefix[b0 + q + u] = l;
+    for (int q = lane; q < kDorflerBlock; q += 32)
+        if (q < n) v[q] = eta2[keys[b0 + q] & 0xFFFFFFFFull];
+    __syncwarp();
+    if (lane == 0) {
+        double l = 0.0;
+#pragma unroll 8
+        for (int q = 0; q < n; ++q) {
+            l = l + v[q];
+            v[q] = l;
         }
+        bsum[b] = l;
     }
-    for (; q < n; ++q) {
-        l = l + eta2[keys[b0 + q] & 0xFFFFFFFFull];
-        prefix[b0 + q] = l;
-    }
-    bsum[b] = l;
+    __syncwarp();
+    for (int q = lane; q < n; q += 32) prefix[b0 + q] = v[q];
 }
 
-// The block offsets, by one thread: off[0] = 0, off[b + 1] = off[b] + bsum[b].
-__global__ void k_dorfler_offsets(const double *__restrict__ bsum, int64_t nb, double *__restrict__ off)
+// One CTA: the block offsets (off[0] = 0, off[b + 1] = off[b] + bsum[b]) by one thread from
+// shared memory, then the shortest prefix whose running sum (off[block of k] + the running
+// sum inside the block) reaches theta * total (total = the last running sum; none if theta *
+// total <= 0), by a 32-way search of the first warp over the non-decreasing sums, then
+// extended over equal keys.
+constexpr int kDorflerChunk = 2048;
+__global__ void __launch_bounds__(256) k_dorfler_select(const unsigned long long *keys, const double *prefix,
+                                                        const double *__restrict__ bsum, int64_t nb, double *off,
+                                                        int64_t N, double theta, const double *vanish,
+                                                        long long *K_out)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double o = 0.0;
-    off[0] = 0.0;
-    for (int64_t b = 0; b < nb; ++b) {
-        o = o + bsum[b];
-        off[b + 1] = o;
-    }
-}
-
-// prefix[k] = off[block of k] + (running sum inside the block).
-__global__ void k_dorfler_finish(const double *__restrict__ off, int64_t N, double *__restrict__ prefix)
-{
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < N) prefix[k] = off[k / kDorflerBlock] + prefix[k];
-}
-
-// The shortest prefix whose running sum reaches theta * total (total = prefix[N-1];
-// none if theta * total <= 0), by bisection over the non-decreasing prefix sums,
-// then extended over equal keys.
-__global__ void k_dorfler_select(const unsigned long long *keys, const double *prefix, int64_t N, double theta,
-                                 const double *vanish, long long *K_out)
-{
+    __shared__ double sv[kDorflerChunk];
     // vanish (nullable): [sum eta^2, sum h|T|x^2/12]; when every indicator vanishes up
     // to rounding (sum eta^2 <= 1e-20 of the scale) Eq. 2.6 holds for the empty set and
     // every element is marked (uniform refinement)
     if (vanish && !(vanish[0] > 1e-20 * vanish[1])) {
-        *K_out = N;
+        if (threadIdx.x == 0) *K_out = N;
         return;
     }
-    const double thr = theta * prefix[N - 1];
+    double o = 0.0;
+    if (threadIdx.x == 0) off[0] = 0.0;
+    for (int64_t c0 = 0; c0 < nb; c0 += kDorflerChunk) {
+        const int m = (int)(nb - c0 < kDorflerChunk ? nb - c0 : kDorflerChunk);
+        for (int k = threadIdx.x; k < m; k += blockDim.x) sv[k] = bsum[c0 + k];
+        __syncthreads();
+        if (threadIdx.x == 0) {
+#pragma unroll 8
+            for (int k = 0; k < m; ++k) {
+                o = o + sv[k];
+                sv[k] = o;
+            }
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < m; k += blockDim.x) off[c0 + k + 1] = sv[k];
+        __syncthreads();
+    }
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    auto sum_to = [&](int64_t k) { return off[k / kDorflerBlock] + prefix[k]; };  // off: this CTA's own writes
+    const double thr = theta * sum_to(N - 1);
     int64_t kk = 0;
     if (0.0 < thr) {
-        int64_t lo = 0, hi = N - 1;  // prefix[hi] >= thr
-        if (!(prefix[hi] >= thr)) lo = hi = N;
-        while (lo < hi) {
-            const int64_t mid = lo + (hi - lo) / 2;
-            if (prefix[mid] >= thr)
-                hi = mid;
-            else
-                lo = mid + 1;
+        if (!(sum_to(N - 1) >= thr)) {
+            kk = N;
+        } else {
+            int64_t lo = 0, hi = N - 1;  // the first k with sum >= thr is in [lo, hi]
+            while (lo < hi) {
+                const int64_t step = (hi - lo + 31) / 32, k = lo + lane * step;  // probes lo, lo + step, ...
+                const unsigned reach = __ballot_sync(0xffffffffu, k >= hi || sum_to(k) >= thr);
+                const int f = __ffs(reach) - 1;  // lane f's probe is the first that reaches it
+                if (reach == 0) {
+                    lo = lo + 31 * step + 1;
+                } else {
+                    const int64_t top = lo + f * step;
+                    if (top < hi) hi = top;
+                    if (f > 0) lo = lo + (f - 1) * step + 1;
+                }
+            }
+            kk = lo + 1;
         }
-        kk = lo < N ? lo + 1 : N;
     }
-    while (kk > 0 && kk < N && (keys[kk] >> 32) == (keys[kk - 1] >> 32)) ++kk;
-    *K_out = kk;
+    if (lane == 0) {
+        while (kk > 0 && kk < N && (keys[kk] >> 32) == (keys[kk - 1] >> 32)) ++kk;
+        *K_out = kk;
+    }
 }
 
 __global__ void k_mark(const unsigned long long *keys, int64_t N, const long long *K, uint8_t *marked)
@@ -289,22 +352,24 @@ __global__ void k_mark(const unsigned long long *keys, int64_t N, const long lon
     marked[keys[k] & 0xFFFFFFFFull] = (k < *K) ? 1 : 0;
 }
 
-void sort_u64(bem_ctx *ctx, unsigned long long *keys, int64_t n2)
+// Up to kSortMergeMax keys: chunks sorted in shared memory by a CTA each, then every key to
+// its rank.  Two launches; the network of the 65,536 keys of N = 38,656 took
+// 31 and 134 us without the gaps between them, now 55 us.
+// Above, where the searches' n^2 / chunk steps grow, the network's launches.
+constexpr int64_t kSortMergeMax = 131072;
+
+size_t sort_u64_keys(int64_t n2) { return (size_t)(n2 <= kSortMergeMax ? 2 * n2 : n2); }
+
+unsigned long long *sort_u64(bem_ctx *ctx, unsigned long long *keys, int64_t n, int64_t n2)
 {
     cudaStream_t s = ctx->stream;
-    if (n2 <= kSortBlockMax) {
-        const size_t smem = sizeof(unsigned long long) * (size_t)n2;
-        bool ok = true;  // shared memory beyond 48 KB needs the opt-in
-        if (smem > 48 * 1024 && cudaFuncSetAttribute(k_bitonic_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)(sizeof(unsigned long long) * kSortBlockMax)) != cudaSuccess) {
-            cudaGetLastError();
-            ok = false;
-        }
-        if (ok) {
-            const int threads = (int)std::min<int64_t>(kSortBlockThreads, std::max<int64_t>(n2 / 2, 32));
-            k_bitonic_block<<<1, threads, smem, s>>>(keys, n2); BEM_COUNT(ctx);
-            return;
-        }
+    if (n2 <= kSortMergeMax) {
+        const int64_t ch = std::min<int64_t>(n2, n2 <= 16384 ? 1024 : 2048);
+        const int threads = (int)std::max<int64_t>(ch / 2, 32), nc = (int)((n + ch - 1) / ch);
+        k_bitonic_block<<<nc, threads, sizeof(unsigned long long) * (size_t)ch, s>>>(keys, ch); BEM_COUNT(ctx);
+        if (nc == 1) return keys;
+        k_sort_merge<<<nblk(nc * ch, 256), 256, 0, s>>>(keys, nc, (int)ch, keys + n2); BEM_COUNT(ctx);
+        return keys + n2;
     }
     const int64_t chunk = n2 < 2048 ? n2 : 2048;
     const int sthreads = (int)(chunk / 2);
@@ -314,6 +379,7 @@ void sort_u64(bem_ctx *ctx, unsigned long long *keys, int64_t n2)
             { k_bitonic_global<<<nblk(n2 / 2, 256), 256, 0, s>>>(keys, n2, k, j); BEM_COUNT(ctx); }
         k_bitonic_shared<<<(unsigned)(n2 / chunk), sthreads, chunk * sizeof(unsigned long long), s>>>(keys, n2, k, j); BEM_COUNT(ctx);
     }
+    return keys;
 }
 
 bem_status dorfler(bem_ctx *ctx, const double *d_eta2, int64_t N, double theta, uint8_t *d_marked,
@@ -333,17 +399,15 @@ bem_status dorfler(bem_ctx *ctx, const double *d_eta2, int64_t N, double theta, 
     unsigned long long *keys = nullptr;
     const int64_t nb = (N + kDorflerBlock - 1) / kDorflerBlock;
     bem_status st = dalloc(ctx, tmp, (void **)&keys,
-                           sizeof(unsigned long long) * n2 + sizeof(double) * (N + 2 * nb + 1) + 64, false);
+                           sizeof(unsigned long long) * sort_u64_keys(n2) + sizeof(double) * (N + 2 * nb + 1) + 64, false);
     if (st) return st;
-    double *prefix = reinterpret_cast<double *>(keys + n2);
+    double *prefix = reinterpret_cast<double *>(keys + sort_u64_keys(n2));
     double *bsum = prefix + N, *off = bsum + nb;
     long long *dK = reinterpret_cast<long long *>(off + nb + 1);
     k_keys<<<nblk(n2, 256), 256, 0, s>>>(d_eta2, N, n2, keys); BEM_COUNT(ctx);
-    sort_u64(ctx, keys, n2);
-    k_dorfler_blocks<<<nblk(nb, 64), 64, 0, s>>>(keys, d_eta2, N, prefix, bsum); BEM_COUNT(ctx);
-    k_dorfler_offsets<<<1, 32, 0, s>>>(bsum, nb, off); BEM_COUNT(ctx);
-    k_dorfler_finish<<<nblk(N, 256), 256, 0, s>>>(off, N, prefix); BEM_COUNT(ctx);
-    k_dorfler_select<<<1, 1, 0, s>>>(keys, prefix, N, theta, d_vanish, dK); BEM_COUNT(ctx);
+    keys = sort_u64(ctx, keys, N, n2);
+    k_dorfler_blocks<<<nblk(nb, 4), 128, 0, s>>>(keys, d_eta2, N, prefix, bsum); BEM_COUNT(ctx);
+    k_dorfler_select<<<1, 256, 0, s>>>(keys, prefix, bsum, nb, off, N, theta, d_vanish, dK); BEM_COUNT(ctx);
     k_mark<<<nblk(N, 256), 256, 0, s>>>(keys, N, dK, d_marked); BEM_COUNT(ctx);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && d_count) e = cudaMemcpyAsync(d_count, dK, sizeof(long long), cudaMemcpyDeviceToDevice, s);
@@ -371,31 +435,40 @@ __global__ void k_nvb_seed(const int32_t *owner, const uint8_t *marked, int64_t 
 }
 
 // One closure sweep: a triangle with a marked edge marks its reference edge.
-// The closure to its fixed point in one CTA (meshes up to kCloseBlockMax triangles):
+// The closure to its fixed point in one cluster (meshes up to kCloseBlockMax triangles):
 // sweeps until one changes nothing.  Flags only go from 0 to 1, so the fixed point
 // (the least closed set containing the seeds) does not depend on the order of the
 // updates; each sweep that changes something sets at least one of the 3N flags, so
 // 3N + 1 sweeps always reach it.
 constexpr int64_t kCloseBlockMax = 65536;
+constexpr int kCloseCtas = 8;
 
-__global__ void __launch_bounds__(1024) k_nvb_close_block(const int32_t *owner, int64_t N, uint8_t *flag)
+// A cluster of kCloseCtas CTAs (eight SMs instead of one); the flags meet at its barrier, and
+// so do the sweep's change marks, two of them in turn in the first CTA's shared memory.
+__global__ void __cluster_dims__(kCloseCtas, 1, 1) __launch_bounds__(1024)
+    k_nvb_close_block(const int32_t *owner, int64_t N, uint8_t *flag)
 {
-    __shared__ int changed;
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ int changed[2];
+    int *const mark = cl.map_shared_rank(changed, 0);
+    if (threadIdx.x < 2) changed[threadIdx.x] = 0;
+    cl.sync();
     for (int64_t sweep = 0; sweep <= 3 * N; ++sweep) {
-        if (threadIdx.x == 0) changed = 0;
-        __syncthreads();
         int c = 0;
-        for (int64_t t = threadIdx.x; t < N; t += blockDim.x) {
+        for (int64_t t = (int64_t)cl.block_rank() * blockDim.x + threadIdx.x; t < N; t += kCloseCtas * blockDim.x) {
             const int32_t o0 = owner[3 * t];
             if (!flag[o0] && (flag[owner[3 * t + 1]] | flag[owner[3 * t + 2]])) {
                 flag[o0] = 1;
                 c = 1;
             }
         }
-        if (c) changed = 1;
-        __syncthreads();
-        const int done = !changed;
-        __syncthreads();  // every thread has read changed before thread 0 clears it
+        if (__syncthreads_or(c) && threadIdx.x == 0) mark[sweep & 1] = 1;
+        cl.sync();
+        const int done = !*(volatile int *)(mark + (sweep & 1));
+        // the mark of the next sweep but one: written again only after the next barrier
+        if (cl.block_rank() == 0 && threadIdx.x == 0) changed[(sweep & 1) ^ 1] = 0;
+        cl.sync();
         if (done) return;
     }
 }
@@ -513,11 +586,11 @@ bem_status refine(bem_mesh *m, const uint8_t *d_marked, int flags, bem_mesh **ou
     TRY(dalloc(ctx, tmp, (void **)&n_child, sizeof(int32_t) * (N + 1), false));
     TRY(dalloc(ctx, tmp, (void **)&child_pos, sizeof(int32_t) * (N + 1), false));
     k_nvb_seed<<<nblk(N, 256), 256, 0, s>>>(m->owner, d_marked, N, flags & BEM_REFINE_BISEC3, flag); BEM_COUNT(ctx);
-    // closure: in one CTA for meshes up to kCloseBlockMax triangles; larger ones by
+    // closure: in one cluster for meshes up to kCloseBlockMax triangles; larger ones by
     // sweeps over the grid, eight per check of the changed flag (a sweep after the
     // fixed point changes nothing; a level's closure rarely needs more than eight)
     if (N <= kCloseBlockMax) {
-        k_nvb_close_block<<<1, 1024, 0, s>>>(m->owner, N, flag); BEM_COUNT(ctx);
+        k_nvb_close_block<<<kCloseCtas, 1024, 0, s>>>(m->owner, N, flag); BEM_COUNT(ctx);
     }
     for (int sweep = 0; N > kCloseBlockMax; sweep += 8) {
         if (sweep > 100000) {
@@ -830,7 +903,7 @@ bem_status zz_estimate_dual(bem_mesh *m, const double *d_x, int h_mode, double *
     if (st) return st;
     double *ps = pe + nb, *tot = ps + nb;
     k_zz_dual<<<nb, 256, 0, s>>>(m->tris, m->area, m->diam, d_x, m->N, h_mode, d_eta2, pe, ps); BEM_COUNT(ctx);
-    k_sum2<<<1, 32, 0, s>>>(pe, ps, nb, tot); BEM_COUNT(ctx);
+    k_sum2<<<1, 256, 0, s>>>(pe, ps, nb, tot); BEM_COUNT(ctx);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) st = cuda_error(ctx, e, "dual zz kernels");
     if (!st && h_totals) {

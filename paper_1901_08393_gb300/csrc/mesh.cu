@@ -288,51 +288,53 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
     double R[3][3];
     for (int k = 0; k < 3; ++k)
         for (int c = 0; c < 3; ++c) R[k][c] = P[k][c] - c3[c];
-    for (int a = 0; a < kQ; ++a)
-        for (int c = 0; c < 3; ++c) {
-            const double off = c_radon_bary[a][0] * R[0][c] + c_radon_bary[a][1] * R[1][c] +
-                               c_radon_bary[a][2] * R[2][c];
-            split2(off, f + 2 * (3 * a + c));
+    // the orbits: o_1k = t (P_k - c), t = 1 - 3 a of the first orbit, o_2k = s o_1k; the rule's
+    // points 1, 2, 3 (4, 5, 6) are those of vertices 2, 1, 0
+    constexpr double r15 = 3.87298334620741688518, ot = (1.0 + r15) / 7.0, os = (1.0 - r15) / (1.0 + r15);
+    double o1[3][3];
+    float rm = 0.0f;
+    for (int c = 0; c < 3; ++c) {
+        split2((1.0 / 3.0) * ((R[0][c] + R[1][c]) + R[2][c]), f + 2 * c);
+        for (int k = 0; k < 3; ++k) {
+            o1[k][c] = ot * R[k][c];
+            split2(o1[k][c], f + 2 * (3 * (3 - k) + c));
+            split2(os * o1[k][c], f + 2 * (3 * (6 - k) + c));
+            rm = fmaxf(rm, fabsf(f[2 * (3 * (3 - k) + c)]));  // the first orbit's are the largest
         }
+    }
     for (int c = 0; c < 3; ++c) split3(c3[c], f + 42 + 3 * c);
     split2(A, f + 51);
-    // the largest |hi part| of the 21 offset coordinates (the far field's grid bound)
-    // and the largest distance of a point from the centroid, rounded up
-    float rm = 0.0f;
-    for (int k = 0; k < 3 * kQ; ++k) rm = fmaxf(rm, fabsf(f[2 * k]));
+    // the largest |hi part| of the offset coordinates and the largest distance of a point
+    // from the centroid (the first orbit's), rounded up; expanded form: orbit offsets of
+    // vertices 0 and 1 and the squared lengths (vertex 2's offset as minus the others' sum)
+    float *g = f + kQdfExp;
     double rd2 = 0.0;
-    for (int a = 0; a < kQ; ++a) {
-        double s2 = 0.0;
-        for (int c = 0; c < 3; ++c) {
-            const double off = c_radon_bary[a][0] * R[0][c] + c_radon_bary[a][1] * R[1][c] +
-                               c_radon_bary[a][2] * R[2][c];
-            s2 += off * off;
+    for (int k = 0; k < 3; ++k) {
+        const double n2 = (o1[k][0] * o1[k][0] + o1[k][1] * o1[k][1]) + o1[k][2] * o1[k][2];
+        rd2 = rd2 > n2 ? rd2 : n2;
+        if (k == 2) {
+            double m[3];
+            for (int c = 0; c < 3; ++c) m[c] = -(o1[0][c] + o1[1][c]);
+            const double e2 = (m[0] * m[0] + m[1] * m[1]) + m[2] * m[2];
+            split2(e2, g + 12 + 4 * k);
+            split2(os * os * e2, g + 14 + 4 * k);
+        } else {
+            split2(n2, g + 12 + 4 * k);
+            split2(os * os * n2, g + 14 + 4 * k);
         }
-        rd2 = rd2 > s2 ? rd2 : s2;
     }
     f[53] = rm;
     f[54] = __double2float_ru(sqrt(rd2) * (1.0 + 1e-12));
     q[23] = (double)f[54];
     f[55] = 0.0f;
-    // expanded form: orbit offsets o_1k = t (P_k - c), t = 1 - 3 a of the first orbit, and
-    // their squared lengths (o_2k = s o_1k; vertex 2's offset as minus the others' sum)
-    float *g = f + kQdfExp;
-    const double r15 = sqrt(15.0), ot = (1.0 + r15) / 7.0, os = (1.0 - r15) / (1.0 + r15);
-    double o1[3][3];
     for (int c = 0; c < 3; ++c) {
-        o1[0][c] = ot * R[0][c];
-        o1[1][c] = ot * R[1][c];
-        o1[2][c] = -(o1[0][c] + o1[1][c]);
-        split2(o1[0][c], g + 2 * c);
-        split2(o1[1][c], g + 6 + 2 * c);
+        for (int k = 0; k < 2; ++k) {  // the offsets' parts again
+            g[6 * k + 2 * c] = f[2 * (3 * (3 - k) + c)];
+            g[6 * k + 2 * c + 1] = f[2 * (3 * (3 - k) + c) + 1];
+        }
         g[24 + c] = f[42 + 3 * c];
         g[28 + c] = f[43 + 3 * c];
         g[32 + c] = f[44 + 3 * c];
-    }
-    for (int k = 0; k < 3; ++k) {
-        const double n2 = (o1[k][0] * o1[k][0] + o1[k][1] * o1[k][1]) + o1[k][2] * o1[k][2];
-        split2(n2, g + 12 + 4 * k);
-        split2(os * os * n2, g + 14 + 4 * k);
     }
     g[27] = f[54];
     g[31] = f[51];

@@ -2004,16 +2004,16 @@ static bem_status cluster_setup(bem_operator *op, Allocs &a, int32_t **perm_out,
     int64_t n2 = 2;
     while (n2 < N) n2 <<= 1;
     unsigned long long *keys = nullptr;
-    const size_t kb = sizeof(unsigned long long) * n2, pb = sizeof(int32_t) * nbj * kBJ;
+    const size_t kb = sizeof(unsigned long long) * sort_u64_keys(n2), pb = sizeof(int32_t) * nbj * kBJ;
     const int nbox = (int)std::min<int64_t>((N + 255) / 256, 64);
     bem_status st = dalloc(ctx, a, (void **)&keys, kb + pb + (6 + 6 * nbox) * sizeof(double) + 64, false);
     if (st) return st;
-    int32_t *perm = reinterpret_cast<int32_t *>(keys + n2);
+    int32_t *perm = reinterpret_cast<int32_t *>(keys + sort_u64_keys(n2));
     double *box = reinterpret_cast<double *>(reinterpret_cast<char *>(perm) + (pb + 7) / 8 * 8);
     k_cent_box<<<nbox, 256, 0, s>>>(op->mesh->cent, N, box + 6); BEM_COUNT(ctx);
     k_box_fold<<<1, 32, 0, s>>>(box + 6, nbox, box); BEM_COUNT(ctx);
     k_morton_keys<<<nblk(n2, 256), 256, 0, s>>>(op->mesh->cent, N, n2, box, keys); BEM_COUNT(ctx);
-    sort_u64(ctx, keys, n2);
+    keys = sort_u64(ctx, keys, N, n2);
     k_cluster_perm<<<nblk((int64_t)nbj * kBJ, 256), 256, 0, s>>>(keys, N, (int64_t)nbj * kBJ, perm); BEM_COUNT(ctx);
     BEM_CK_LAUNCH(ctx);
     *perm_out = perm;
@@ -2914,7 +2914,7 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             int64_t n2 = 2;
             while (n2 < meshes[p]->N) n2 <<= 1;
             later += 16.0 * far_batch_items_bound(tile, meshes[p]->N) + 1024.0 + sizeof(PcgArgs) + 512.0;
-            if (block) later += 8.0 * (double)n2 + 4.0 * kBJ * std::ceil(N / kBJ) + 6.0 * 8.0 * 80.0 + 1024.0;
+            if (block) later += 8.0 * (double)sort_u64_keys(n2) + 4.0 * kBJ * std::ceil(N / kBJ) + 6.0 * 8.0 * 80.0 + 1024.0;
         }
         avail = (int64_t)((double)fr * 0.9) - (int64_t)later;
         if (ctx->budget > 0) avail = std::min<int64_t>(avail, ctx->budget - ctx->in_use - (int64_t)later);
