@@ -498,6 +498,43 @@ __device__ __forceinline__ double symv_row4(const float2 *__restrict__ prow, con
     return df_to_double(s);
 }
 
+// The same over the partials of symv_h16_tiles' groups: the columns' (FP32) of tiles (J, I),
+// J < I, then the rows' of the groups of g tiles (I, I), (I, I + g), ...
+__device__ __forceinline__ double symv_row4_groups(const float2 *__restrict__ prow, const float *__restrict__ pcol,
+                                                   int nb, int g, int64_t i, int q)
+{
+    const int I = (int)(i / kSB), r = (int)(i % kSB), n = I + (nb - I + g - 1) / g;
+    const int n0 = (q * n) / 4, n1 = ((q + 1) * n) / 4;
+    const int64_t rbase = tile_pos(I, I, nb) * kSB + r;
+    auto load = [&](int k) {
+        const int64_t o = k < I ? tile_pos(k, I, nb) * kSB + r : rbase + (int64_t)(k - I) * g * kSB;
+        return k < I ? make_float2(__ldcg(pcol + o), 0.f) : __ldcg(prow + o);
+    };
+    float2 s = make_float2(0.f, 0.f);
+    int k = n0;
+    for (; k + 16 <= n1; k += 16) {
+        float2 v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = load(k + u);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) s = df_add(s, v[u]);
+    }
+    for (; k + 4 <= n1; k += 4) {
+        float2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = load(k + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s = df_add(s, v[u]);
+    }
+    for (; k < n1; ++k) s = df_add(s, load(k));
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const float2 t = make_float2(__shfl_xor_sync(0xffffffffu, s.x, o), __shfl_xor_sync(0xffffffffu, s.y, o));
+        s = (q & o) ? df_add(t, s) : df_add(s, t);
+    }
+    return df_to_double(s);
+}
+
 // Product of the packed FP32 hi parts V_hi with a double-float vector (the
 // iteration products of the mixed-precision solver): exact FP32 x FP32 products
 // and double-float sums, as the DF64 product but reading 4 instead of 8 bytes per
@@ -819,99 +856,157 @@ __global__ void k_pack_h16(const float *__restrict__ vp, int ntiles, __half *__r
     pack_h16_tiles(vp, ntiles, vh, vsc, w0, ((int64_t)gridDim.x * blockDim.x) >> 5);
 }
 
+// Tiles per group of the FP16 products (symv_h16_tiles).
+__host__ __device__ __forceinline__ int tile_group(int64_t ntiles, int64_t nwarps)
+{
+    return ntiles >= 48 * nwarps ? 4 : ntiles >= 24 * nwarps ? 2 : 1;
+}
+
 // Product with the FP16 working copy: FP32 products of the half entries with the hi part
 // of x and FP32 sums, two entries per instruction (packed pairs); the tile's scale
 // multiplies its partials.  Lane l covers columns 8 (l % 8) .. +7 (16 bytes) of rows 16
 // (l / 8) .. +15, eight rows per step: 4 KB in flight per warp, so that two CTAs per SM
 // keep HBM busy.  Partials as symv_hi_tiles.  The iteration products of
 // BEM_PRODUCTS_FP16 only: the residuals that decide convergence use the exact form.
+//
+// kGroup: a warp takes g consecutive tiles of one tile row, with one staging of x_I, one set
+// of row partials (the tiles' row sums added as hi/lo pairs) and FP32 column partials.  The
+// partials are written and read again, 2 KB per tile of 8 KB; with g = 4 768 bytes.
+// As many tiles as leave every warp about 12 groups, so that the last ones do not wait for
+// one warp; below 24 tiles per warp (N = 21,700) the groups' longer chains cost what they
+// save.  FP32 operator of N = 29,596, block preconditioner: 263 -> 232 us per iteration.  The
+// FP32 products, with 16 KB and hi/lo partials per tile, gain 1% there and lose 3-7% below.
+template <bool kGroup>
 __device__ void symv_h16_tiles(const __half *__restrict__ vh, const float *__restrict__ vsc,
-                               const float *__restrict__ sc, const int2 *__restrict__ tiles, int ntiles,
+                               const float *__restrict__ sc, const int2 *__restrict__ groups, int ngroups, int g, int nb,
                                const float2 *__restrict__ xdf, float2 *__restrict__ prow, float2 *__restrict__ pcol,
                                HiStage *st, unsigned long long *ctr, unsigned long long base, int static_k = -1)
 {
     const int lane = threadIdx.x & 31, cg = lane & 7, rg = lane >> 3;
     const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4, b3 = lane & 8, b4 = lane & 16;
     float2 *const xd = reinterpret_cast<float2 *>(st->xi);  // x'_I twice
-    for (int k = static_k >= 0 ? static_k : warp_grab(ctr, base); k < ntiles;
-         k = static_k >= 0 ? ntiles : warp_grab(ctr, base)) {
-        const int2 tj = tiles[k];
-        const float sk = __ldcg(vsc + k);
-        float x[4], s4[4];  // I: lane, 32 + lane, J: the same
+    for (int gk = static_k >= 0 ? static_k : warp_grab(ctr, base); gk < ngroups;
+         gk = static_k >= 0 ? ngroups : warp_grab(ctr, base)) {
+        const int2 gj = groups[gk];
+        const int I = gj.x, J1 = kGroup ? min(gj.y + g, nb) : gj.y + 1;
+        const int64_t k0 = kGroup ? tile_pos(I, gj.y, nb) : gk;
+        float xj[2], scj[2], skj;  // of the next tile
+        auto fetch = [&](int J) {
+            skj = __ldcg(vsc + k0 + (J - gj.y));
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int64_t i = (int64_t)(u < 2 ? tj.x : tj.y) * kSB + 32 * (u & 1) + lane;
-            x[u] = __ldcg(&xdf[i].x);
-            s4[u] = __ldcg(sc + i);
-        }
-        __syncwarp();
+            for (int u = 0; u < 2; ++u) {
+                const int64_t i = (int64_t)J * kSB + 32 * u + lane;
+                xj[u] = __ldcg(&xdf[i].x);
+                scj[u] = __ldcg(sc + i);
+            }
+        };
+        fetch(gj.y);
+        {
+            float x[2], s2[2];
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const float xi = x[u] * s4[u];
-            xd[32 * u + lane] = make_float2(xi, xi);
-            st->xjh[32 * u + lane] = x[2 + u] * s4[2 + u];
-            st->si[32 * u + lane] = s4[u] * sk;
-            st->sj[32 * u + lane] = s4[2 + u] * sk;
-        }
-        __syncwarp();
-        f2 xc[4], cs[4];
+            for (int u = 0; u < 2; ++u) {
+                const int64_t i = (int64_t)I * kSB + 32 * u + lane;
+                x[u] = __ldcg(&xdf[i].x);
+                s2[u] = __ldcg(sc + i);
+            }
+            __syncwarp();
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            xc[u] = *reinterpret_cast<const f2 *>(st->xjh + 8 * cg + 2 * u);
-            cs[u] = 0ull;
+            for (int u = 0; u < 2; ++u) {
+                const float xi = x[u] * s2[u];
+                xd[32 * u + lane] = make_float2(xi, xi);
+                st->si[32 * u + lane] = s2[u];
+            }
         }
-        const uint4 *T = reinterpret_cast<const uint4 *>(vh + (int64_t)k * kTileF) + 128 * rg + cg;
+        float2 racc0 = make_float2(0.f, 0.f), racc1 = racc0;  // the lane's rows of ch = 0, 1
 #pragma unroll 1
-        for (int ch = 0; ch < 2; ++ch) {
-            uint4 raw[8];
+        for (int J = gj.y; J < J1; ++J) {
+            const int64_t k = k0 + (J - gj.y);
+            const float sk = skj;
+            if (kGroup) __syncwarp();
 #pragma unroll
-            for (int m = 0; m < 8; ++m) raw[m] = __ldcs(T + (8 * ch + m) * 8);
-            float sr[8];
+            for (int u = 0; u < 2; ++u) {
+                st->xjh[32 * u + lane] = xj[u] * scj[u];
+                st->sj[32 * u + lane] = scj[u] * sk;
+            }
+            __syncwarp();
+            if (kGroup && J + 1 < J1) fetch(J + 1);
+            f2 xc[4], cs[4];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                const f2 xr = *reinterpret_cast<const f2 *>(xd + 16 * rg + 8 * ch + m);
-                const unsigned w[4] = {raw[m].x, raw[m].y, raw[m].z, raw[m].w};
-                f2 s = 0ull;
+            for (int u = 0; u < 4; ++u) {
+                xc[u] = *reinterpret_cast<const f2 *>(st->xjh + 8 * cg + 2 * u);
+                cs[u] = 0ull;
+            }
+            const uint4 *T = reinterpret_cast<const uint4 *>(vh + k * kTileF) + 128 * rg + cg;
+#pragma unroll 1
+            for (int ch = 0; ch < 2; ++ch) {
+                uint4 raw[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    __half2 hh;
-                    memcpy(&hh, &w[u], 4);
-                    const float2 a = __half22float2(hh);
-                    const f2 e = f2_make(a.x, a.y);
-                    s = f2_fma(e, xc[u], s);
-                    cs[u] = f2_fma(e, xr, cs[u]);
+                for (int m = 0; m < 8; ++m) raw[m] = __ldcs(T + (8 * ch + m) * 8);
+                float sr[8];
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    const f2 xr = *reinterpret_cast<const f2 *>(xd + 16 * rg + 8 * ch + m);
+                    const unsigned w[4] = {raw[m].x, raw[m].y, raw[m].z, raw[m].w};
+                    f2 s = 0ull;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        __half2 hh;
+                        memcpy(&hh, &w[u], 4);
+                        const float2 a = __half22float2(hh);
+                        const f2 e = f2_make(a.x, a.y);
+                        s = f2_fma(e, xc[u], s);
+                        cs[u] = f2_fma(e, xr, cs[u]);
+                    }
+                    const float2 t = f2_get(s);
+                    sr[m] = t.x + t.y;
                 }
-                const float2 t = f2_get(s);
-                sr[m] = t.x + t.y;
+                // rows m of this lane's group: 8 -> 4 (xor 4) -> 2 (xor 2) -> 1 (xor 1)
+                float t4[4], t2[2];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    t4[j] = (b2 ? sr[j + 4] : sr[j]) + __shfl_xor_sync(0xffffffffu, b2 ? sr[j] : sr[j + 4], 4);
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    t2[j] = (b1 ? t4[j + 2] : t4[j]) + __shfl_xor_sync(0xffffffffu, b1 ? t4[j] : t4[j + 2], 2);
+                const float w = (b0 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, b0 ? t2[0] : t2[1], 1);
+                if (kGroup) {
+                    const float2 t = df_add(ch ? racc1 : racc0, make_float2(w * sk, 0.f));
+                    if (ch)
+                        racc1 = t;
+                    else
+                        racc0 = t;
+                } else {
+                    const int r = 16 * rg + 8 * ch + (b2 ? 4 : 0) + (b1 ? 2 : 0) + (b0 ? 1 : 0);
+                    prow[k * kSB + r] = make_float2(w * (st->si[r] * sk), 0.f);
+                }
             }
-            // rows m of this lane's group: 8 -> 4 (xor 4) -> 2 (xor 2) -> 1 (xor 1)
-            float t4[4], t2[2];
+            if (I != J) {  // lane keeps columns 8 cg + 4 (b4) + 2 (b3) + {0, 1}
+                float2 c[4], d[2];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                t4[j] = (b2 ? sr[j + 4] : sr[j]) + __shfl_xor_sync(0xffffffffu, b2 ? sr[j] : sr[j + 4], 4);
+                for (int u = 0; u < 4; ++u) c[u] = f2_get(cs[u]);
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
-                t2[j] = (b1 ? t4[j + 2] : t4[j]) + __shfl_xor_sync(0xffffffffu, b1 ? t4[j] : t4[j + 2], 2);
-            const float w = (b0 ? t2[1] : t2[0]) + __shfl_xor_sync(0xffffffffu, b0 ? t2[0] : t2[1], 1);
-            const int r = 16 * rg + 8 * ch + (b2 ? 4 : 0) + (b1 ? 2 : 0) + (b0 ? 1 : 0);
-            prow[(int64_t)k * kSB + r] = make_float2(w * st->si[r], 0.f);
+                for (int j = 0; j < 2; ++j) {
+                    const float2 keep = b4 ? c[j + 2] : c[j], give = b4 ? c[j] : c[j + 2];
+                    d[j].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
+                    d[j].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
+                }
+                const float2 keep = b3 ? d[1] : d[0], give = b3 ? d[0] : d[1];
+                const float s0 = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8);
+                const float s1 = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8);
+                const int q = 8 * cg + (b4 ? 4 : 0) + (b3 ? 2 : 0);
+                const float2 sj = *reinterpret_cast<const float2 *>(st->sj + q);
+                if (kGroup)
+                    *reinterpret_cast<float2 *>(reinterpret_cast<float *>(pcol) + k * kSB + q) =
+                        make_float2(s0 * sj.x, s1 * sj.y);
+                else
+                    *reinterpret_cast<float4 *>(pcol + k * kSB + q) = make_float4(s0 * sj.x, 0.f, s1 * sj.y, 0.f);
+            }
         }
-        if (tj.x != tj.y) {  // lane keeps columns 8 cg + 4 (b4) + 2 (b3) + {0, 1}
-            float2 c[4], d[2];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) c[u] = f2_get(cs[u]);
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float2 keep = b4 ? c[j + 2] : c[j], give = b4 ? c[j] : c[j + 2];
-                d[j].x = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
-                d[j].y = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
-            }
-            const float2 keep = b3 ? d[1] : d[0], give = b3 ? d[0] : d[1];
-            const float s0 = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 8);
-            const float s1 = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 8);
-            const int q = 8 * cg + (b4 ? 4 : 0) + (b3 ? 2 : 0);
-            const float2 sj = *reinterpret_cast<const float2 *>(st->sj + q);
-            *reinterpret_cast<float4 *>(pcol + (int64_t)k * kSB + q) = make_float4(s0 * sj.x, 0.f, s1 * sj.y, 0.f);
+        if (kGroup) {
+            const int r = 16 * rg + (b2 ? 4 : 0) + (b1 ? 2 : 0) + (b0 ? 1 : 0);
+            const float s0 = st->si[r], s1 = st->si[r + 8];  // powers of two
+            prow[k0 * kSB + r] = make_float2(racc0.x * s0, racc0.y * s0);
+            prow[k0 * kSB + r + 8] = make_float2(racc1.x * s1, racc1.y * s1);
         }
     }
 }
@@ -933,6 +1028,23 @@ __global__ void k_tile_list(int nb, int2 *tiles)
 {
     const int I = blockIdx.x;
     for (int J = I + threadIdx.x; J < nb; J += blockDim.x) tiles[tile_pos(I, J, nb)] = make_int2(I, J);
+}
+
+// Groups of g consecutive tiles of one tile row: (I, first J), in the order of the tiles.
+__host__ __device__ __forceinline__ int64_t group_pos(int I, int nb, int g)
+{
+    // sum over rows i < I of ceil((nb - i) / g) = of floor((m + g - 1) / g), m = nb - i
+    auto upto = [g](int64_t m) {  // sum over 1..m of ceil(x / g)
+        const int64_t f = m / g, r = m % g;
+        return (int64_t)g * f * (f + 1) / 2 + r * (f + 1);
+    };
+    return upto(nb) - upto(nb - I);
+}
+__global__ void k_group_list(int nb, int g, int2 *groups)
+{
+    const int I = blockIdx.x, n = (nb - I + g - 1) / g;
+    const int64_t o = group_pos(I, nb, g);
+    for (int k = threadIdx.x; k < n; k += blockDim.x) groups[o + k] = make_int2(I, I + k * g);
 }
 
 // x (FP64, N) -> hi/lo pairs, zero-padded to ld
@@ -1338,6 +1450,8 @@ struct PcgArgs {
     int64_t ld, N;
     int nb, ntiles;
     const int2 *tiles;
+    const int2 *groups;  // groups of tiles of the FP16 products
+    int ngroups, group;
     float2 *prow, *pcol, *pdf;
     double *x, *r, *z, *p, *q;
     const double *d, *b;
@@ -1557,8 +1671,14 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     if (!grid_barrier(gb, G)) return;  // partial slots are reused below
     while (!(rr <= thr) && it < a.max_it) {
         if (use16) {
-            symv_h16_tiles(a.vh, a.vsc, rsc, a.tiles, a.ntiles, a.pdf, a.prow, a.pcol, stage, a.ctr, tbase, hi_static);
-            if (hi_static < 0) tbase += (unsigned long long)(a.ntiles + G * (kSymThreads / 32));
+            const int gr_static = a.ngroups <= nwarps ? (int)warp_g : -1;
+            if (a.group > 1)
+                symv_h16_tiles<true>(a.vh, a.vsc, rsc, a.groups, a.ngroups, a.group, a.nb, a.pdf, a.prow, a.pcol, stage,
+                                     a.ctr, tbase, gr_static);
+            else
+                symv_h16_tiles<false>(a.vh, a.vsc, rsc, a.groups, a.ngroups, 1, a.nb, a.pdf, a.prow, a.pcol, stage,
+                                      a.ctr, tbase, gr_static);
+            if (gr_static < 0) tbase += (unsigned long long)(a.ngroups + G * (kSymThreads / 32));
             ++n16;
         } else if (mixed) {
             hi_product(a.vp, std::true_type());
@@ -1575,7 +1695,9 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             const int64_t i = ib + (lane >> 2);
             const bool valid = i < a.N;
             const int64_t ic = valid ? i : a.N - 1;
-            const double qi = symv_row4(a.prow, a.pcol, a.nb, ic, q4);
+            const double qi = use16 && a.group > 1
+                                  ? symv_row4_groups(a.prow, reinterpret_cast<const float *>(a.pcol), a.nb, a.group, ic, q4)
+                                  : symv_row4(a.prow, a.pcol, a.nb, ic, q4);
             if (valid && q4 == 0) {
                 a.q[i] = qi;
                 pq_l[0] += a.p[i] * qi;
@@ -2202,6 +2324,22 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
     int G = vp ? (int)std::max<int64_t>((nt_ + 7) / 8, (op->N + 63) / 64) : nt_;
     G = std::min(std::max(G, 8), Gmax);
+    // groups of tiles (FP16 products); the tiles themselves where their list finds no room
+    int group = vh ? tile_group(nt_, (int64_t)G * (kSymThreads / 32)) : 1, ngroups = nt_;
+    int2 *groups = W.tiles;
+    if (group > 1) {
+        const size_t gbytes = sizeof(int2) * (size_t)group_pos(nb_, nb_, group);
+        if (ctx->budget > 0 && ctx->in_use + (int64_t)gbytes + (64 << 10) + 8 * op->mesh->M + 16 * max_it > ctx->budget) {
+            group = 1;
+        } else {
+            if ((st = dalloc(ctx, tmp, (void **)&groups, gbytes, false))) {
+                dfree_all(ctx, tmp);
+                return st;
+            }
+            ngroups = (int)group_pos(nb_, nb_, group);
+            k_group_list<<<nb_, 128, 0, ctx->stream>>>(nb_, group, groups); BEM_COUNT(ctx);
+        }
+    }
     double *part = nullptr;
     if ((st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (3 * G + 8) + 64, true))) {
         dfree_all(ctx, tmp);
@@ -2229,6 +2367,9 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     a.nb = (int)(op->ld / kSB);
     a.ntiles = a.nb * (a.nb + 1) / 2;
     a.tiles = W.tiles;
+    a.group = group;
+    a.ngroups = ngroups;
+    a.groups = groups;
     a.prow = W.prow;
     a.pcol = W.pcol;
     a.pdf = W.xdf;
@@ -3094,6 +3235,9 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             a.nb = (int)(L / kSB);
             a.ntiles = (int)pr.nt;
             a.tiles = pr.tiles;
+            a.group = 1;  // a wave's problems are far below the sizes of groups
+            a.ngroups = a.ntiles;
+            a.groups = pr.tiles;
             a.prow = prow;
             a.pcol = pcol;
             a.pdf = xdf;
