@@ -251,7 +251,7 @@ bem_status matvec_f64(bem_operator *op, const double *x, double *y);
 // How the algorithmic bytes of a persistent solve are counted once its counts are read.
 struct PersistentRun {
     int prof = -1;  // profiler record of the launch
-    bool f32op = false, mixed = false, calpc = false, h16 = false, f64 = false;
+    bool f32op = false, mixed = false, calpc = false, h16 = false, f64 = false, resident = false;
     double n2 = 0.0;  // N^2
 };
 // A solve whose results are still travelling to pinned host memory: solve_capacity

@@ -1966,6 +1966,294 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
     }
 }
 
+// Small solves (N <= 16 x SMs): the operator stays in shared memory for the whole solve.  CTA
+// 4 k + s owns rows 16 s .. + 15 of the cluster k of 64 rows (the block preconditioner's, else
+// 64 consecutive rows) and holds them whole, 16 x ld FP32 entries (hi parts of a DF64
+// operator: 152 KB at N = 2,432).  Every CTA keeps the whole direction p, each thread its columns
+// in registers, so an iteration has two grid barriers instead of four: q = V p of the own
+// rows and p.q; then r of the cluster's 64 rows (each of its four CTAs updates a copy), z of
+// the own rows, r.z and r.r; then p = z + beta p everywhere.  Products are exact FP32
+// products with two-sums (two_sum_acc), which costs little here: what bounds an iteration is
+// the latency of two barriers, of the loads that follow them and of chains of FP64 operations
+// (sums as trees, loads in flight together, reciprocals off the chains: 18 -> 13 us at N =
+// 2,352).  Per iteration, DF64, Jacobi / block: N = 604 20 / 22 -> 10 / 11 us, N = 1,200 21 /
+// 23 -> 12 / 13, N = 2,352 22 / 25 -> 13 / 14.  The line lies where the rows no longer fit: at N =
+// 2,700 the tiled solver takes 20 / 23 us.
+constexpr int kResRows = 16;
+constexpr int kResThreads = 512;
+constexpr int kResWarps = kResThreads / 32;
+constexpr int kResMaxCtas = 160;  // five partials per lane, 160 KB of rows
+
+// df_from_double by integer operations: the FP64 pipe converts two values per clock and SM.
+// Rounds hi to nearest (ties away from zero).
+__device__ __forceinline__ float2 df_split(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    if (e < 949 || e > 1149) return v == 0.0 ? make_float2(0.f, 0.f) : df_from_double(v);
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const unsigned long long m = (b & 0x7fffffffffffffffull) + (1ull << 28);
+    const float hi = __uint_as_float(sign | (unsigned)((m >> 29) - (896ull << 23)));
+    const int rest = ((int)((unsigned)b << 3)) >> 3;  // the low 29 bits, signed: v - hi in units of 2^(e - 1075)
+    return make_float2(hi, (float)rest * __uint_as_float(sign | (unsigned)(e - 948) << 23));
+}
+
+template <class T, int P>  // P = ceil(ld / 1024): pairs of columns per thread
+__global__ void __launch_bounds__(kResThreads, 1) k_pcg_res(PcgArgs a)
+{
+    static_assert(kBJ == 64 && kResWarps == kResRows, "four CTAs per cluster, a warp per row");
+    extern __shared__ float vs[];
+    __shared__ float2 part[kResRows][kResWarps + 1];
+    __shared__ double rs[kBJ], zs[kResRows], tots[2];
+    __shared__ int32_t gi[kBJ];
+    const int G = gridDim.x, cta = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int blk = cta >> 2, r0 = kResRows * (cta & 3), ld = (int)a.ld, np = ld / 2;
+    const bool blockpc = a.precond == BEM_PRECOND_BLOCK, jacobi = a.precond == BEM_PRECOND_JACOBI;
+    const T *const V = reinterpret_cast<const T *>(a.V);
+    double *const pA = a.part, *const pB = a.part + G, *const pC = a.part + 3 * G;
+    GridBar gb{a.bar, a.err, 0u, a.bar_limit_ns > 0 ? a.bar_limit_ns : kBarrierLimitNs, a.absent_cta == cta};
+    if (t < kBJ) {
+        const int64_t i = (int64_t)blk * kBJ + t;
+        gi[t] = blockpc ? a.bperm[i] : i < a.N ? (int32_t)i : -1;
+    }
+    __syncthreads();
+    const int grow = t < kBJ ? gi[t] : -1;                     // row of the cluster of this thread
+    const int gz = gi[r0 + w];                                 // row of this warp
+    const int own = w == 0 ? gi[r0 + (lane >> 1)] : -1;        // row of this pair of lanes of warp 0
+    // hi and lo parts of columns 2 c, 2 c + 1 of row g
+    auto entries = [&](int g, int c, f2 &hi, f2 &lo) {
+        if constexpr (sizeof(T) == 8) {
+            const float4 e = g < 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                                   : __ldg(reinterpret_cast<const float4 *>(V + (int64_t)g * ld) + c);
+            hi = f2_make(e.x, e.z);
+            lo = f2_make(e.y, e.w);
+        } else {
+            const float2 e = g < 0 ? make_float2(0.f, 0.f) : __ldg(reinterpret_cast<const float2 *>(V + (int64_t)g * ld) + c);
+            hi = f2_make(e.x, e.y);
+            lo = 0ull;
+        }
+    };
+#pragma unroll 4
+    for (int r = 0; r < kResRows; ++r)
+        for (int c = t; c < np; c += kResThreads) {
+            f2 hi, lo;
+            entries(gi[r0 + r], c, hi, lo);
+            *reinterpret_cast<f2 *>(vs + r * ld + 2 * c) = hi;
+        }
+    double m0 = 0.0, m1 = 0.0;  // row 16 s + w of the cluster's inverse block
+    if (blockpc) {
+        const double *Mi = a.binv + (int64_t)blk * kBJ * kBJ + (r0 + w) * kBJ;
+        m0 = Mi[lane];
+        m1 = Mi[lane + 32];
+    }
+    const double dz = jacobi && gz >= 0 ? 1.0 / a.d[gz] : 1.0;
+    double p[P][2];
+    f2 xh[P], xl[P];
+    __syncthreads();
+
+    // (V x) of row own, x in (xh, xl): the resident hi parts, or (kDf) all of V
+    auto product = [&](auto df) -> double {
+        constexpr bool kDf = decltype(df)::value;
+#pragma unroll 1
+        for (int h = 0; h < kResRows; h += 8) {
+            f2 s[8], l[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) s[r] = l[r] = 0ull;
+#pragma unroll
+            for (int m = 0; m < P; ++m) {
+                const int c = t + kResThreads * m;
+                if (c >= np) continue;  // uniform in the warp: ld is a multiple of 64
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    f2 v, vl = 0ull;
+                    if (kDf)
+                        entries(gi[r0 + h + r], c, v, vl);
+                    else
+                        v = *reinterpret_cast<const f2 *>(vs + (h + r) * ld + 2 * c);
+                    two_sum_acc(s[r], l[r], v, xh[m], xl[m]);
+                    if (kDf) l[r] = f2_fma(vl, xh[m], l[r]);
+                }
+            }
+            float2 u[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                const float2 x = f2_get(s[r]), y = f2_get(l[r]);
+                u[r] = df_add_u(make_float2(x.x, y.x), make_float2(x.y, y.y));
+            }
+            // rows 8 -> 4 (xor 16) -> 2 (xor 8) -> 1 (xor 4), then xor 2, 1
+            const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) u[j] = df_add_u(b4 ? u[j + 4] : u[j], shfl_df(b4 ? u[j] : u[j + 4], 16));
+#pragma unroll
+            for (int j = 0; j < 2; ++j) u[j] = df_add_u(b3 ? u[j + 2] : u[j], shfl_df(b3 ? u[j] : u[j + 2], 8));
+            float2 z = df_add_u(b2 ? u[1] : u[0], shfl_df(b2 ? u[0] : u[1], 4));
+            z = df_add_u(z, shfl_df(z, 2));
+            z = df_add(z, shfl_df(z, 1));
+            if ((lane & 3) == 0) part[h + (lane >> 2 & 1) + (b3 ? 2 : 0) + (b4 ? 4 : 0)][w] = z;
+        }
+        __syncthreads();
+        if (w > 0) return 0.0;
+        const float2 *q = part[lane >> 1] + 8 * (lane & 1);
+        float2 v = df_add_u(df_add_u(df_add_u(q[0], q[1]), df_add_u(q[2], q[3])),
+                            df_add_u(df_add_u(q[4], q[5]), df_add_u(q[6], q[7])));
+        const float2 o = shfl_df(v, 1);
+        v = lane & 1 ? df_add(o, v) : df_add(v, o);
+        return df_to_double(v);
+    };
+    // fixed-order sum of the G <= kResMaxCtas partials of one value, by a warp
+    auto total = [&](const double *slot) {
+        double v[5];
+#pragma unroll
+        for (int u = 0; u < 5; ++u) v[u] = lane + 32 * u < G ? __ldcg(slot + lane + 32 * u) : 0.0;
+        return warp_sum(((v[0] + v[1]) + (v[2] + v[3])) + v[4]);
+    };
+    // z = M^-1 r of the own rows and the partials of r.z and r.r; r by threads 0 .. 63
+    auto apply = [&](double r) {
+        if (t < kBJ) rs[t] = r;
+        __syncthreads();
+        double z;
+        if (blockpc)
+            z = warp_sum(m0 * rs[lane] + m1 * rs[lane + 32]);
+        else
+            z = rs[r0 + w] * dz;
+        if (lane == 0) {
+            zs[w] = gz >= 0 ? z : 0.0;
+            if (gz >= 0) a.z[gz] = z;
+        }
+        __syncthreads();
+        if (w < 2) {  // warp 0: r.z, warp 1: r.r
+            const double ri = lane < kResRows ? rs[r0 + lane] : 0.0;
+            const double v = warp_sum(ri * (w ? ri : zs[lane & (kResRows - 1)]));
+            if (lane == 0) pB[w * G + cta] = v;
+        }
+    };
+    // all of a vector, this thread's columns
+    auto load = [&](const double *v, double (&d)[P][2]) {
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            const int c = 2 * (t + kResThreads * m);
+            d[m][0] = c < a.N ? __ldcg(v + c) : 0.0;
+            d[m][1] = c + 1 < a.N ? __ldcg(v + c + 1) : 0.0;
+        }
+    };
+    auto split = [&](const double (&d)[P][2]) {
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            const float2 u = df_split(d[m][0]), v = df_split(d[m][1]);
+            xh[m] = f2_make(u.x, v.x);
+            xl[m] = f2_make(u.y, v.y);
+        }
+    };
+    const double bown = own >= 0 ? a.b[own] : 0.0;
+    double xown = own >= 0 && a.has_x0 ? a.x[own] : 0.0, pown, z[P][2];
+    double r = grow >= 0 ? a.b[grow] : 0.0;
+    // r = b - V x of the cluster's rows, x as every CTA left it in memory
+    auto residual = [&]() -> bool {
+        double x[P][2];
+        load(a.x, x);
+        split(x);
+        const double v = product(std::bool_constant<sizeof(T) == 8>());
+        if (own >= 0 && !(lane & 1)) a.r[own] = bown - v;
+        if (!grid_barrier(gb, G)) return false;
+        r = grow >= 0 ? __ldcg(a.r + grow) : 0.0;
+        return true;
+    };
+    // r.z, r.r and z after the barrier that follows apply
+    auto totals = [&]() {
+        load(a.z, z);
+        if (w < 2) {
+            const double v = total(pB + w * G);
+            if (lane == 0) tots[w] = v;
+        }
+        __syncthreads();
+    };
+    if (a.has_x0 && !residual()) return;
+    apply(r);
+    if (w == 0) {
+        const double bb = warp_sum(lane & 1 ? 0.0 : bown * bown);
+        if (lane == 0) pC[cta] = bb;
+    }
+    if (!grid_barrier(gb, G)) return;
+    const double bb = total(pC), thr = a.tol * a.tol * (bb > 0.0 ? bb : 1.0);
+    totals();
+    double rz = tots[0], rr = tots[1], rr_true = rr;
+#pragma unroll
+    for (int m = 0; m < P; ++m) {
+        p[m][0] = z[m][0];
+        p[m][1] = z[m][1];
+    }
+    pown = zs[lane >> 1];
+    split(p);
+    int it = 0, ndf = 1;
+    bool done = rr <= thr;  // of a residual formed from x
+    while (!done && it < a.max_it) {
+        const double irz = 1.0 / rz;  // not in the chain from r.z to beta
+        const double q = product(std::false_type());
+        if (w == 0) {
+            const bool on = own >= 0 && !(lane & 1);
+            if (on) a.q[own] = q;
+            const double pq = warp_sum(on ? pown * q : 0.0);
+            if (lane == 0) pA[cta] = pq;
+        }
+        if (!grid_barrier(gb, G)) return;
+        double alpha = 0.0;
+        if (w < 2) {
+            const double qg = grow >= 0 ? __ldcg(a.q + grow) : 0.0;
+            alpha = rz / total(pA);
+            r -= alpha * qg;
+            xown += alpha * pown;  // warp 0
+        }
+        apply(r);
+        if (!grid_barrier(gb, G)) return;
+        totals();
+        rr = tots[1];
+        ++it;
+        // reliable update, as in pcg_body, but for convergence only at half the tolerance: one
+        // more iteration of about 70, and the confirmed residual stays below the tolerance
+        if (rr <= a.delta2 * rr_true || rr <= 0.25 * thr || (rr <= thr && it == a.max_it)) {
+            if (own >= 0 && !(lane & 1)) a.x[own] = xown;
+            if (!grid_barrier(gb, G)) return;
+            if (!residual()) return;
+            apply(r);
+            if (!grid_barrier(gb, G)) return;
+            totals();
+            rr = rr_true = tots[1];
+            ++ndf;
+            done = rr <= thr;
+        }
+        const double beta = tots[0] * irz;
+        if (a.lanczos && cta == 0 && t == 0 && it - 1 < a.lanczos_cap) {
+            a.lanczos[2 * (it - 1)] = alpha;
+            a.lanczos[2 * (it - 1) + 1] = beta;
+        }
+        rz = tots[0];
+#pragma unroll
+        for (int m = 0; m < P; ++m) {
+            p[m][0] = fma(beta, p[m][0], z[m][0]);
+            p[m][1] = fma(beta, p[m][1], z[m][1]);
+        }
+        pown = fma(beta, pown, zs[lane >> 1]);
+        split(p);
+    }
+    if (own >= 0 && !(lane & 1)) a.x[own] = xown;
+    if (cta == 0 && t == 0) {
+        a.out[0] = rr;
+        a.out[1] = bb;
+        a.out[2] = (double)it;
+        a.out[3] = (double)ndf;
+        a.out[4] = 0.0;
+        a.n16_out[0] = 0.0;
+    }
+}
+
+template <class T>
+static const void *res_kernel(int64_t ld)
+{
+    return ld <= 2 * kResThreads   ? (const void *)k_pcg_res<T, 1>
+           : ld <= 4 * kResThreads ? (const void *)k_pcg_res<T, 2>
+                                   : (const void *)k_pcg_res<T, 3>;
+}
+
 // ------------------------------------------------------------------ host side
 struct Work {
     double *r, *z, *p, *q, *b, *x, *d;  // vectors of length ld
@@ -2238,6 +2526,10 @@ static bem_status persistent_results(bem_ctx *ctx, const double *h, const Persis
         prof_set_units(ctx, r.prof, 8.0 * n2 * h[3]);
         return BEM_OK;
     }
+    if (r.resident) {  // V read once into shared memory, DF64 residuals from memory
+        prof_set_units(ctx, r.prof, r.f32op ? 4.0 * n2 : 8.0 * n2 * h[3]);
+        return BEM_OK;
+    }
     const double i16 = r.h16 ? h[7] : 0.0, i32 = h[2] - i16;
     const double bytes = (r.f32op  ? 2.0 * n2 * (i32 + h[3]) + n2 * i16
                           : r.mixed ? 4.0 * n2 * h[3] + 2.0 * n2 * (i32 + 1.0) + n2 * i16 + (r.h16 ? 3.0 * n2 : 0.0)
@@ -2264,19 +2556,36 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     if (!coop || !W.tiles) return BEM_OK;
     if (f32op) delta = 1.0;  // a packed copy is needed; residuals are replaced only at convergence
     const int nb_ = (int)(op->ld / kSB), nt_ = nb_ * (nb_ + 1) / 2;
-    const void *kern = precond == BEM_PRECOND_CALDERON ? (const void *)k_pcg_cal : (const void *)k_pcg_df;
-    BEM_CK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSymSmem));
-    BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kSymThreads, kSymSmem));
-    if (per_sm < 1) return BEM_OK;
     Allocs tmp;
     bem_status st = BEM_OK;
     float *vp = nullptr;
-    if (delta > 0.0) {
-        const size_t vbytes = packed_bytes((size_t)nt_, (size_t)op->ld);
-        if (ctx->budget <= 0 || ctx->in_use + (int64_t)vbytes + (64 << 10) <= ctx->budget)
-            if ((st = dalloc(ctx, tmp, (void **)&vp, vbytes, false))) return st;
+    const size_t vbytes = packed_bytes((size_t)nt_, (size_t)op->ld);
+    const bool room = delta > 0.0 && (ctx->budget <= 0 || ctx->in_use + (int64_t)vbytes + (64 << 10) <= ctx->budget);
+    if (f32op && !room) return BEM_OK;  // no room for the packed copy: host-driven refinement
+    // resident solver: whole rows of FP32 entries in shared memory, four CTAs per 64 rows
+    const void *kern = f32op ? res_kernel<float>(op->ld) : res_kernel<float2>(op->ld);
+    size_t smem = sizeof(float) * kResRows * (size_t)op->ld;
+    int threads = kResThreads;
+    const int rG = (int)((op->N + kBJ - 1) / kBJ * (kBJ / kResRows));
+    bool resident = room && rG <= kResMaxCtas && precond != BEM_PRECOND_CALDERON && !(inexact_lambda > 0.0) && rG <= ctx->sm_count;
+    if (resident) {
+        // the most that any solve asks of the kernel, whatever another thread sets meanwhile
+        const size_t most = sizeof(float) * kResRows * (kResMaxCtas / (kBJ / kResRows)) * kBJ;
+        BEM_CK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
+        BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+        resident = per_sm >= 1;
     }
-    if (f32op && !vp) return BEM_OK;  // no room for the packed copy: host-driven refinement
+    if (resident) {
+        if ((st = ensure_full(op))) return st;
+    } else {
+        kern = precond == BEM_PRECOND_CALDERON ? (const void *)k_pcg_cal : (const void *)k_pcg_df;
+        smem = kSymSmem;
+        threads = kSymThreads;
+        BEM_CK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem));
+        if (per_sm < 1) return BEM_OK;
+        if (room && (st = dalloc(ctx, tmp, (void **)&vp, vbytes, false))) return st;
+    }
     auto pack = [&](const float *V, float *to) {  // a packed copy of an FP32 matrix
         k_tile_scale<<<nblk(op->ld, 256), 256, 0, ctx->stream>>>(V, op->ld, op->N, packed_scale(to, (size_t)nt_));
         BEM_COUNT(ctx);
@@ -2292,7 +2601,7 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
         }
         pack(op->cal_C, dvp);
     }
-    if (f32op) {
+    if (f32op && vp) {
         pack((const float *)op->V, vp);
     }
     // FP16 working copy for the iteration products (N^2 bytes and a scale per tile)
@@ -2323,7 +2632,7 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     // products one tile per warp (8 per CTA), its row passes 8 rows per warp.
     const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
     int G = vp ? (int)std::max<int64_t>((nt_ + 7) / 8, (op->N + 63) / 64) : nt_;
-    G = std::min(std::max(G, 8), Gmax);
+    G = resident ? rG : std::min(std::max(G, 8), Gmax);
     // groups of tiles (FP16 products); the tiles themselves where their list finds no room
     int group = vh ? tile_group(nt_, (int64_t)G * (kSymThreads / 32)) : 1, ngroups = nt_;
     int2 *groups = W.tiles;
@@ -2341,11 +2650,11 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
         }
     }
     double *part = nullptr;
-    if ((st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (3 * G + 8) + 64, true))) {
+    if ((st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (4 * G + 8) + 64, true))) {
         dfree_all(ctx, tmp);
         return st;
     }
-    double *out = part + 3 * G;  // [0..4]: r.r, b.b, iterations, DF64 residuals, inexact stop
+    double *out = part + 4 * G;  // [0..4]: r.r, b.b, iterations, DF64 residuals, inexact stop
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(out + 6);
     unsigned *bar = reinterpret_cast<unsigned *>(ctr + 1);
     int *err = reinterpret_cast<int *>(bar + 2);
@@ -2413,8 +2722,7 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     a.absent_cta = ctx->bar_absent_cta < G ? ctx->bar_absent_cta : -1;
     void *args[] = {&a};
     const int prof = prof_start(ctx, BEM_KERNEL_MATVEC, 0.0);
-    cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(G), dim3(kSymThreads), args, kSymSmem,
-                                                ctx->stream);
+    cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3(G), dim3(threads), args, smem, ctx->stream);
     BEM_COUNT(ctx);
     prof_stop(ctx, prof);
     if (e != cudaSuccess) {
@@ -2429,7 +2737,8 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     PersistentRun run;
     run.prof = prof;
     run.f32op = f32op;
-    run.mixed = vp != nullptr;
+    run.mixed = room;
+    run.resident = resident;
     run.calpc = calpc;
     run.n2 = (double)op->N * (double)op->N;
     run.h16 = vh != nullptr;
