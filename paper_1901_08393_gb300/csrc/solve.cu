@@ -1522,16 +1522,14 @@ __device__ __forceinline__ void grid_totals(const double *slot, int G, double (&
     if (w < n) {
         const double *p = slot + (int64_t)w * G;
         double v = 0.0;
-        for (int k0 = 0; k0 < G; k0 += 256) {  // eight loads in flight
-            double t[8];
+        for (int k0 = 0; k0 < G; k0 += 320) {  // ten loads in flight (G <= 304), a tree of sums
+            double t[10];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < 10; ++u) {
                 const int k = k0 + 32 * u + lane;
                 t[u] = k < G ? __ldcg(p + k) : 0.0;
             }
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (k0 + 32 * u < G) v += t[u];
+            v += (((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]))) + (t[8] + t[9]);
         }
         v = warp_sum(v);
         if (lane == 0) res[w] = v;
@@ -1540,6 +1538,20 @@ __device__ __forceinline__ void grid_totals(const double *slot, int G, double (&
 #pragma unroll
     for (int j = 0; j < n; ++j) r[j] = res[j];
     __syncthreads();  // res is rewritten by the next call
+}
+
+// df_from_double by integer operations: the FP64 pipe converts two values per clock and SM.
+// Rounds hi to nearest (ties away from zero).
+__device__ __forceinline__ float2 df_split(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const int e = (int)(b >> 52) & 0x7ff;
+    if (e < 949 || e > 1149) return v == 0.0 ? make_float2(0.f, 0.f) : df_from_double(v);
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const unsigned long long m = (b & 0x7fffffffffffffffull) + (1ull << 28);
+    const float hi = __uint_as_float(sign | (unsigned)((m >> 29) - (896ull << 23)));
+    const int rest = ((int)((unsigned)b << 3)) >> 3;  // the low 29 bits, signed: v - hi in units of 2^(e - 1075)
+    return make_float2(hi, (float)rest * __uint_as_float(sign | (unsigned)(e - 948) << 23));
 }
 
 // CTAs per SM of the persistent solvers: 16 warps of 128 registers keep as many bytes in
@@ -1629,6 +1641,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
         if (!grid_barrier(gb, G)) return;
     }
     int n16 = 0, seg = 0;
+    const double dinv = jacobi && i0 < a.N ? 1.0 / a.d[i0] : 1.0;  // of the thread's first row, mostly its only one
     double sums[2] = {0.0, 0.0}, bb_l[1] = {0.0};  // r.z, r.r
     for (int64_t i = i0; i < a.ld; i += stride) {
         if (i < a.N) {
@@ -1670,6 +1683,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     int it = 0, ndf = prod0 ? 1 : 0, inexact_stop = 0;
     if (!grid_barrier(gb, G)) return;  // partial slots are reused below
     while (!(rr <= thr) && it < a.max_it) {
+        const double irz = 1.0 / rz;  // not in the chain from r.z to beta
         if (use16) {
             const int gr_static = a.ngroups <= nwarps ? (int)warp_g : -1;
             if (a.group > 1)
@@ -1723,7 +1737,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             for (int64_t i = i0; i < a.N; i += stride) {
                 a.x[i] += alpha * a.p[i];
                 const double ri = a.r[i] - alpha * a.q[i];
-                const double zi = jacobi ? ri / a.d[i] : ri;
+                const double zi = !jacobi ? ri : i == i0 ? ri * dinv : ri / a.d[i];
                 a.r[i] = ri;
                 a.z[i] = zi;
                 sums[0] += ri * zi;
@@ -1805,7 +1819,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             ++ndf;
             if (use16 && rr_true > kH16Progress * rr_true_prev) use16 = false;  // the same in every CTA
         }
-        const double beta = tot[0] / rz;
+        const double beta = tot[0] * irz;
         if (a.lanczos && cta == 0 && threadIdx.x == 0 && it - 1 < a.lanczos_cap) {
             a.lanczos[2 * (it - 1)] = alpha;
             a.lanczos[2 * (it - 1) + 1] = beta;
@@ -1814,7 +1828,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
         for (int64_t i = i0; i < a.N; i += stride) {
             const double pi = a.z[i] + beta * a.p[i];
             a.p[i] = pi;
-            a.pdf[i] = df_from_double(pi);
+            a.pdf[i] = df_split(pi);
         }
         if (!grid_barrier(gb, G)) return;
     }
@@ -1891,15 +1905,15 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
             const double2 *r = reinterpret_cast<const double2 *>(a.V + row * a.ld);
             const double2 *xv = reinterpret_cast<const double2 *>(v);
             const int64_t n2 = a.ld / 2;
-            double acc = 0.0;
+            double a0 = 0.0, a1 = 0.0;
 #pragma unroll 4
             for (int64_t k = lane; k < n2; k += 32) {
                 const double2 m = __ldg(r + k);
                 const double2 w = xv[k];  // written by other CTAs before the last barrier
-                acc = fma(m.x, w.x, acc);
-                acc = fma(m.y, w.y, acc);
+                a0 = fma(m.x, w.x, a0);
+                a1 = fma(m.y, w.y, a1);
             }
-            acc = warp_sum(acc);
+            const double acc = warp_sum(a0 + a1);
             if (lane == 0) f(row, acc);
         }
         __syncwarp();
@@ -1908,6 +1922,8 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
     auto each = [&](auto f) {
         for (int64_t row = warp_g + lane * nwarps; row < a.N; row += 32 * nwarps) f(row);
     };
+    const int64_t first = warp_g + lane * nwarps;  // the lane's first row, mostly its only one
+    const double dinv = a.jacobi && first < a.N ? 1.0 / a.d[first] : 1.0;
     double sums[2] = {0.0, 0.0}, one[1] = {0.0}, tot[2];
     if (a.has_x0) product(a.x, [&](int64_t i, double y) { a.q[i] = y; });
     each([&](int64_t i) {
@@ -1929,6 +1945,7 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
     int it = 0;
     if (!grid_barrier(gb, G)) return;  // partial slots are reused below
     while (rr > thr && it < a.max_it) {
+        const double irz = 1.0 / rz;  // not in the chain from r.z to beta
         double pq[1] = {0.0};
         product(a.p, [&](int64_t i, double y) {
             a.q[i] = y;
@@ -1941,7 +1958,7 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
         sums[0] = sums[1] = 0.0;
         each([&](int64_t i) {
             a.x[i] += alpha * a.p[i];
-            const double ri = a.r[i] - alpha * a.q[i], zi = a.jacobi ? ri / a.d[i] : ri;
+            const double ri = a.r[i] - alpha * a.q[i], zi = !a.jacobi ? ri : i == first ? ri * dinv : ri / a.d[i];
             a.r[i] = ri;
             a.z[i] = zi;
             sums[0] += ri * zi;
@@ -1952,7 +1969,7 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
         grid_totals(pB, G, tot);
         rr = tot[1];
         ++it;
-        const double beta = tot[0] / rz;
+        const double beta = tot[0] * irz;
         rz = tot[0];
         each([&](int64_t i) { a.p[i] = a.z[i] + beta * a.p[i]; });
         if (!grid_barrier(gb, G)) return;
@@ -1983,20 +2000,6 @@ constexpr int kResRows = 16;
 constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
 constexpr int kResMaxCtas = 160;  // five partials per lane, 160 KB of rows
-
-// df_from_double by integer operations: the FP64 pipe converts two values per clock and SM.
-// Rounds hi to nearest (ties away from zero).
-__device__ __forceinline__ float2 df_split(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const int e = (int)(b >> 52) & 0x7ff;
-    if (e < 949 || e > 1149) return v == 0.0 ? make_float2(0.f, 0.f) : df_from_double(v);
-    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
-    const unsigned long long m = (b & 0x7fffffffffffffffull) + (1ull << 28);
-    const float hi = __uint_as_float(sign | (unsigned)((m >> 29) - (896ull << 23)));
-    const int rest = ((int)((unsigned)b << 3)) >> 3;  // the low 29 bits, signed: v - hi in units of 2^(e - 1075)
-    return make_float2(hi, (float)rest * __uint_as_float(sign | (unsigned)(e - 948) << 23));
-}
 
 template <class T, int P>  // P = ceil(ld / 1024): pairs of columns per thread
 __global__ void __launch_bounds__(kResThreads, 1) k_pcg_res(PcgArgs a)
