@@ -121,9 +121,7 @@ typedef struct {
                               operator's own product (DF64, or the exact FP32 one) after every
                               10^2-fold drop of ||r|| (or after 400 iterations without it), and
                               the FP32 copy taken for the rest of the solve if a replaced residual
-                              has fallen by less than 10x since the previous one.  Small solves
-                              (16 rows per SM, N <= 2,432) hold the FP32 entries in shared memory
-                              and multiply with those whatever is asked for here.  tol holds for
+                              has fallen by less than 10x since the previous one.  tol holds for
                               the operator in every mode. */
 } bem_solve_opts;
 #define BEM_PRODUCTS_DEFAULT 0

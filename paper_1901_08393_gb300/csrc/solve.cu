@@ -2565,12 +2565,18 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     const size_t vbytes = packed_bytes((size_t)nt_, (size_t)op->ld);
     const bool room = delta > 0.0 && (ctx->budget <= 0 || ctx->in_use + (int64_t)vbytes + (64 << 10) <= ctx->budget);
     if (f32op && !room) return BEM_OK;  // no room for the packed copy: host-driven refinement
+    // default: FP16 for FP32 operators (whose stored entries are FP32 roundings already)
+    // under the block preconditioner (a condition number the FP16 copy's perturbation
+    // leaves room for; diag(V) on strongly graded meshes does not), else the packed
+    // FP32 hi parts
+    if (products == BEM_PRODUCTS_DEFAULT)
+        products = (f32op && precond == BEM_PRECOND_BLOCK) ? BEM_PRODUCTS_FP16 : BEM_PRODUCTS_FP32;
     // resident solver: whole rows of FP32 entries in shared memory, four CTAs per 64 rows
     const void *kern = f32op ? res_kernel<float>(op->ld) : res_kernel<float2>(op->ld);
     size_t smem = sizeof(float) * kResRows * (size_t)op->ld;
     int threads = kResThreads;
     const int rG = (int)((op->N + kBJ - 1) / kBJ * (kBJ / kResRows));
-    bool resident = room && rG <= kResMaxCtas && precond != BEM_PRECOND_CALDERON && !(inexact_lambda > 0.0) && rG <= ctx->sm_count;
+    bool resident = room && products != BEM_PRODUCTS_FP16 && rG <= kResMaxCtas && precond != BEM_PRECOND_CALDERON && !(inexact_lambda > 0.0) && rG <= ctx->sm_count;
     if (resident) {
         // the most that any solve asks of the kernel, whatever another thread sets meanwhile
         const size_t most = sizeof(float) * kResRows * (kResMaxCtas / (kBJ / kResRows)) * kBJ;
@@ -2610,12 +2616,6 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     // FP16 working copy for the iteration products (N^2 bytes and a scale per tile)
     __half *vh = nullptr;
     float *vsc = nullptr;
-    // default: FP16 for FP32 operators (whose stored entries are FP32 roundings already)
-    // under the block preconditioner (a condition number the FP16 copy's perturbation
-    // leaves room for; diag(V) on strongly graded meshes does not), else the packed
-    // FP32 hi parts
-    if (products == BEM_PRODUCTS_DEFAULT)
-        products = (f32op && precond == BEM_PRECOND_BLOCK) ? BEM_PRODUCTS_FP16 : BEM_PRODUCTS_FP32;
     if (products == BEM_PRODUCTS_FP16 && vp && !calpc) {
         const size_t hb = (size_t)nt_ * kTileF * sizeof(__half), sb = ((size_t)nt_ * sizeof(float) + 255) / 256 * 256;
         if (ctx->budget <= 0 || ctx->in_use + (int64_t)(hb + sb) + (64 << 10) <= ctx->budget) {

@@ -34,11 +34,11 @@ def test_resident_solve_is_that_of_the_operators_entries(m):
         bound = 2.0 / s[-1] * (1e-11 * np.linalg.norm(area) + 2.0 ** -44 * s[0] * np.linalg.norm(x))
         for precond in (bem.PRECOND_NONE, bem.PRECOND_JACOBI, bem.PRECOND_BLOCK):
             for start in (None, x0):
-                _, phi, info = bem.solve_capacity(op, tol=1e-11, precond=precond, x0=start)
+                _, phi, info = bem.solve_capacity(op, tol=1e-11, precond=precond, x0=start, products=bem.PRODUCTS_FP32)
                 assert info["converged"] and info["relres"] <= 1e-11
                 assert info["outer"] >= 2 or info["iterations"] == 0
                 assert np.linalg.norm(x - phi) <= bound, (prec, precond, np.linalg.norm(x - phi), bound)
-                _, again, _ = bem.solve_capacity(op, tol=1e-11, precond=precond, x0=start)
+                _, again, _ = bem.solve_capacity(op, tol=1e-11, precond=precond, x0=start, products=bem.PRODUCTS_FP32)
                 assert np.array_equal(phi, again)
         op.close()
     ctx.close()
