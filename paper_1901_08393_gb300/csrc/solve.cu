@@ -2576,7 +2576,8 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     size_t smem = sizeof(float) * kResRows * (size_t)op->ld;
     int threads = kResThreads;
     const int rG = (int)((op->N + kBJ - 1) / kBJ * (kBJ / kResRows));
-    bool resident = room && products != BEM_PRODUCTS_FP16 && rG <= kResMaxCtas && precond != BEM_PRECOND_CALDERON && !(inexact_lambda > 0.0) && rG <= ctx->sm_count;
+    bool resident = room && products != BEM_PRODUCTS_FP16 && precond != BEM_PRECOND_CALDERON &&
+                    !(inexact_lambda > 0.0) && rG <= std::min(kResMaxCtas, ctx->sm_count);
     if (resident) {
         // the most that any solve asks of the kernel, whatever another thread sets meanwhile
         const size_t most = sizeof(float) * kResRows * (kResMaxCtas / (kBJ / kResRows)) * kBJ;
@@ -2802,7 +2803,9 @@ static bem_status pcg_f64_persistent(bem_operator *op, Work &W, const double *rh
     const int G = (int)std::min<int64_t>((op->N + kMvRows - 1) / kMvRows, (int64_t)std::min(per_sm, 2) * ctx->sm_count);
     Allocs tmp;
     double *part = nullptr;
-    bem_status st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (3 * (size_t)G + 8), true);
+    const size_t pbytes = sizeof(double) * (3 * (size_t)G + 8);
+    if (ctx->budget > 0 && ctx->in_use + (int64_t)pbytes + 1024 > ctx->budget) return BEM_OK;  // the host loop needs no more
+    bem_status st = dalloc(ctx, tmp, (void **)&part, pbytes, true);
     if (st) return st;
     double *out = part + 3 * G;
     unsigned *bar = reinterpret_cast<unsigned *>(out + 6);
