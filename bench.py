@@ -70,13 +70,14 @@ MAX_N = 20000
 THETA = 0.5
 TOL = 1e-10
 FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 rate (recipe table)
-FAR_FLOPS_PER_ENTRY = 49 * 11 + 16  # FP64 far field: per point pair 3 sub, 5 for r^2, rsqrt, 2 accumulate
-# Double-float far field: FP32 operations per entry of its grid form, which all but the
-# closest far pairs take (per point pair 44 FP32 arithmetic + 6 min/max + 1 MUFU; per row
-# point 31 for its split on the pair's grid and the outer sum; per entry 119 for the exact
-# centroid difference, the grid choice and the area products), against the FP32 issue
+# FP64 far field, by the method's own count: per point pair 3 sub, 5 for r^2, rsqrt, 2 accumulate
+# (the kernel takes fewer operations: 402 per entry)
+FAR_FLOPS_PER_ENTRY = 49 * 11 + 16
+# Double-float far field: FP32 operations per entry of its expanded form, which all but the
+# closest far pairs take (16 per point pair; about 520 per entry for the exact centroid
+# difference, the dot products and the area products), against the FP32 issue
 # peak 152 SMs x 128 lanes x 2.07 GHz.
-DF_FAR_OPS_PER_ENTRY = 49 * 51 + 7 * 31 + 119
+DF_FAR_OPS_PER_ENTRY = 49 * 16 + 520
 FP32_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
 PCG_TRAFFIC_RATIO = 18.072 / 18.294  # ncu DRAM bytes / algorithmic bytes of the persistent solver
 PRECISIONS = {"df64": 2, "f64": 0, "f32": 1}
@@ -1052,9 +1053,8 @@ def main():
                    "cap_final": recs[-1]["cap"], "parallelism": f"replicas x{ws}",
                    "far_tiles_autotuned": dict(zip(("N<1024", "N<4096", "N<16384", "larger"),
                                                    [["32x256", "16x256", "64x256", "8x128", "16x128", "32x128",
-                                                     "8x128 shared m8", "16x128 shared m8", "32x128 shared m8",
-                                                     "8x128 shared m9", "8x64 shared m16", "8x64 shared m18",
-                                                     "8x128 shared m6 unrolled", "32x128 shared m6 unrolled"][v - 1]
+                                                     "8x128 m5", "16x128 m5", "32x128 m5", "4x128 m5", "8x64 m10",
+                                                     "4x64 m10", "2x64 m10", "1x64 m10"][v - 1]
                                                     if v else None
                                                     for v in ctx.far_tiles()[PREC]])),
                    "l2": "256 MB buffer written before every step; V (up to 3.2 GB) exceeds L2"},
