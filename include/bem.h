@@ -103,7 +103,8 @@ typedef struct {
                               FP32 hi parts of V (a packed copy of the upper triangle, 2 N^2 bytes
                               while the solve runs), and r is replaced by b - V x formed with the
                               DF64 product whenever ||r|| has dropped by this factor since the
-                              last such residual and before convergence is declared, so tol
+                              last such residual and before convergence is declared (when ||r||
+                              is at half of tol; at tol under BEM_PRECOND_CALDERON), so tol
                               holds for the DF64 operator.  0: default 1e-4; < 0 or >= 1: DF64
                               products only */
     double inexact_lambda; /* > 0 (persistent solver): stop as soon as the update's energy norm

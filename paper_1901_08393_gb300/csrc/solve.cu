@@ -1682,7 +1682,11 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     double rr_true_prev = rr;
     int it = 0, ndf = prod0 ? 1 : 0, inexact_stop = 0;
     if (!grid_barrier(gb, G)) return;  // partial slots are reused below
-    while (!(rr <= thr) && it < a.max_it) {
+    // DF64 operators: convergence is confirmed at half the tolerance, one more iteration of
+    // about 60, so that the confirmed residual stays below the tolerance as in k_pcg_res
+    const double stop = !kCal && mixed && !a.f32op ? 0.25 * thr : thr;
+    bool done = rr <= thr;  // of a residual formed from x (products in DF64 only: the recursive one)
+    while (!done && it < a.max_it) {
         const double irz = 1.0 / rz;  // not in the chain from r.z to beta
         if (use16) {
             const int gr_static = a.ngroups <= nwarps ? (int)warp_g : -1;
@@ -1780,7 +1784,9 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             }
         }
         ++seg;
-        if (mixed && (rr <= (use16 ? kH16Delta2 : a.delta2) * rr_true || rr <= thr || (use16 && seg >= kH16SegMax))) {
+        if (!mixed) done = rr <= thr;
+        if (mixed && (rr <= (use16 ? kH16Delta2 : a.delta2) * rr_true || rr <= stop || (rr <= thr && it == a.max_it) ||
+                      (use16 && seg >= kH16SegMax))) {
             seg = 0;
             // reliable update: replace the recursive residual by b - V x with the
             // DF64 product (the direction p is kept)
@@ -1816,6 +1822,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             rr = tot[1];
             rr_true_prev = rr_true;
             rr_true = rr;
+            done = rr <= thr;
             ++ndf;
             if (use16 && rr_true > kH16Progress * rr_true_prev) use16 = false;  // the same in every CTA
         }
