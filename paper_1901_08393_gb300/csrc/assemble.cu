@@ -170,10 +170,17 @@ __device__ __forceinline__ float f64_to_f32_trunc(double v)
 {
     return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), (unsigned)__double2hiint(v) - (896u << 20), 3));
 }
-// |v| truncated, at least 2^-127
+// |v| truncated, at least 2^-127; |v| < 2^128
 __device__ __forceinline__ float f64_to_f32_abs(double v)
 {
     const unsigned h = max((unsigned)__double2hiint(v) & 0x7fffffffu, 896u << 20) - (896u << 20);
+    return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), h, 3));
+}
+// The same for any v: infinity or NaN from 2^128 on (infinity and NaN among them), so that no
+// comparison takes it for an ordinary length.
+__device__ __forceinline__ float f64_to_f32_len(double v)
+{
+    const unsigned h = min(max((unsigned)__double2hiint(v) & 0x7fffffffu, 896u << 20), 1151u << 20) - (896u << 20);
     return __uint_as_float(__funnelshift_l((unsigned)__double2loint(v), h, 3));
 }
 // -2 v for a normal v (a zero becomes -+2^-1022)
@@ -261,9 +268,9 @@ __device__ __forceinline__ void far_f64_body(const double *__restrict__ q64, con
     for (int r = 0; r < rows; ++r) {
         const int64_t i = i0 + r;
         const bool valid = j < c1 && i <= j;
-        const float fx = f64_to_f32_abs(sc[r][0] - cj[0]), fy = f64_to_f32_abs(sc[r][1] - cj[1]),
-                    fz = f64_to_f32_abs(sc[r][2] - cj[2]);
-        const float D2 = fx * fx + fy * fy + fz * fz, Rs = f64_to_f32_abs(sx[r][23]) + Rj;
+        const float fx = f64_to_f32_len(sc[r][0] - cj[0]), fy = f64_to_f32_len(sc[r][1] - cj[1]),
+                    fz = f64_to_f32_len(sc[r][2] - cj[2]);
+        const float D2 = fx * fx + fy * fy + fz * fz, Rs = f64_to_f32_len(sx[r][23]) + Rj;
         // where the bounds hold and |x - y|^2 is a normal FP32 number; not for NaN
         const bool wide = D2 >= kFarSpread2 * (Rs * Rs) && D2 >= 0x1p-68f && D2 <= 0x1p100f;
         if (valid && wide) {
