@@ -1116,17 +1116,10 @@ static bem_status cheb_cols(bem_ctx *ctx, bem_mesh *pm, const float *dinv, int64
 // (coalesced), and the rows' entries over the stars of the others:
 //   Z[z] = sum_{T at z} U[(T, k(z))],   V^dual[z][w] = sum_{T' at w} Z[z][(T', l(w))]
 //   R[i][T'] = sum_{T at i} curl phi_i|T V^T[T][T'],  D[i][j] = sum_{T' at j} curl phi_j|T' . R[i][T'].
-// Scratch: 92 N^2 bytes (V^bary has 288 N^2).  DF64 sums in double-float (2^-47; FP64 sums
-// ran at 1/64 of that rate).
+// Scratch: U 72 N^2 bytes, Z and R 12 each, V^T 8: 104 N^2 with N / 2 vertices (V^bary has
+// 288 N^2).  Every sum is FP64, as on the path without scratch.
 
-// Sums of contracted elements: double (F64) or hi/lo pairs.
-__device__ __forceinline__ double u_add(double a, double b) { return a + b; }
-__device__ __forceinline__ float2 u_add(float2 a, float2 b) { return df_add(a, b); }
-__device__ __forceinline__ double u_double(double a) { return a; }
-__device__ __forceinline__ double u_double(float2 a) { return df_to_double(a); }
-template <typename T> struct ContractElem { using type = float2; };
-template <> struct ContractElem<double> { using type = double; };
-
+// Six entries of a row of V^bary.
 __device__ __forceinline__ void vb_row6(const float2 *p, float2 (&v)[6])
 {
     const float4 *q = reinterpret_cast<const float4 *>(p);
@@ -1147,70 +1140,105 @@ __device__ __forceinline__ void vb_row6(const double *p, double (&v)[6])
         v[2 * u + 1] = f.y;
     }
 }
-__device__ __forceinline__ void vb_row6(const float *p, float2 (&v)[6])
+__device__ __forceinline__ void vb_row6(const float *p, float (&v)[6])
 {
     const float2 *q = reinterpret_cast<const float2 *>(p);
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
         const float2 f = __ldg(q + u);
-        v[2 * u] = make_float2(f.x, 0.0f);
-        v[2 * u + 1] = make_float2(f.y, 0.0f);
+        v[2 * u] = f.x;
+        v[2 * u + 1] = f.y;
     }
 }
-__device__ __forceinline__ float2 vb_one(const float2 *p) { return *p; }
-__device__ __forceinline__ double vb_one(const double *p) { return *p; }
-__device__ __forceinline__ float2 vb_one(const float *p) { return make_float2(*p, 0.0f); }
+
+// FP64 sums of four entries.  Additions and conversions take the FP64 pipe (2 lanes per SM
+// and cycle), seven of the one and eight of the other for four hi/lo pairs.  So the hi parts add
+// by two-sums, their errors and the lo parts by two-sums again, and the errors of those
+// plainly: three floats s + l + r within 2^-70 of the sum.  s at least 2^-60 converts by integer
+// operations; a zero or subnormal l or r becomes at most 2^-126 there, which the additions
+// round away.  Two FP64 operations: the dual operator of N = 3,072 (DF64) takes 1.42 ms with
+// double-float sums, 1.77 with FP64 sums of converted entries, 1.47 like this.
+__device__ __forceinline__ double f32_bits_to_f64(float v)
+{
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + (896u << 20))), (int)(b << 29));
+}
+__device__ __forceinline__ bool f64_by_bits(float v)  // 2^-60 <= v, finite
+{
+    constexpr unsigned lo = (127u - 60u) << 23;
+    return __float_as_uint(v) - lo < 0x7f800000u - lo;
+}
+__device__ __forceinline__ double sum4(double a, double b, double c, double d) { return (a + b) + (c + d); }
+__device__ __forceinline__ double sum4(float2 a, float2 b, float2 c, float2 d)
+{
+    float s, t, u, e1, e2, e3, r = 0.0f, l = a.y;
+    two_sum(a.x, b.x, s, e1);
+    two_sum(c.x, d.x, t, e2);
+    two_sum(s, t, u, e3);
+    const float low[6] = {b.y, c.y, d.y, e1, e2, e3};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        float q, e;
+        two_sum(l, low[k], q, e);
+        l = q;
+        r += e;
+    }
+    if (f64_by_bits(u)) return f32_bits_to_f64(u) + (f32_bits_to_f64(l) + f32_bits_to_f64(r));
+    return sum4(df_to_double(a), df_to_double(b), df_to_double(c), df_to_double(d));
+}
+__device__ __forceinline__ double sum4(float a, float b, float c, float d)
+{
+    float s, t, u, e1, e2, e3, q, e;
+    two_sum(a, b, s, e1);
+    two_sum(c, d, t, e2);
+    two_sum(s, t, u, e3);
+    two_sum(e1, e2, q, e);
+    float l, f;
+    two_sum(q, e3, l, f);
+    if (f64_by_bits(u)) return f32_bits_to_f64(u) + (f32_bits_to_f64(l) + f32_bits_to_f64(e + f));
+    return sum4((double)a, (double)b, (double)c, (double)d);
+}
 
 // Tile of 8 triangles T (one per warp) x 32 triangles T' (one per lane), pairs T <= T' only:
-// 18 loads of 16 bytes per thread; the results go through shared memory so that rows and
+// 18 loads of 16 bytes per thread (DF64); the results go through shared memory so that rows and
 // mirrored rows are written in whole segments.  Children 0, 5 belong to vertex 0, 1, 2 to
 // vertex 1, 3, 4 to vertex 2.
-template <typename T, typename E>
-__global__ void __launch_bounds__(256) k_contract(const T *__restrict__ Vb, int64_t ldb, int64_t N, E *__restrict__ U,
-                                                  double *__restrict__ VT)
+template <typename T>
+__global__ void __launch_bounds__(256) k_contract(const T *__restrict__ Vb, int64_t ldb, int64_t N,
+                                                  double *__restrict__ U, double *__restrict__ VT)
 {
     const int64_t t0 = 8 * (int64_t)blockIdx.y, s0 = 32 * (int64_t)blockIdx.x;
     if (s0 + 31 < t0) return;
-    __shared__ E us[24][97];
+    __shared__ double us[24][97];
     __shared__ double vs[8][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t t = t0 + w, t2 = s0 + lane;
     if (t < N && t2 < N && t <= t2) {
-        E c[6][3];  // the row's children by columns
-        if (t < t2) {
+        constexpr int ca[3] = {0, 1, 3}, cb[3] = {5, 2, 4};  // the children of a triangle at its vertices
+        double tot = 0.0;
 #pragma unroll
-            for (int a = 0; a < 6; ++a) {
-                E v[6];
-                vb_row6(Vb + (6 * t + a) * ldb + 6 * t2, v);
-                c[a][0] = u_add(v[0], v[5]);
-                c[a][1] = u_add(v[1], v[2]);
-                c[a][2] = u_add(v[3], v[4]);
-            }
-        } else {  // entries below the diagonal from above it
+        for (int k = 0; k < 3; ++k) {
+            T a[6], b[6];
+            if (t < t2) {
+                vb_row6(Vb + (6 * t + ca[k]) * ldb + 6 * t2, a);
+                vb_row6(Vb + (6 * t + cb[k]) * ldb + 6 * t2, b);
+            } else {  // entries below the diagonal from above it
 #pragma unroll
-            for (int a = 0; a < 6; ++a) {
-                E v[6];
-#pragma unroll
-                for (int b = 0; b < 6; ++b) {
-                    const int lo = a < b ? a : b, hi = a < b ? b : a;
-                    v[b] = vb_one(Vb + (6 * t + lo) * ldb + 6 * t + hi);
+                for (int c = 0; c < 6; ++c) {
+                    a[c] = Vb[(6 * t + min(c, ca[k])) * ldb + 6 * t + max(c, ca[k])];
+                    b[c] = Vb[(6 * t + min(c, cb[k])) * ldb + 6 * t + max(c, cb[k])];
                 }
-                c[a][0] = u_add(v[0], v[5]);
-                c[a][1] = u_add(v[1], v[2]);
-                c[a][2] = u_add(v[3], v[4]);
             }
-        }
-        E tot;
+            double r = 0.0;
 #pragma unroll
-        for (int l = 0; l < 3; ++l) {
-            const E u0 = u_add(c[0][l], c[5][l]), u1 = u_add(c[1][l], c[2][l]), u2 = u_add(c[3][l], c[4][l]);
-            us[3 * w][3 * lane + l] = u0;
-            us[3 * w + 1][3 * lane + l] = u1;
-            us[3 * w + 2][3 * lane + l] = u2;
-            const E r = u_add(u_add(u0, u1), u2);
-            tot = l ? u_add(tot, r) : r;
+            for (int l = 0; l < 3; ++l) {
+                const double v = sum4(a[ca[l]], a[cb[l]], b[ca[l]], b[cb[l]]);
+                us[3 * w + k][3 * lane + l] = v;
+                r += v;
+            }
+            tot += r;
         }
-        vs[w][lane] = u_double(tot);
+        vs[w][lane] = tot;
     }
     __syncthreads();
     const int64_t L = 3 * N;
@@ -1251,38 +1279,43 @@ __global__ void k_star_table(const double *V, const int32_t *tris, const double 
 }
 
 // Z[z] = sum of the star's rows of U; grid (columns, vertices).
-template <typename E>
-__global__ void __launch_bounds__(256) k_star_rows(const E *__restrict__ U, const int32_t *__restrict__ row,
-                                                   const int32_t *__restrict__ v2t_off, int64_t L, E *__restrict__ Z)
+__global__ void __launch_bounds__(256) k_star_rows(const double *__restrict__ U, const int32_t *__restrict__ row,
+                                                   const int32_t *__restrict__ v2t_off, int64_t L,
+                                                   double *__restrict__ Z)
 {
     const int64_t z = blockIdx.y, c = (int64_t)blockIdx.x * 256 + threadIdx.x;
     if (c >= L) return;
     const int32_t b = v2t_off[z], e = v2t_off[z + 1];
-    E s = E();
+    double s = 0.0;
     for (int32_t p = b; p < e; p += 4) {  // four loads in flight
-        E v[4];
+        double v[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (p + u < e) v[u] = U[(int64_t)row[p + u] * L + c];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (p + u < e) s = u_add(s, v[u]);
+            if (p + u < e) s += v[u];
     }
     Z[z * L + c] = s;
 }
 
 // V^dual[z][w], w >= z, mirrored.
-template <typename E, typename O>
-__global__ void __launch_bounds__(128) k_dual_gather(const E *__restrict__ Z, const int32_t *__restrict__ row,
+template <typename O>
+__global__ void __launch_bounds__(128) k_dual_gather(const double *__restrict__ Z, const int32_t *__restrict__ row,
                                                      const int32_t *__restrict__ v2t_off, int64_t L, int64_t M, O *Vd,
                                                      int64_t ldd)
 {
     const int64_t z = blockIdx.y, w = z + (int64_t)blockIdx.x * 128 + threadIdx.x;
     if (w >= M) return;
-    E s = E();
-    for (int32_t q = v2t_off[w]; q < v2t_off[w + 1]; ++q) s = u_add(s, Z[z * L + row[q]]);
-    Vd[z * ldd + w] = s;
-    Vd[w * ldd + z] = s;
+    double s = 0.0;
+    for (int32_t q = v2t_off[w]; q < v2t_off[w + 1]; ++q) s += Z[z * L + row[q]];
+    O v;
+    if constexpr (std::is_same<O, double>::value)
+        v = s;
+    else
+        v = df_from_double(s);
+    Vd[z * ldd + w] = v;
+    Vd[w * ldd + z] = v;
 }
 
 // R[i][T'] (three components); grid (columns, vertices).
@@ -1326,17 +1359,16 @@ __global__ void __launch_bounds__(128) k_hyper_gather(const double *__restrict__
 template <typename T>
 static bem_status dual_contract(const bem_operator *ob, bem_mesh *pm, bem_operator *op, int *bad, bool *done)
 {
-    using E = typename ContractElem<T>::type;
+    using O = typename std::conditional<std::is_same<T, double>::value, double, float2>::type;  // of V^dual
     bem_ctx *ctx = pm->ctx;
     cudaStream_t s = ctx->stream;
     const int64_t N = pm->N, M = pm->M, L = 3 * N;
     *done = false;
-    const size_t ub = sizeof(E) * (size_t)L * (size_t)L, zb = sizeof(E) * (size_t)L * (size_t)M,
+    const size_t ub = sizeof(double) * (size_t)L * (size_t)L, zb = sizeof(double) * (size_t)L * (size_t)M,
                  vb = sizeof(double) * (size_t)N * (size_t)N, rb = 3 * sizeof(double) * (size_t)N * (size_t)M,
                  tb = (size_t)L * (3 * sizeof(double) + sizeof(int32_t));
     Allocs tu, tr;
-    E *U = nullptr, *Z = nullptr;
-    double *VT = nullptr, *R = nullptr, *curl = nullptr;
+    double *U = nullptr, *Z = nullptr, *VT = nullptr, *R = nullptr, *curl = nullptr;
     if (ctx->budget > 0 && ctx->in_use + (int64_t)(ub + zb + vb + rb + tb) + (1 << 20) > ctx->budget) return BEM_OK;
     if (dalloc(ctx, tu, (void **)&U, ub, false) || dalloc(ctx, tu, (void **)&Z, zb, false) ||
         dalloc(ctx, tr, (void **)&VT, vb, false) || dalloc(ctx, tr, (void **)&R, rb, false) ||
@@ -1349,9 +1381,9 @@ static bem_status dual_contract(const bem_operator *ob, bem_mesh *pm, bem_operat
     int32_t *row = reinterpret_cast<int32_t *>(curl + 3 * L);
     *done = true;
     k_star_table<<<nblk(M, 128), 128, 0, s>>>(pm->verts, pm->tris, pm->area, pm->v2t_off, pm->v2t, M, row, curl, bad); BEM_COUNT(ctx);
-    k_contract<T, E><<<dim3(nblk(N, 32), nblk(N, 8)), 256, 0, s>>>((const T *)ob->V, ob->ld, N, U, VT); BEM_COUNT(ctx);
-    k_star_rows<E><<<dim3(nblk(L, 256), (unsigned)M), 256, 0, s>>>(U, row, pm->v2t_off, L, Z); BEM_COUNT(ctx);
-    k_dual_gather<E, E><<<dim3(nblk(M, 128), (unsigned)M), 128, 0, s>>>(Z, row, pm->v2t_off, L, M, (E *)op->V, op->ld); BEM_COUNT(ctx);
+    k_contract<T><<<dim3(nblk(N, 32), nblk(N, 8)), 256, 0, s>>>((const T *)ob->V, ob->ld, N, U, VT); BEM_COUNT(ctx);
+    k_star_rows<<<dim3(nblk(L, 256), (unsigned)M), 256, 0, s>>>(U, row, pm->v2t_off, L, Z); BEM_COUNT(ctx);
+    k_dual_gather<O><<<dim3(nblk(M, 128), (unsigned)M), 128, 0, s>>>(Z, row, pm->v2t_off, L, M, (O *)op->V, op->ld); BEM_COUNT(ctx);
     dfree_all(ctx, tu);  // stream-ordered
     k_star_field<<<dim3(nblk(N, 128), (unsigned)M), 128, 0, s>>>(VT, curl, pm->v2t_off, pm->v2t, N, R); BEM_COUNT(ctx);
     k_hyper_gather<<<dim3(nblk(M, 128), (unsigned)M), 128, 0, s>>>(R, curl, pm->v2t_off, pm->v2t, N, op->mesh->area, M,
