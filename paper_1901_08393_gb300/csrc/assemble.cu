@@ -145,6 +145,13 @@ struct FarTileS {
 constexpr FarTileS kFarTiles[kFarTileVariants] = {
     {32, 256, 0}, {16, 256, 0}, {64, 256, 0}, {8, 128, 0}, {16, 128, 0}, {32, 128, 0}, {8, 128, 5},
     {16, 128, 5}, {32, 128, 5}, {4, 128, 5},  {8, 64, 10}, {4, 64, 10},  {2, 64, 10}, {1, 64, 10}};
+constexpr bool far_rows_divide_cols()
+{
+    for (const FarTileS &t : kFarTiles)
+        if (t.cols % t.rows) return false;
+    return true;
+}
+static_assert(far_rows_divide_cols(), "a column tile holds whole row tiles (far_items)");
 
 // The far-field bodies take the tile origin (first row i0, first column cbase) as
 // arguments: the per-operator kernels derive it from the block index, the batched
@@ -1260,17 +1267,22 @@ int far_batch_variant(const bem_ctx *ctx, int precision, int64_t N)
     return far_bucket(N) > 0 && kFarTiles[v].rows * kFarTiles[v].cols < kFarBatchArea ? 6 : v;
 }
 
+// Tiles of variant v that reach the diagonal of N rows or above: K column tiles; the rows of
+// column tile m take K - m of them.
+static int64_t far_items(int v, int64_t N)
+{
+    const int64_t R = kFarTiles[v].rows, C = kFarTiles[v].cols, K = (N + C - 1) / C;
+    return C / R * (K * (K + 1) / 2 - 1) + (N - (K - 1) * C + R - 1) / R;
+}
+
 double far_batch_items_bound(int tile, int64_t N)
 {
-    int R = 8, C = 64;  // the smallest tile of kFarBatchArea entries or more
-    if (tile > 0) {
-        R = kFarTiles[tile - 1].rows;
-        C = kFarTiles[tile - 1].cols;
-    } else if (far_bucket(N) == 0) {
-        R = 1;
-    }
-    const double n = (double)N;
-    return n * n / (2.0 * R * C) + n / std::min(R, 4) + 2.0;  // 4 x 128 has the fewest rows of that area
+    if (tile > 0) return (double)far_items(tile - 1, N);
+    int64_t most = 0;
+    for (int v = 0; v < kFarTileVariants; ++v)
+        if (far_bucket(N) == 0 || kFarTiles[v].rows * kFarTiles[v].cols >= kFarBatchArea)
+            most = std::max(most, far_items(v, N));
+    return (double)most;
 }
 
 bem_status far_tune(bem_operator *op)

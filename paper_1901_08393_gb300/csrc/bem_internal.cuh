@@ -241,8 +241,8 @@ bem_status batch_assemble(bem_ctx *ctx, const BatchAsm &b, cudaEvent_t *ev);
 // captured from that stream.
 bem_status record_timing_event(bem_ctx *ctx, cudaEvent_t e);
 // The autotuned far-field variant of (precision, N) in ctx for a batch wave whose largest
-// mesh has N triangles (0 while not timed), and a bound on the tiles listed for a mesh
-// (tile: the requested variant, 0 for the autotuned one).
+// mesh has N triangles (0 while not timed), and the most tiles listed for a mesh (tile: the
+// requested variant, 0 for any that a batch may choose).
 int far_batch_variant(const bem_ctx *ctx, int precision, int64_t N);
 double far_batch_items_bound(int tile, int64_t N);
 
