@@ -1885,6 +1885,20 @@ __global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_batch(const PcgAr
 // per iteration.  The host loop it replaces launched three kernels per iteration and read
 // r.r back after each: 30 us per iteration at N = 192, now 11 (evaluation of the 192-triangle
 // cube from host arrays 1.34 -> 0.80 ms).
+//
+// Large products are bound by the FP64 pipe (2 lanes per SM and cycle: 1.43 ms at N = 30,000)
+// while enough of V is in flight: two CTAs per SM of up to 128 registers, twelve loads of 16
+// bytes per lane, past L1, which keeps the vector.  Left to 66 registers the loads waited for
+// one another.  Per iteration, host loop / 66 registers / now: N = 4,800 78 / 63 / 57 us, 10,092
+// 243 / 254 / 223, 12,288 315 / 359 / 316, 20,172 754 / 859 / 751, 38,988 2,691 / 3,081 / 2,680.
+constexpr int kF64Ctas = 2;
+__device__ __forceinline__ double2 ld_once(const double2 *p)
+{
+    double2 v;
+    asm("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
 struct PcgF64Args {
     const double *V;
     int64_t ld, N;
@@ -1900,7 +1914,7 @@ struct PcgF64Args {
     int absent_cta;
 };
 
-__global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
+__global__ void __launch_bounds__(kMvThreads, kF64Ctas) k_pcg_f64(PcgF64Args a)
 {
     const int G = gridDim.x, cta = blockIdx.x, lane = threadIdx.x & 31;
     const int64_t warp_g = ((int64_t)cta * kMvThreads + threadIdx.x) >> 5, nwarps = ((int64_t)G * kMvThreads) >> 5;
@@ -1913,9 +1927,9 @@ __global__ void __launch_bounds__(kMvThreads) k_pcg_f64(PcgF64Args a)
             const double2 *xv = reinterpret_cast<const double2 *>(v);
             const int64_t n2 = a.ld / 2;
             double a0 = 0.0, a1 = 0.0;
-#pragma unroll 4
+#pragma unroll 12
             for (int64_t k = lane; k < n2; k += 32) {
-                const double2 m = __ldg(r + k);
+                const double2 m = ld_once(r + k);
                 const double2 w = xv[k];  // written by other CTAs before the last barrier
                 a0 = fma(m.x, w.x, a0);
                 a1 = fma(m.y, w.y, a1);
@@ -2806,8 +2820,8 @@ static bem_status pcg_f64_persistent(bem_operator *op, Work &W, const double *rh
         const bem_status st = ensure_full(op);
         if (st) return st;
     }
-    // a row per warp where that fits, at most 2 CTAs per SM (more only wait at barriers)
-    const int G = (int)std::min<int64_t>((op->N + kMvRows - 1) / kMvRows, (int64_t)std::min(per_sm, 2) * ctx->sm_count);
+    // a row per warp where that fits, at most kF64Ctas CTAs per SM (more only wait at barriers)
+    const int G = (int)std::min<int64_t>((op->N + kMvRows - 1) / kMvRows, (int64_t)std::min(per_sm, kF64Ctas) * ctx->sm_count);
     Allocs tmp;
     double *part = nullptr;
     const size_t pbytes = sizeof(double) * (3 * (size_t)G + 8);
