@@ -1522,7 +1522,7 @@ __device__ __forceinline__ void grid_totals(const double *slot, int G, double (&
     if (w < n) {
         const double *p = slot + (int64_t)w * G;
         double v = 0.0;
-        for (int k0 = 0; k0 < G; k0 += 320) {  // ten loads in flight (G <= 304), a tree of sums
+        for (int k0 = 0; k0 < G; k0 += 320) {  // ten loads in flight (mostly G <= 304), a tree of sums
             double t[10];
 #pragma unroll
             for (int u = 0; u < 10; ++u) {
@@ -1561,16 +1561,25 @@ __device__ __forceinline__ float2 df_split(double v)
 // 60 -> 42 us in all.
 constexpr int kPcgCtas = 2;
 
+// Products in DF64 alone (reliable_delta < 0, or no room for the packed copy) stage whole
+// tiles per CTA and wait for them: three CTAs per SM of 80 registers, without the packed
+// products' code, hide that better once every CTA has tiles enough, two do before.  Per
+// iteration, Jacobi / block, two CTAs and three: N = 7,500 78 / 86 and 79 / 91 us, 10,092 119 / 128
+// and 117 / 129, 14,700 224 / 233 and 210 / 223, 22,188 484 / 498 and 433 / 447, 32,448 993 / 1,008
+// and 909 / 932.
+constexpr int kPcgCtasDf = 3, kPcgDfTiles = 40;  // from this many tiles per CTA on
+
 // kCal: the build with the operator preconditioner (BEM_PRECOND_CALDERON), kept out of
-// the other solvers' kernels (its Chebyshev and D^reg phases cost registers).
-template <bool kCal>
+// the other solvers' kernels (its Chebyshev and D^reg phases cost registers).  kMixed:
+// false: products in DF64 alone.
+template <bool kCal, bool kMixed>
 __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const int cta)
 {
     extern __shared__ float2 sm[];
     const int64_t stride = (int64_t)G * kSymThreads;
     const int64_t i0 = (int64_t)cta * kSymThreads + threadIdx.x;
     double *const pA = a.part, *const pB = a.part + G;  // one value; two values
-    const bool mixed = a.vp != nullptr;
+    const bool mixed = kMixed && a.vp != nullptr;
     const bool blockpc = a.precond == BEM_PRECOND_BLOCK, jacobi = a.precond == BEM_PRECOND_JACOBI;
     const bool calpc = kCal && a.precond == BEM_PRECOND_CALDERON;
     const bool zlocal = !blockpc && !calpc;  // z_i from r_i alone
@@ -1849,8 +1858,9 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     }
 }
 
-__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_df(PcgArgs a) { pcg_body<false>(a, gridDim.x, blockIdx.x); }
-__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_cal(PcgArgs a) { pcg_body<true>(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_df(PcgArgs a) { pcg_body<false, true>(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kSymThreads, kPcgCtasDf) k_pcg_df_only(PcgArgs a) { pcg_body<false, false>(a, gridDim.x, blockIdx.x); }
+__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_cal(PcgArgs a) { pcg_body<true, true>(a, gridDim.x, blockIdx.x); }
 
 // Independent solves in one cooperative launch: problem p owns the CTAs
 // [begin[p], begin[p + 1]) and runs the same solver on them, with its own grid
@@ -1876,7 +1886,7 @@ __global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_batch(const PcgAr
     const int p = s_p;
     const int b0 = begin[p], b1 = begin[p + 1];
     if ((int)blockIdx.x >= b1) return;  // CTAs past the last group
-    pcg_body<false>(sa, b1 - b0, (int)blockIdx.x - b0);
+    pcg_body<false, true>(sa, b1 - b0, (int)blockIdx.x - b0);
 }
 
 // The whole (Jacobi-)PCG of a native FP64 operator in one cooperative launch: one warp per
@@ -2599,6 +2609,7 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     const int rG = (int)((op->N + kBJ - 1) / kBJ * (kBJ / kResRows));
     bool resident = room && products != BEM_PRODUCTS_FP16 && precond != BEM_PRECOND_CALDERON &&
                     !(inexact_lambda > 0.0) && rG <= std::min(kResMaxCtas, ctx->sm_count);
+    const bool df_only = !room && precond != BEM_PRECOND_CALDERON && nt_ >= kPcgDfTiles * kPcgCtasDf * ctx->sm_count;
     if (resident) {
         // the most that any solve asks of the kernel, whatever another thread sets meanwhile
         const size_t most = sizeof(float) * kResRows * (kResMaxCtas / (kBJ / kResRows)) * kBJ;
@@ -2609,7 +2620,9 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
     if (resident) {
         if ((st = ensure_full(op))) return st;
     } else {
-        kern = precond == BEM_PRECOND_CALDERON ? (const void *)k_pcg_cal : (const void *)k_pcg_df;
+        kern = precond == BEM_PRECOND_CALDERON ? (const void *)k_pcg_cal
+               : df_only                       ? (const void *)k_pcg_df_only
+                                               : (const void *)k_pcg_df;
         smem = kSymSmem;
         threads = kSymThreads;
         BEM_CK(ctx, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -2652,10 +2665,10 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
             }
         }
     }
-    // Up to kPcgCtas CTAs per SM.  On small levels, CTAs that would only wait at the grid
+    // Up to kPcgCtas (kPcgCtasDf) CTAs per SM.  On small levels, CTAs that would only wait at the grid
     // barriers are left out: DF64 products take one tile per CTA, the mixed mode's
     // products one tile per warp (8 per CTA), its row passes 8 rows per warp.
-    const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
+    const int Gmax = std::min(per_sm, df_only ? kPcgCtasDf : kPcgCtas) * ctx->sm_count;
     int G = vp ? (int)std::max<int64_t>((nt_ + 7) / 8, (op->N + 63) / 64) : nt_;
     G = resident ? rG : std::min(std::max(G, 8), Gmax);
     // groups of tiles (FP16 products); the tiles themselves where their list finds no room
