@@ -360,7 +360,7 @@ bem_status bem_operator_preconditioner(const bem_operator *op, int32_t which, fl
  * operator precision (aopts->precision BEM_PREC_DF64 or BEM_PREC_F32).  It cuts the
  * problems, in their given order, into waves whose device memory fits what is
  * available at creation -- 90% of the device's free memory, and the context's HBM
- * budget if it has one -- and at most 2 x (number of SMs) problems per wave; one
+ * budget if it has one -- and at most 3 x (number of SMs) problems per wave; one
  * arena sized for the largest wave holds the operators and the solver state of the
  * wave that runs (a problem that alone exceeds it: BEM_ERR_OOM).  It also times the
  * far-field tiles of the size classes present and, for BEM_PRECOND_BLOCK, computes the

@@ -1865,8 +1865,9 @@ __global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_cal(PcgArgs a) { 
 // Independent solves in one cooperative launch: problem p owns the CTAs
 // [begin[p], begin[p + 1]) and runs the same solver on them, with its own grid
 // barrier, tile counter and partials; a problem that converges releases its CTAs.
-__global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_batch(const PcgArgs *__restrict__ args,
-                                                              const int *__restrict__ begin, int P)
+template <bool kMixed, int kCtas>
+__global__ void __launch_bounds__(kSymThreads, kCtas) k_pcg_batch(const PcgArgs *__restrict__ args,
+                                                                  const int *__restrict__ begin, int P)
 {
     __shared__ PcgArgs sa;
     __shared__ int s_p;
@@ -1886,7 +1887,7 @@ __global__ void __launch_bounds__(kSymThreads, kPcgCtas) k_pcg_batch(const PcgAr
     const int p = s_p;
     const int b0 = begin[p], b1 = begin[p + 1];
     if ((int)blockIdx.x >= b1) return;  // CTAs past the last group
-    pcg_body<false, true>(sa, b1 - b0, (int)blockIdx.x - b0);
+    pcg_body<false, kMixed>(sa, b1 - b0, (int)blockIdx.x - b0);
 }
 
 // The whole (Jacobi-)PCG of a native FP64 operator in one cooperative launch: one warp per
@@ -3213,6 +3214,7 @@ struct BatchProblem {
 // proportion to N^2, so that they finish at about the same time.
 struct BatchGroup {
     int count = 0, G = 0;
+    const void *kern = nullptr;  // k_pcg_batch
     std::vector<int> idx;    // problems (batch indices), in launch order
     std::vector<int> begin;  // CTA ranges
     PcgArgs *d_args = nullptr;
@@ -3293,7 +3295,11 @@ static bem_status batch_enqueue(bem_batch *bt, BatchWave &w)
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        BEM_CK(ctx, cudaLaunchKernelEx(&cfg, k_pcg_batch, (const PcgArgs *)gr.d_args, (const int *)gr.d_begin, gr.count));
+        const PcgArgs *args = gr.d_args;
+        const int *begin = gr.d_begin;
+        int count = gr.count;
+        void *kargs[] = {&args, &begin, &count};
+        BEM_CK(ctx, cudaLaunchKernelExC(&cfg, gr.kern, kargs));
         BEM_COUNT(ctx);
     }
     if ((st = record_timing_event(ctx, w.ev[5]))) return st;
@@ -3341,13 +3347,23 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             return set_error(ctx, BEM_ERR_INVALID, "mesh %d is not a triangle mesh of this context", p);
     const int ss = (aopts && aopts->ss_order > 0) ? aopts->ss_order : 4;
     if (ss < 2 || ss > kMaxSS) return set_error(ctx, BEM_ERR_INVALID, "ss_order outside 2..16");
-    int coop = 0, per_sm = 0;
+    int coop = 0, per_sm = 0, per_sm3 = 0;
     BEM_CK(ctx, cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device));
     if (!coop) return set_error(ctx, BEM_ERR_CUDA, "the device has no cooperative launch");
-    BEM_CK(ctx, cudaFuncSetAttribute(k_pcg_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSymSmem));
-    BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pcg_batch, kSymThreads, kSymSmem));
-    const int Gmax = std::min(per_sm, kPcgCtas) * ctx->sm_count;
-    if (Gmax < 1) return set_error(ctx, BEM_ERR_CUDA, "the batch solver cannot be resident on this device");
+    const double rd = sopts ? sopts->reliable_delta : 0.0;
+    const double delta = rd == 0.0 ? 1e-4 : (rd > 0.0 && rd < 1.0 ? rd : 0.0);
+    const bool packed = prec == BEM_PREC_F32 || delta > 0.0;
+    // two CTAs per SM, or three: for groups of more problems than two hold, and for large DF64
+    // operators without a packed copy
+    const void *kern2 = packed ? (const void *)k_pcg_batch<true, kPcgCtas> : (const void *)k_pcg_batch<false, kPcgCtas>;
+    const void *kern3 = packed ? (const void *)k_pcg_batch<true, 3> : (const void *)k_pcg_batch<false, 3>;
+    for (const void *k : {kern2, kern3})
+        BEM_CK(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSymSmem));
+    BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern2, kSymThreads, kSymSmem));
+    BEM_CK(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm3, kern3, kSymThreads, kSymSmem));
+    const int Gmax2 = std::min(per_sm, kPcgCtas) * ctx->sm_count;
+    const int Gmax = std::max(std::min(per_sm3, 3) * ctx->sm_count, Gmax2);
+    if (Gmax2 < 1) return set_error(ctx, BEM_ERR_CUDA, "the batch solver cannot be resident on this device");
     bem_status st = assembly_prepare(ctx);
     if (st) return st;
     BEM_CK(ctx, cudaStreamSynchronize(ctx->stream));  // meshes built on the context's stream
@@ -3360,9 +3376,6 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
     bt->precision = prec;
     bt->tol = (sopts && sopts->tol > 0) ? sopts->tol : 1e-10;
     const int max_it = (sopts && sopts->max_it > 0) ? sopts->max_it : 10000;
-    const double rd = sopts ? sopts->reliable_delta : 0.0;
-    const double delta = rd == 0.0 ? 1e-4 : (rd > 0.0 && rd < 1.0 ? rd : 0.0);
-    const bool packed = prec == BEM_PREC_F32 || delta > 0.0;
     const bool block = precond == BEM_PRECOND_BLOCK;
     {
         const int pr = sopts ? sopts->products : BEM_PRODUCTS_DEFAULT;
@@ -3478,12 +3491,20 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
         const int P = w.count;
         // Groups: the wave's problems by decreasing N, a new group when N^2 falls below
         // half the group's first or the group has as many problems as CTAs can serve
-        // (8 per problem that can use them, else what it can use).  Within a group, CTAs
+        // (8 per problem that can use them, else what it can use; below N = 2,000, where
+        // latency is most of an iteration, half of that up to 4, and for problems of one
+        // CTA as many as three CTAs per SM hold).  Within a group, CTAs
         // per problem in proportion to its bytes per product (N^2; iteration counts are
         // alike), at least one, at most what the single-problem rule can use (a tile per
         // warp, 8 rows per warp), so that the group's problems finish at about the same
         // time; small, latency-bound problems share one launch instead of holding CTAs
-        // that the large ones need.
+        // that the large ones need.  CTAs that the rounding leaves go to those with the
+        // most bytes per CTA.
+        //
+        // 8 CTAs per problem against the smaller share, FP32 operators, block
+        // preconditioner: 150 of N = 192 2.19 / 1.79 ms, 456 of N = 588 23.5 / 19.2, 100 of N = 972 8.9 /
+        // 8.0, 100 of N = 1,728 15.9 / 15.3, 100 of N = 2,352 24.8 / 24.7 (DF64 38.9 / 39.1), 40
+        // of N = 7,500 73.2 / 76.0.  DF64 products alone: three CTAs per SM as for a single solve.
         std::vector<int64_t> want(P);
         for (int k = 0; k < P; ++k) {
             const int64_t N = meshes[w.first + k]->N, nt = bt->prob[w.first + k].nt;
@@ -3499,31 +3520,49 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             BatchGroup gr;
             const int k0 = order[pos];
             const double n0 = (double)meshes[w.first + k0]->N;
-            const int per = (int)std::min<int64_t>(want[k0], 8);
-            const int cap = std::max(1, Gmax / std::max(per, 1));
+            const int per = n0 < 2000.0 ? (int)std::min<int64_t>((want[k0] + 1) / 2, 4) : (int)std::min<int64_t>(want[k0], 8);
+            const int cap = want[k0] == 1 ? Gmax : std::max(1, Gmax2 / per);
+            int64_t ntiles = 0;
             while (pos < order.size() && (int)gr.idx.size() < cap) {
                 const int k = order[pos];
                 const double n = (double)meshes[w.first + k]->N;
                 if (!gr.idx.empty() && 2.0 * n * n < n0 * n0) break;
                 gr.idx.push_back(k);
+                ntiles += bt->prob[w.first + k].nt;
                 ++pos;
             }
             const int Pg = (int)gr.idx.size();
+            const bool three = Pg > Gmax2 || (!packed && ntiles >= (int64_t)kPcgDfTiles * Gmax);
+            const int Gg = three ? Gmax : Gmax2;
+            gr.kern = three ? kern3 : kern2;
             double wsum = 0.0;
             for (int k : gr.idx) wsum += (double)meshes[w.first + k]->N * (double)meshes[w.first + k]->N;
             int gsum = 0;
             for (int k : gr.idx) {
                 const double N = (double)meshes[w.first + k]->N;
-                const int64_t share = (int64_t)((double)(Gmax - Pg) * N * N / wsum) + 1;
+                const int64_t share = (int64_t)((double)(Gg - Pg) * N * N / wsum) + 1;
                 g[k] = (int)std::min<int64_t>(share, want[k]);
                 gsum += g[k];
             }
-            while (gsum > Gmax) {  // rounding: take from the largest
+            while (gsum > Gg) {  // rounding: take from the largest
                 int km = gr.idx[0];
                 for (int k : gr.idx)
                     if (g[k] > g[km]) km = k;
                 --g[km];
                 --gsum;
+            }
+            for (; gsum < Gg; ++gsum) {
+                int km = -1;
+                double most = 0.0;
+                for (int k : gr.idx) {
+                    const double N = (double)meshes[w.first + k]->N;
+                    if (g[k] < want[k] && N * N / g[k] > most) {
+                        most = N * N / g[k];
+                        km = k;
+                    }
+                }
+                if (km < 0) break;
+                ++g[km];
             }
             gr.count = Pg;
             gr.begin.assign(Pg + 1, 0);
