@@ -296,7 +296,10 @@ __device__ __forceinline__ float recip_pow2(float s) { return __int_as_float((25
 
 // BEM_PRODUCTS_FP16: replaced residual after every 10^2-fold drop of ||r|| (r.r by
 // 10^4); fallback to the exact products when a replacement finds r.r above
-// kH16Progress times the previous replacement's (||r|| fallen by less than 10x)
+// kH16Progress times the previous replacement's (||r|| fallen by less than 10x).  The exact
+// products then start afresh from z: the FP16 products' direction is not conjugate to what
+// follows, and CG that kept it could stagnate (tensor-graded cube of 10,800 triangles, FP32
+// operator, Jacobi, 1e-8: 20,000 iterations without an answer, 551 from z).
 constexpr double kH16Delta2 = 1e-4;
 constexpr double kH16Progress = 1e-2;
 // a segment this long without reaching its drop also ends in a replaced residual (and
@@ -1697,6 +1700,7 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
     bool done = rr <= thr;  // of a residual formed from x (products in DF64 only: the recursive one)
     while (!done && it < a.max_it) {
         const double irz = 1.0 / rz;  // not in the chain from r.z to beta
+        bool restart = false;
         if (use16) {
             const int gr_static = a.ngroups <= nwarps ? (int)warp_g : -1;
             if (a.group > 1)
@@ -1833,9 +1837,12 @@ __device__ __forceinline__ void pcg_body(const PcgArgs &a, const int G, const in
             rr_true = rr;
             done = rr <= thr;
             ++ndf;
-            if (use16 && rr_true > kH16Progress * rr_true_prev) use16 = false;  // the same in every CTA
+            if (use16 && rr_true > kH16Progress * rr_true_prev) {  // the same in every CTA
+                use16 = false;
+                restart = true;
+            }
         }
-        const double beta = tot[0] * irz;
+        const double beta = restart ? 0.0 : tot[0] * irz;
         if (a.lanczos && cta == 0 && threadIdx.x == 0 && it - 1 < a.lanczos_cap) {
             a.lanczos[2 * (it - 1)] = alpha;
             a.lanczos[2 * (it - 1) + 1] = beta;
