@@ -355,15 +355,22 @@ __global__ void k_mark(const unsigned long long *keys, int64_t N, const long lon
 // Up to kSortMergeMax keys: chunks sorted in shared memory by a CTA each, then every key to
 // its rank.  Two launches; the network of the 65,536 keys of N = 38,656 took
 // 31 and 134 us without the gaps between them, now 55 us.
-// Above, where the searches' n^2 / chunk steps grow, the network's launches.
+// Above, where the searches' n^2 / chunk steps grow, and where a memory budget leaves no room
+// for the second array, the network's launches.
 constexpr int64_t kSortMergeMax = 131072;
 
-size_t sort_u64_keys(int64_t n2) { return (size_t)(n2 <= kSortMergeMax ? 2 * n2 : n2); }
+size_t sort_u64_keys(int64_t n2) { return (size_t)(n2 > 1024 && n2 <= kSortMergeMax ? 2 * n2 : n2); }
 
-unsigned long long *sort_u64(bem_ctx *ctx, unsigned long long *keys, int64_t n, int64_t n2)
+size_t sort_u64_keys_within(const bem_ctx *ctx, int64_t n2, size_t more)
+{
+    const size_t nk = sort_u64_keys(n2), bytes = (sizeof(unsigned long long) * nk + more + 255) / 256 * 256;
+    return ctx->budget > 0 && ctx->in_use + (int64_t)bytes > ctx->budget ? (size_t)n2 : nk;
+}
+
+unsigned long long *sort_u64(bem_ctx *ctx, unsigned long long *keys, size_t n_keys, int64_t n, int64_t n2)
 {
     cudaStream_t s = ctx->stream;
-    if (n2 <= kSortMergeMax) {
+    if (n_keys == sort_u64_keys(n2) && n2 <= kSortMergeMax) {
         const int64_t ch = std::min<int64_t>(n2, n2 <= 16384 ? 1024 : 2048);
         const int threads = (int)std::max<int64_t>(ch / 2, 32), nc = (int)((n + ch - 1) / ch);
         k_bitonic_block<<<nc, threads, sizeof(unsigned long long) * (size_t)ch, s>>>(keys, ch); BEM_COUNT(ctx);
@@ -398,14 +405,14 @@ bem_status dorfler(bem_ctx *ctx, const double *d_eta2, int64_t N, double theta, 
     Allocs tmp;
     unsigned long long *keys = nullptr;
     const int64_t nb = (N + kDorflerBlock - 1) / kDorflerBlock;
-    bem_status st = dalloc(ctx, tmp, (void **)&keys,
-                           sizeof(unsigned long long) * sort_u64_keys(n2) + sizeof(double) * (N + 2 * nb + 1) + 64, false);
+    const size_t rest = sizeof(double) * (N + 2 * nb + 1) + 64, nk = sort_u64_keys_within(ctx, n2, rest);
+    bem_status st = dalloc(ctx, tmp, (void **)&keys, sizeof(unsigned long long) * nk + rest, false);
     if (st) return st;
-    double *prefix = reinterpret_cast<double *>(keys + sort_u64_keys(n2));
+    double *prefix = reinterpret_cast<double *>(keys + nk);
     double *bsum = prefix + N, *off = bsum + nb;
     long long *dK = reinterpret_cast<long long *>(off + nb + 1);
     k_keys<<<nblk(n2, 256), 256, 0, s>>>(d_eta2, N, n2, keys); BEM_COUNT(ctx);
-    keys = sort_u64(ctx, keys, N, n2);
+    keys = sort_u64(ctx, keys, nk, N, n2);
     k_dorfler_blocks<<<nblk(nb, 4), 128, 0, s>>>(keys, d_eta2, N, prefix, bsum); BEM_COUNT(ctx);
     k_dorfler_select<<<1, 256, 0, s>>>(keys, prefix, bsum, nb, off, N, theta, d_vanish, dK); BEM_COUNT(ctx);
     k_mark<<<nblk(N, 256), 256, 0, s>>>(keys, N, dK, d_marked); BEM_COUNT(ctx);

@@ -279,10 +279,12 @@ bem_status zz_estimate_dual(bem_mesh *m, const double *d_x, int h_mode, double *
 bem_status zz_estimate(bem_mesh *m, const double *d_phi, int h_mode, double *d_eta2,
                        double *h_totals, double *d_totals = nullptr);
 // Ascending sort of n different 64-bit keys below ~0, padded by ~0 to n2 (a power of two), on
-// the context's stream, in an array of sort_u64_keys(n2) keys; returns where the n sorted keys
-// are in it.
+// the context's stream, in an array of n_keys keys; returns where the n sorted keys are in it.
+// n_keys: sort_u64_keys(n2), or n2 (in place, by more launches).  sort_u64_keys_within: the
+// first where the context's budget holds it and `more` bytes, else the second.
 size_t sort_u64_keys(int64_t n2);
-unsigned long long *sort_u64(bem_ctx *ctx, unsigned long long *keys, int64_t n, int64_t n2);
+size_t sort_u64_keys_within(const bem_ctx *ctx, int64_t n2, size_t more);
+unsigned long long *sort_u64(bem_ctx *ctx, unsigned long long *keys, size_t n_keys, int64_t n, int64_t n2);
 // n_marked (nullable) synchronises the stream; d_vanish (nullable, device: the ZZ
 // totals) marks everything when the estimator vanishes up to rounding; d_count
 // (nullable, device) receives the count without synchronising.

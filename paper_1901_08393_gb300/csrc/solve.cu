@@ -1458,7 +1458,7 @@ struct PcgArgs {
     float2 *prow, *pcol, *pdf;
     double *x, *r, *z, *p, *q;
     const double *d, *b;
-    double *part;             // 3 x G per-CTA partials
+    double *part;             // 3 x G per-CTA partials (k_pcg_res: 4 x G)
     unsigned *bar;            // [0] grid-barrier arrival counter (zero at launch)
     unsigned long long *ctr;  // tile counter (never decreases)
     int *err;
@@ -2445,8 +2445,8 @@ static bem_status pcg(bem_operator *op, Work &W, const double *rhs, double tol, 
 // cooperative launch of the needed size is not possible (the caller then runs the
 // host-driven loop).
 // Cluster order and inverse blocks of the block-Jacobi preconditioner (scratch in tmp).
-// Cluster order of the block preconditioner (depends on the mesh only): scratch and
-// perm (nbj x kBJ, -1 padding) in a.
+// Cluster order of the block preconditioner (depends on the mesh only): perm (nbj x kBJ,
+// -1 padding) in a.
 static bem_status cluster_setup(bem_operator *op, Allocs &a, int32_t **perm_out, int *nbj_out)
 {
     bem_ctx *ctx = op->mesh->ctx;
@@ -2456,17 +2456,28 @@ static bem_status cluster_setup(bem_operator *op, Allocs &a, int32_t **perm_out,
     int64_t n2 = 2;
     while (n2 < N) n2 <<= 1;
     unsigned long long *keys = nullptr;
-    const size_t kb = sizeof(unsigned long long) * sort_u64_keys(n2), pb = sizeof(int32_t) * nbj * kBJ;
+    const size_t pb = sizeof(int32_t) * nbj * kBJ;
     const int nbox = (int)std::min<int64_t>((N + 255) / 256, 64);
-    bem_status st = dalloc(ctx, a, (void **)&keys, kb + pb + (6 + 6 * nbox) * sizeof(double) + 64, false);
+    // under a memory budget the keys are given back once they are read (the inverse blocks,
+    // allocated next, need more); else one allocation for all
+    Allocs tmp;
+    const size_t ob = pb + (6 + 6 * nbox) * sizeof(double) + 64;
+    const size_t nk = sort_u64_keys_within(ctx, n2, ob + 512);
+    bem_status st = dalloc(ctx, ctx->budget > 0 ? tmp : a, (void **)&keys,
+                           sizeof(unsigned long long) * nk + (ctx->budget > 0 ? 0 : ob), false);
     if (st) return st;
-    int32_t *perm = reinterpret_cast<int32_t *>(keys + sort_u64_keys(n2));
+    int32_t *perm = reinterpret_cast<int32_t *>(keys + nk);
+    if (ctx->budget > 0 && (st = dalloc(ctx, a, (void **)&perm, ob, false))) {
+        dfree_all(ctx, tmp);
+        return st;
+    }
     double *box = reinterpret_cast<double *>(reinterpret_cast<char *>(perm) + (pb + 7) / 8 * 8);
     k_cent_box<<<nbox, 256, 0, s>>>(op->mesh->cent, N, box + 6); BEM_COUNT(ctx);
     k_box_fold<<<1, 32, 0, s>>>(box + 6, nbox, box); BEM_COUNT(ctx);
     k_morton_keys<<<nblk(n2, 256), 256, 0, s>>>(op->mesh->cent, N, n2, box, keys); BEM_COUNT(ctx);
-    keys = sort_u64(ctx, keys, N, n2);
+    keys = sort_u64(ctx, keys, nk, N, n2);
     k_cluster_perm<<<nblk((int64_t)nbj * kBJ, 256), 256, 0, s>>>(keys, N, (int64_t)nbj * kBJ, perm); BEM_COUNT(ctx);
+    dfree_all(ctx, tmp);  // stream-ordered
     BEM_CK_LAUNCH(ctx);
     *perm_out = perm;
     *nbj_out = nbj;
@@ -2696,11 +2707,12 @@ static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, b
         }
     }
     double *part = nullptr;
-    if ((st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (4 * G + 8) + 64, true))) {
+    const int nparts = resident ? 4 : 3;  // values per CTA
+    if ((st = dalloc(ctx, tmp, (void **)&part, sizeof(double) * (nparts * G + 8) + 64, true))) {
         dfree_all(ctx, tmp);
         return st;
     }
-    double *out = part + 4 * G;  // [0..4]: r.r, b.b, iterations, DF64 residuals, inexact stop
+    double *out = part + nparts * G;  // [0..4]: r.r, b.b, iterations, DF64 residuals, inexact stop
     unsigned long long *ctr = reinterpret_cast<unsigned long long *>(out + 6);
     unsigned *bar = reinterpret_cast<unsigned *>(ctr + 1);
     int *err = reinterpret_cast<int *>(bar + 2);
