@@ -79,7 +79,7 @@ FAR_FLOPS_PER_ENTRY = 49 * 11 + 16
 # peak 152 SMs x 128 lanes x 2.07 GHz.
 DF_FAR_OPS_PER_ENTRY = 49 * 16 + 520
 FP32_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
-PCG_TRAFFIC_RATIO = 18.072 / 18.294  # ncu DRAM bytes / algorithmic bytes of the persistent solver
+PCG_TRAFFIC_RATIO = 16.979 / 16.911  # ncu DRAM bytes / algorithmic bytes of the persistent solver
 PRECISIONS = {"df64": 2, "f64": 0, "f32": 1}
 PREC = 2
 PC = 1
@@ -257,7 +257,7 @@ def roofline(prec, far_n, far_ms, far_units, mv_n, mv_ms, mv_units, peaks, peak_
         avg_s = mv_ms / max(mv_n, 1) / 1e3
         achieved = bytes_ / avg_s / 1e9
         # DRAM bytes (read + write) over algorithmic bytes of one ncu capture of k_pcg_df
-        # (adaptive polycube level N = 12,558: 18.07 GB measured, 18.29 GB algorithmic);
+        # (cube of N = 12,288: 16.98 GB measured, 16.91 GB algorithmic);
         # traffic scales with the bytes of the products, so the ratio carries to full size
         traffic = PCG_TRAFFIC_RATIO * bytes_ if prec == 2 else None
         roof = {"kernel": {0: "k_matvec<double>", 1: "k_matvec<float>",

@@ -85,12 +85,9 @@ static void gauss_legendre(int n, double *x, double *w)
     }
 }
 
-static bem_status far_df_attributes(bem_ctx *ctx);
-
 static bem_status assembly_constants(bem_ctx *ctx)
 {
     if (ctx->device < 64 && g_asm_ready[ctx->device]) return BEM_OK;
-    if (bem_status st = far_df_attributes(ctx)) return st;
     const double r15 = std::sqrt(15.0);
     const double wa = (155.0 - r15) / 1200.0, wb = (155.0 + r15) / 1200.0;
     const double w7[kQ] = {9.0 / 40.0, wa, wa, wa, wb, wb, wb};
@@ -227,9 +224,11 @@ __device__ __noinline__ double far_f64_close(const double *__restrict__ qi, cons
 // correction y t / 2 + 3/8 y t^2, t = 1 - S y^2: 3 FP64 operations (y^2, t, the sum of y t)
 // and the t^2 term, below 2^-34, in FP32, where rsqrt took about 8.  Conversions are integer
 // operations.  7 FP64 operations per point pair instead of 15; bound by the FP64 pipe (2
-// lanes per SM and cycle: 84% of it, 402 operations per entry).  Rotated polycubes, best tile:
-// N = 604 434 -> 238 us, N = 2,416 3.40 -> 2.43 ms, N = 9,664 51.2 -> 34.7 ms.  Error of an entry (CPU emulation against 80 bits): r.m.s. 0.9 -
-// 1.3e-16, 1.0 - 1.4e-16 before.  Close pairs are put aside per warp as in far_df_body.
+// lanes per SM and cycle: 91% of it, 402 operations per entry).  Rotated polycubes, best tile:
+// N = 604 434 -> 238 us, N = 2,416 3.40 -> 2.43 ms, N = 9,664 51.2 -> 34.7 ms.  Error of an
+// entry against extended precision on the same points, emulated on cubes, graded cubes and
+// polycubes: r.m.s. 8.1 - 8.3e-17, at most 4e-16; 8.9 - 9.2e-17 and 4e-16 for FP64 sums of
+// rsqrt.  Close pairs are put aside per warp as in far_df_body.
 template <int R, int C>
 __device__ __forceinline__ void far_f64_body(const double *__restrict__ q64, const double *__restrict__ cent,
                                              double *__restrict__ V, int64_t ld, int64_t r1, int64_t c1, int64_t i0,
@@ -574,7 +573,8 @@ __device__ __noinline__ float2 far_df_close(const float *__restrict__ qi, const 
 //
 // 16 FP32 operations per point pair and about 520 per entry, against 50 and 336 of the
 // form that took each of the 49 differences on a grid (three subtractions and squares
-// each).  Bound by FP32 issue (73% of the 128 lanes per SM and cycle).  Measured on rotated
+// each).  Bound by FP32 issue (72% of the 128 lanes per SM and cycle, 81% of the issue
+// slots).  Measured on rotated
 // polycubes, best tile of each: N = 604 116 -> 35 us, N = 2,416 418 -> 166 us, N = 9,664
 // 4.60 -> 2.03 ms, N = 21,744 22.3 -> 9.88 ms (10.6 -> 23.9 Gpairs/s).
 constexpr double kOrbS = (1.0 - kSqrt15) / (1.0 + kSqrt15);
@@ -765,6 +765,8 @@ __device__ __forceinline__ void far_df_expanded(const float4 *ri, const float4 *
 // (broadcast reads).
 template <int C>
 constexpr size_t far_df_smem() { return sizeof(float4) * 9 * C; }
+static_assert(far_df_smem<256>() + 64 * 9 * sizeof(float4) + 8 * 64 * sizeof(unsigned short) <= 48 * 1024,
+              "the largest tile (64 x 256) fits the default shared memory per CTA");
 
 // Close pairs (below 1.5 (R_i + R_j): 0.1-0.7% of the pairs from N = 5,000 on, most of them
 // on meshes of a few hundred triangles) cost three times the others: each warp puts its
@@ -1483,20 +1485,6 @@ static void far_batch_launch(const BatchAsm &b, cudaStream_t s)
 {
     const size_t smem = std::is_same<T, float2>::value ? far_df_smem<C>() : 0;
     k_far_batch<T, R, C, MB><<<(unsigned)b.n_far, C, smem, s>>>(b.prob, b.far_items);
-}
-
-// The DF64 tiles of 256 columns whose shared memory (row staging + the column
-// offsets on the pair grid) exceeds the default 48 KB per CTA.
-static bem_status far_df_attributes(bem_ctx *ctx)
-{
-    const int dyn = (int)far_df_smem<256>();
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_df<32, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_df<64, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 32, 256, 0>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    BEM_CK(ctx, cudaFuncSetAttribute(k_far_batch<float2, 64, 256, 0>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    return BEM_OK;
 }
 
 // Event record that also fires when a captured graph replays (an external event node

@@ -17,10 +17,10 @@ constexpr int kQ64Stride = 24;     // doubles per triangle in the FP64 point tab
 constexpr int kQ32Stride = 24;     // floats per triangle in the FP32 offset table
 constexpr int kQdfStride = 92;     // floats per triangle in the double-float table:
                                    // [0,42) offsets hi/lo, [42,51) centroid as 3 floats
-                                   // per coordinate, [51,53) area hi/lo, [53] the
-                                   // largest |hi| of the offsets, [54] the largest
-                                   // distance of a point from the centroid, [56,92)
-                                   // nine float4 of the expanded form (kQdfExp)
+                                   // per coordinate, [51,53) area hi/lo, [54] the
+                                   // largest distance of a point from the centroid,
+                                   // [53] and [55] unused, [56,92) nine float4 of the
+                                   // expanded form (kQdfExp)
 constexpr int kQdfExp = 56;        // offsets of the first orbit's points of vertices 0 and 1
                                    // (x, y, z as hi/lo: 12 floats), per vertex k |o_1k|^2 and
                                    // |o_2k|^2 as hi/lo (3 x 4), then the centroid's first,
@@ -100,7 +100,7 @@ struct bem_mesh {
                                 // largest distance of a point from the centroid
     float *q32 = nullptr;       // N x 24: 7 offsets from the centroid (x,y,z)
     double *cent = nullptr;     // N x 4: centroid (x,y,z), area
-    float *qdf = nullptr;       // N x 56: double-float table (see kQdfStride)
+    float *qdf = nullptr;       // N x kQdfStride: double-float table
     int32_t *v2t_off = nullptr; // M + 1
     int32_t *v2t = nullptr;     // 3N, ascending triangle index per vertex
     int32_t *owner = nullptr;   // 3N: half-edge -> first half-edge of its edge

@@ -292,21 +292,19 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
     // points 1, 2, 3 (4, 5, 6) are those of vertices 2, 1, 0
     constexpr double r15 = 3.87298334620741688518, ot = (1.0 + r15) / 7.0, os = (1.0 - r15) / (1.0 + r15);
     double o1[3][3];
-    float rm = 0.0f;
     for (int c = 0; c < 3; ++c) {
         split2((1.0 / 3.0) * ((R[0][c] + R[1][c]) + R[2][c]), f + 2 * c);
         for (int k = 0; k < 3; ++k) {
             o1[k][c] = ot * R[k][c];
             split2(o1[k][c], f + 2 * (3 * (3 - k) + c));
             split2(os * o1[k][c], f + 2 * (3 * (6 - k) + c));
-            rm = fmaxf(rm, fabsf(f[2 * (3 * (3 - k) + c)]));  // the first orbit's are the largest
         }
     }
     for (int c = 0; c < 3; ++c) split3(c3[c], f + 42 + 3 * c);
     split2(A, f + 51);
-    // the largest |hi part| of the offset coordinates and the largest distance of a point
-    // from the centroid (the first orbit's), rounded up; expanded form: orbit offsets of
-    // vertices 0 and 1 and the squared lengths (vertex 2's offset as minus the others' sum)
+    // the largest distance of a point from the centroid (the first orbit's), rounded up;
+    // expanded form: orbit offsets of vertices 0 and 1 and the squared lengths (vertex 2's
+    // offset as minus the others' sum)
     float *g = f + kQdfExp;
     double rd2 = 0.0;
     for (int k = 0; k < 3; ++k) {
@@ -323,7 +321,7 @@ __global__ void k_geometry(const double *verts, const int32_t *tris, int64_t N, 
             split2(os * os * n2, g + 14 + 4 * k);
         }
     }
-    f[53] = rm;
+    f[53] = 0.0f;
     f[54] = __double2float_ru(sqrt(rd2) * (1.0 + 1e-12));
     q[23] = (double)f[54];
     f[55] = 0.0f;

@@ -560,7 +560,9 @@ __device__ __forceinline__ double symv_row4_groups(const float2 *__restrict__ pr
 // sum's error is a few units of 2^-24 q, 2^-43 of the largest product.  The lanes' sums are
 // added by two-sums.  Bound by HBM: 163 us at N = 21,744 (946 MB, 5.8 TB/s of 6.76
 // measured) with 16 warps of 128 registers per SM, against 211 us with either kind of sums
-// and 24 warps of 80.
+// and 24 warps of 80.  The residuals that decide convergence are summed by two-sums; these
+// sums only steer the iteration.  Uniform surfaces take the same iterations within 2; the
+// tensor-graded cube of 60,492 triangles (FP32 operator, Jacobi, 1e-10) 4,193 -> 4,330, in 7.46 -> 6.31 s.
 __device__ __forceinline__ int warp_grab(unsigned long long *ctr, unsigned long long base)
 {
     int k = 0;
@@ -2033,8 +2035,8 @@ __global__ void __launch_bounds__(kMvThreads, kF64Ctas) k_pcg_f64(PcgF64Args a)
 // the latency of two barriers, of the loads that follow them and of chains of FP64 operations
 // (sums as trees, loads in flight together, reciprocals off the chains: 18 -> 13 us at N =
 // 2,352).  Per iteration, DF64, Jacobi / block: N = 604 20 / 22 -> 10 / 11 us, N = 1,200 21 /
-// 23 -> 12 / 13, N = 2,352 22 / 25 -> 13 / 14.  The line lies where the rows no longer fit: at N =
-// 2,700 the tiled solver takes 20 / 23 us.
+// 23 -> 12 / 13, N = 2,352 22 / 25 -> 13 / 14.  The line is one CTA of 16 rows per SM (N = 2,432
+// on 152); above it the tiled solver runs, 20 / 23 us at N = 2,700.
 constexpr int kResRows = 16;
 constexpr int kResThreads = 512;
 constexpr int kResWarps = kResThreads / 32;
@@ -2441,10 +2443,6 @@ static bem_status pcg(bem_operator *op, Work &W, const double *rhs, double tol, 
     return BEM_OK;
 }
 
-// The persistent DF64 solver (k_pcg_df).  Returns BEM_OK with *ran = false when a
-// cooperative launch of the needed size is not possible (the caller then runs the
-// host-driven loop).
-// Cluster order and inverse blocks of the block-Jacobi preconditioner (scratch in tmp).
 // Cluster order of the block preconditioner (depends on the mesh only): perm (nbj x kBJ,
 // -1 padding) in a.
 static bem_status cluster_setup(bem_operator *op, Allocs &a, int32_t **perm_out, int *nbj_out)
@@ -2500,6 +2498,7 @@ static bem_status block_inverse_launch(bem_operator *op, const int32_t *perm, in
     return BEM_OK;
 }
 
+// Cluster order and inverse blocks of the block-Jacobi preconditioner (scratch in tmp).
 // Cluster order and inverse blocks of the block-Jacobi preconditioner (scratch in tmp).
 static bem_status block_setup(bem_operator *op, Allocs &tmp, int32_t **perm_out, double **binv_out, int *nbj_out)
 {
@@ -2592,6 +2591,9 @@ static bem_status persistent_results(bem_ctx *ctx, const double *h, const Persis
     return BEM_OK;
 }
 
+// The persistent solvers of DF64 and FP32 operators (k_pcg_res, k_pcg_df, k_pcg_df_only,
+// k_pcg_cal).  Returns BEM_OK with *ran = false when a cooperative launch of the needed size
+// is not possible (the caller then runs the host-driven loop).
 static bem_status pcg_persistent(bem_operator *op, Work &W, const double *rhs, bool has_x0, double tol, int max_it,
                                  int precond, double delta, const int32_t *bperm, const double *binv, int nbj,
                                  double inexact_lambda, int h_mode, int *its_out, int *ndf_out, double *rel_out,
@@ -3642,7 +3644,7 @@ bem_status bem_batch_create(bem_ctx *ctx, int32_t count, bem_mesh *const *meshes
             a.nb = (int)(L / kSB);
             a.ntiles = (int)pr.nt;
             a.tiles = pr.tiles;
-            a.group = 1;  // a wave's problems are far below the sizes of groups
+            a.group = 1;  // single tiles, whatever the problem's share of the CTAs
             a.ngroups = a.ntiles;
             a.groups = pr.tiles;
             a.prow = prow;
