@@ -1947,13 +1947,19 @@ __global__ void __launch_bounds__(kMvThreads, kF64Ctas) k_pcg_f64(PcgF64Args a)
             const double2 *xv = reinterpret_cast<const double2 *>(v);
             const int64_t n2 = a.ld / 2;
             double a0 = 0.0, a1 = 0.0;
-#pragma unroll 12
-            for (int64_t k = lane; k < n2; k += 32) {
-                const double2 m = ld_once(r + k);
-                const double2 w = xv[k];  // written by other CTAs before the last barrier
-                a0 = fma(m.x, w.x, a0);
-                a1 = fma(m.y, w.y, a1);
-            }
+            auto steps = [&](auto unrolled) {
+#pragma unroll(decltype(unrolled)::value)
+                for (int64_t k = lane; k < n2; k += 32) {
+                    const double2 m = ld_once(r + k);
+                    const double2 w = xv[k];  // written by other CTAs before the last barrier
+                    a0 = fma(m.x, w.x, a0);
+                    a1 = fma(m.y, w.y, a1);
+                }
+            };
+            if (n2 < 12 * 32)  // shorter rows (N < 768) would run in the remainder's loop: 192 triangles +1% per call
+                steps(std::integral_constant<int, 4>());
+            else
+                steps(std::integral_constant<int, 12>());
             const double acc = warp_sum(a0 + a1);
             if (lane == 0) f(row, acc);
         }
