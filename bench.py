@@ -871,7 +871,7 @@ def main():
                     help="adaptive workload: stop each solve by the rule of the Remark after Alg. 1 (i), "
                          "|||x_k - x_(k-1)||| <= LAMBDA eta(x_k) (the paper uses ~1e-3); 0: PCG to 1e-10")
     ap.add_argument("--far-tile", type=int, default=0,
-                    help="adaptive and dual workloads: far-field tile variant 1..12 instead of the autotuned "
+                    help="adaptive and dual workloads: far-field tile variant 1..14 instead of the autotuned "
                          "one (no timing launches: for profiling captures)")
     ap.add_argument("--graded", default="adaptive", choices=["adaptive", "tensor"],
                     help="graded60k: adaptive -- the unit cube (192 triangles) graded by the DF64 adaptive loop "
